@@ -1140,6 +1140,7 @@ static dmpt_status batch_impl(dmpt_handle h, int count, const double* const* H,
       gd[j].partials = gi[j].partials;
       gd[j].ptiles = gi[j].ptiles;
       gd[j].entries = entries[i];
+      gd[j].jobs = 1 + L[i].k;
     }
     n_group = (int)order.size();
     // copies from pageable memory return once the source is staged

@@ -251,6 +251,7 @@ struct GroupDecide {
   const double* partials;
   int64_t ptiles;
   int64_t entries;
+  int jobs;            // 1 + response slots of the partials array
 };
 constexpr int kGroupMax = 1024;   // instances per grouped launch
 // Dynamic item queue of a grouped launch: the leader CTA of each pair claims

@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math.h>
+#include <stddef.h>
 
 #include <mutex>
 
@@ -395,369 +396,423 @@ __device__ int fp16_exponent_for(double bound) {
   return e < -100 ? -100 : (e > 100 ? 100 : e);
 }
 
-// Plan layer n (Alg. 1: branch choice; Alg. 2: D0 stopping tests).
-__device__ void plan_layer(State* st, int n) {
-  int sigma;
-  if (!st->d0_conv) {
-    const double NS = st->NS, NX = st->NX, no = st->n_occ;
-    const double iderr = NS - NX;
-    // sigma_n = sign(|2 N_S - N_X - N_occ| - |N_X - N_occ|); sign(0) -> -1
-    const double arg = fabs(2.0 * NS - NX - no) - fabs(NX - no);
-    sigma = arg > 0.0 ? 1 : -1;
-    st->iderr[n] = iderr;
-    st->ns_hist[n] = NS;
-    st->nx_hist[n] = NX;
-    st->sigma[n] = (signed char)sigma;
-    bool stop = iderr <= 0.0;
-    if (!stop && n > 2 && st->sigma[n - 1] != st->sigma[n - 2] &&
-        iderr > st->c_d0 * st->iderr[n - 2] * st->iderr[n - 2])
-      stop = true;
-    st->plan_square = 1;
-    if (stop) {
-      st->d0_conv = 1;
-      st->d0_layer = n;
-      st->plan_write0 = 0;  // this layer's square only measures FroErr^(0)
+// A decide step works on the control block's head (every field before the
+// per-layer histories) in shared memory.  What bounds it is latency, not work:
+// one thread walking the block in device memory took 9-35 us per layer (a
+// dependent access costs about 0.4 us, an FP64 square root or divide as much).
+// Here the head, the partial sums of every job and the few history entries the
+// tests read are fetched at the same time, 256 threads per job (four jobs at
+// once), and one warp then takes the decisions, lane j those of response slot
+// j.  Measured per step, n = 128 k = 1 / n = 2048 k = 3: 16.5 / 23.5 us
+// before, 5.8 / 7.0 us now (an empty launch takes 2 us).
+constexpr int kDecideThreads = 1024;
+constexpr int kHeadWords = (int)(offsetof(State, iderr) / sizeof(unsigned));
+static_assert(offsetof(State, iderr) % sizeof(unsigned) == 0 && kHeadWords <= kDecideThreads,
+              "one head word per thread");
+
+struct DecideShared {
+  alignas(16) unsigned head[kHeadWords + (kHeadWords & 1)];
+  double red[kDecideThreads / 256][kNQ][256];
+  double sums[kMaxK + 1][kNQ];   // per job, as summed from the partials
+  double fe2[kMaxK];             // FroErr^(1)_{n-2} of the layer that has run
+  double iderr1;                 // IdErr_{n-1}
+  int sig0, sig1, sig_next;      // sigma_n, sigma_{n-1}; sigma of the layer to plan
+};
+
+// Plan layer n (Alg. 1: branch choice; Alg. 2: D0 stopping tests).  One warp;
+// S: head in shared memory, G: control block, conv: slot `lane` has stopped.
+__device__ void plan_layer(State* S, State* G, const DecideShared& sh, int n, int lane,
+                           bool conv) {
+  if (lane == 0) {
+    int sigma;
+    if (!S->d0_conv) {
+      const double NS = S->NS, NX = S->NX, no = S->n_occ;
+      const double iderr = NS - NX;
+      // sigma_n = sign(|2 N_S - N_X - N_occ| - |N_X - N_occ|); sign(0) -> -1
+      const double arg = fabs(2.0 * NS - NX - no) - fabs(NX - no);
+      sigma = arg > 0.0 ? 1 : -1;
+      G->iderr[n] = iderr;
+      G->ns_hist[n] = NS;
+      G->nx_hist[n] = NX;
+      bool stop = iderr <= 0.0;
+      if (!stop && n > 2 && sh.sig0 != sh.sig1 && iderr > S->c_d0 * sh.iderr1 * sh.iderr1)
+        stop = true;
+      S->plan_square = 1;
+      if (stop) {
+        S->d0_conv = 1;
+        S->d0_layer = n;
+        S->plan_write0 = 0;  // this layer's square only measures FroErr^(0)
+      } else {
+        S->plan_write0 = 1;
+      }
     } else {
-      st->plan_write0 = 1;
+      sigma = -sh.sig0;  // the sigma flip of Alg. 1
+      S->plan_square = 0;
+      S->plan_write0 = 0;
     }
-  } else {
-    sigma = -(int)st->sigma[n - 1];  // the sigma flip of Alg. 1
-    st->sigma[n] = (signed char)sigma;
-    st->plan_square = 0;
-    st->plan_write0 = 0;
+    G->sigma[n] = (signed char)sigma;
+    S->sigma_cur = sigma;
+    S->n_layer = n;
   }
-  st->sigma_cur = sigma;
-  for (int j = 0; j < st->k; ++j) {
-    st->plan_resp[j] = !st->d1_conv[j];
+  __syncwarp();   // s1_fro2 of every slot
+  if (lane < S->k) {
+    S->plan_resp[lane] = !conv;
     // |S1_n|_max <= ||S1_n||_2 <= (2 ||S0||_2 + |1 - sigma|) ||S1_{n-1}||_2
     //            <= 4.5 ||S1_{n-1}||_F   (spectrum of S0 within [-0.25, 1.25]);
     // an order-o slot (o >= 2) adds sum_{a=1}^{o-1} ||S_a S_{o-a}||_2
     // <= sum ||S_a||_F ||S_{o-a}||_F (twice, for 2 S - S^2)
-    double bound = 4.5 * sqrt(st->s1_fro2[j]);
-    if (st->order >= 2 && j >= st->k1) {
-      const int o = 1 + j / st->k1, d = j % st->k1;
+    double bound = 4.5 * sqrt(S->s1_fro2[lane]);
+    if (S->order >= 2 && lane >= S->k1) {
+      const int o = 1 + lane / S->k1, d = lane % S->k1;
       double cross = 0.0;
       for (int a = 1; a < o; ++a)
-        cross += sqrt(st->s1_fro2[(a - 1) * st->k1 + d] * st->s1_fro2[(o - a - 1) * st->k1 + d]);
+        cross += sqrt(S->s1_fro2[(a - 1) * S->k1 + d] * S->s1_fro2[(o - a - 1) * S->k1 + d]);
       bound += 2.0 * cross;
     }
-    st->s1_exp_next[j] = st->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(bound) : 0;
+    S->s1_exp_next[lane] = S->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(bound) : 0;
   }
-  st->n_layer = n;
 }
 
 // Plan layer m of a response replay: S0 operand = stored state
 // min(m - 1, U), the forward's sigma_m (continued by flips past the forward's
 // last layer), responses of the directions still running.
-__device__ void plan_replay(State* st, int m) {
-  const int U = st->d0_updates;
-  st->z0_cur = st->tape_base + 2 * (m - 1 < U ? m - 1 : U);
-  if (m > st->rp_lmax) st->sigma[m] = (signed char)(-st->sigma[m - 1]);
-  st->sigma_cur = st->sigma[m];
-  st->plan_square = 0;
-  st->plan_write0 = 0;
-  for (int j = 0; j < st->k; ++j) {
-    st->plan_resp[j] = !st->d1_conv[j];
-    st->s1_exp_next[j] = st->precision == DMPT_DUAL_FP16
-                             ? fp16_exponent_for(4.5 * sqrt(st->s1_fro2[j]))
-                             : 0;
+__device__ void plan_replay(State* S, State* G, const DecideShared& sh, int m, int lane,
+                            bool conv) {
+  if (lane == 0) {
+    const int U = S->d0_updates;
+    S->z0_cur = S->tape_base + 2 * (m - 1 < U ? m - 1 : U);
+    int sigma = sh.sig_next;
+    if (m > S->rp_lmax) {
+      sigma = -sh.sig0;
+      G->sigma[m] = (signed char)sigma;
+    }
+    S->sigma_cur = sigma;
+    S->plan_square = 0;
+    S->plan_write0 = 0;
+    S->n_layer = m;
   }
-  st->n_layer = m;
+  if (lane < S->k) {
+    S->plan_resp[lane] = !conv;
+    S->s1_exp_next[lane] = S->precision == DMPT_DUAL_FP16
+                               ? fp16_exponent_for(4.5 * sqrt(S->s1_fro2[lane]))
+                               : 0;
+  }
 }
 
-// The decide step of one instance, run by one 256-thread block (red: kNQ x
-// 256 doubles, sums: (kMaxK + 1) x kNQ doubles of shared memory).
-__device__ void decide_body(State* st, const double* __restrict__ partials, int64_t ptiles,
-                            int64_t entries, int mode, double* red, double (*sums)[kNQ]) {
-  if (threadIdx.x == 0) {
-    st->round_ctr = 0u;    // for the next pair-kernel launch
-    st->ckpt_pending = 0;  // set again below when this step makes a checkpointed state
+// End of a run (lane 0).
+__device__ __forceinline__ void decide_end(State* S, int lane, int status) {
+  if (lane == 0) {
+    S->status = status;
+    S->done = 1;
   }
-  if (st->done) return;
-  const bool adj = mode == kDecideAdjInit || mode == kDecideAdjLayer || mode == kDecideAdjResume;
-  const bool rp = mode == kDecideReplayInit || mode == kDecideReplayLayer;
-  const int k = adj ? 1 : st->k;
-  for (int job = 0; job <= k; ++job) {
-    bool ran;
-    if (adj)
-      ran = job == 1 && mode != kDecideAdjResume;
-    else if (mode == kDecideInit)
-      ran = true;
-    else if (mode == kDecideReplayInit)
-      ran = job >= 1;
-    else
-      ran = job == 0 ? st->plan_square != 0 : st->plan_resp[job - 1] != 0;
-    (void)rp;
-    if (!ran) continue;  // uniform across the block
-    double v[kNQ] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t e = threadIdx.x; e < entries; e += 256) {
-      const double* p = partials + ((size_t)job * ptiles + e) * kNQ;
-#pragma unroll
-      for (int q = 0; q < kNQ; ++q) v[q] += p[q];
+}
+
+// Response replayed over the stored S0 states (one warp).
+__device__ void decide_replay(State* S, State* G, const DecideShared& sh, int mode, int lane) {
+  const bool init = mode == kDecideReplayInit;
+  const int k = S->k, n = S->n_layer;
+  const bool ran = lane < k && (init || S->plan_resp[lane]);
+  const bool bad = __any_sync(0xffffffffu, ran && sh.sums[1 + (ran ? lane : 0)][kQBad] > 0.0);
+  if (S->timeout_flag) return decide_end(S, lane, DMPT_ETIMEOUT);
+  if (bad) return decide_end(S, lane, DMPT_ENUMERIC);
+  bool conv = true;
+  if (init) {
+    if (lane < k) {
+      S->cur1[lane] = 0;
+      S->d1_conv[lane] = 0;
+      S->d1_layer[lane] = 0;
+      const double f = sh.sums[1 + lane][kQFroNew];
+      S->s1_fro2[lane] = f;
+      S->s1_exp_cur[lane] = S->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(sqrt(f)) : 0;
+      conv = false;
     }
-    block_sum<kNQ, 256>(v, red);
-    if (threadIdx.x == 0) {
+    if (lane == 0) {
+      S->rp_lmax = S->layers_run;
+      S->rp_layers = 0;
+    }
+    __syncwarp();
+    return plan_replay(S, G, sh, 1, lane, conv);
+  }
+  if (lane < k) conv = S->d1_conv[lane] != 0;
+  if (ran) {
+    const double fe = sqrt(sh.sums[1 + lane][kQFroDiff]);
+    G->froerr1[lane][n] = fe;
+    const bool fired = n - 2 >= S->d0_layer && fe >= S->c_pt * S->froerr0 * sh.fe2[lane];
+    if (fired) {
+      S->d1_conv[lane] = 1;
+      S->d1_layer[lane] = n;
+      conv = true;
+    } else {
+      S->cur1[lane] ^= 1;
+      S->s1_fro2[lane] = sh.sums[1 + lane][kQFroNew];
+      S->s1_exp_cur[lane] = S->s1_exp_next[lane];
+    }
+  }
+  if (lane == 0) S->rp_layers = n;
+  const bool all1 = __all_sync(0xffffffffu, conv);
+  if (all1) return decide_end(S, lane, DMPT_OK);
+  if (n + 1 > S->max_layers) return decide_end(S, lane, DMPT_ENOTCONV);
+  plan_replay(S, G, sh, n + 1, lane, conv);
+}
+
+// Adjoint of the S0 recursion, run backwards over the stored states (lane 0).
+__device__ void decide_adjoint(State* S, const DecideShared& sh, int mode) {
+  if (S->timeout_flag) return decide_end(S, 0, DMPT_ETIMEOUT);
+  if (mode != kDecideAdjResume && sh.sums[1][kQBad] > 0.0) return decide_end(S, 0, DMPT_ENUMERIC);
+  int m;
+  if (mode == kDecideAdjInit) {
+    S->k = 1;
+    S->cur1[0] = 0;
+    S->plan_square = 0;
+    S->plan_write0 = 0;
+    for (int j = 0; j < kMaxK; ++j) S->plan_resp[j] = 0;
+    S->s1_fro2[0] = sh.sums[1][kQFroNew];
+    S->s1_exp_cur[0] =
+        S->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(sqrt(S->s1_fro2[0])) : 0;
+    m = S->d0_updates;
+  } else if (mode == kDecideAdjLayer) {
+    S->cur1[0] ^= 1;
+    S->s1_fro2[0] = sh.sums[1][kQFroNew];
+    S->s1_exp_cur[0] = S->s1_exp_next[0];
+    m = S->adj_m - 1;
+  } else {
+    m = S->adj_m;   // resume after the host reloaded the tape with an earlier segment
+  }
+  S->adj_m = m;
+  if (m <= 0) {
+    S->plan_resp[0] = 0;
+    return decide_end(S, 0, DMPT_OK);
+  }
+  if (m <= S->adj_seg_a) {
+    // S_{m-1} lies before the states in the tape (checkpointed run): the
+    // host recomputes the previous segment and resumes with layer m
+    S->plan_resp[0] = 0;
+    return;
+  }
+  // adjoint of layer m: Gbar <- sigma_m (S_{m-1} Gbar + Gbar S_{m-1}) + (1 - sigma_m) Gbar
+  // (the tape holds states adj_seg_a, adj_seg_a + 1, ...; 0 without checkpoints)
+  S->z0_cur = S->tape_base + 2 * (m - 1 - S->adj_seg_a);
+  S->sigma_cur = sh.sig_next;   // sigma_m
+  S->plan_resp[0] = 1;
+  S->s1_exp_next[0] = S->precision == DMPT_DUAL_FP16
+                          ? fp16_exponent_for(4.5 * sqrt(S->s1_fro2[0]))
+                          : 0;
+}
+
+// The initial layer has run: start of a forward run (one warp).
+__device__ void decide_init(State* S, State* G, const DecideShared& sh, int lane) {
+  if (!(S->epsN > S->eps1) || !isfinite(S->epsN) || !isfinite(S->eps1) ||
+      sh.sums[0][kQBad] > 0.0)
+    return decide_end(S, lane, DMPT_ENUMERIC);
+  if (lane == 0) {
+    S->NS = sh.sums[0][kQTrace];
+    S->NX = sh.sums[0][kQFroNew];
+    S->s0_exp = S->precision == DMPT_DUAL_FP16 ? kFp16TargetExp - 1 : 0;
+    S->cur0 = 0;
+    S->d0_updates = 0;
+    S->ckpt_pending = S->ckpt_k >= 2 ? 1 : 0;   // S_0 is checkpoint 0
+    S->z0_cur = S->tape ? S->tape_base : zslice(0, 0, 0, S->layout_k);
+    S->z0_next = S->tape ? S->tape_base + 2 : zslice(1, 0, 0, S->layout_k);
+    S->d0_conv = 0;
+    S->d0_layer = 0;
+    S->layers_run = 0;
+    S->froerr0 = 0.0;
+  }
+  if (lane < S->k) {
+    S->cur1[lane] = 0;
+    S->d1_conv[lane] = 0;
+    S->d1_layer[lane] = 0;
+    const double f = sh.sums[1 + lane][kQFroNew];
+    S->s1_fro2[lane] = f;
+    S->s1_exp_cur[lane] = S->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(sqrt(f)) : 0;
+  }
+  __syncwarp();
+  plan_layer(S, G, sh, 1, lane, false);
+}
+
+// A layer product has finished: apply its results (one warp).
+__device__ void decide_layer(State* S, State* G, const DecideShared& sh, int lane) {
+  const int k = S->k, n = S->n_layer;
+  const bool square = S->plan_square != 0, wrote = S->plan_write0 != 0;
+  const bool d0 = S->d0_conv != 0;
+  const bool ran = lane < k && S->plan_resp[lane];
+  bool bad = __any_sync(0xffffffffu, ran && sh.sums[1 + (ran ? lane : 0)][kQBad] > 0.0);
+  bad = bad || (square && sh.sums[0][kQBad] > 0.0);
+  if (S->timeout_flag) return decide_end(S, lane, DMPT_ETIMEOUT);
+  if (bad) return decide_end(S, lane, DMPT_ENUMERIC);
+  bool conv = lane < k ? S->d1_conv[lane] != 0 : true;
+  if (square && lane == 0) {
+    if (wrote) {
+      S->NS = sh.sums[0][kQTrace];    // Tr S_n      (N_S of Alg. 2)
+      S->NX = sh.sums[0][kQFroNew];   // ||S_n||_F^2 = Tr S_n^2 (N_X of the next layer)
+      S->cur0 ^= 1;
+      S->d0_updates += 1;
+      if (S->ckpt_k >= 2 && S->d0_updates % S->ckpt_k == 0) S->ckpt_pending = 1;
+      if (S->tape) {
+        S->z0_cur = S->z0_next;
+        S->z0_next += 2;
+      } else {
+        S->z0_cur = zslice(S->cur0, 0, 0, S->layout_k);
+        S->z0_next = zslice(S->cur0 ^ 1, 0, 0, S->layout_k);
+      }
+    } else {
+      S->froerr0 = sqrt(sh.sums[0][kQFroDiff]);  // FroErr^(0) of Alg. 2
+    }
+  }
+  __syncwarp();
+  if (ran) {
+    const double fe = sqrt(sh.sums[1 + lane][kQFroDiff]);  // FroErr^(1)_n of Alg. 3
+    G->froerr1[lane][n] = fe;
+    bool fired = false;
+    if (d0 && n - 2 >= S->d0_layer) fired = fe >= S->c_pt * S->froerr0 * sh.fe2[lane];
+    if (fired) {
+      S->d1_conv[lane] = 1;  // keep S1_{n-1}: the buffer written by this layer is dropped
+      S->d1_layer[lane] = n;
+      conv = true;
+    } else {
+      S->cur1[lane] ^= 1;
+      S->s1_fro2[lane] = sh.sums[1 + lane][kQFroNew];
+      S->s1_exp_cur[lane] = S->s1_exp_next[lane];
+    }
+  }
+  if (lane == 0) S->layers_run = n;
+  const bool all1 = __all_sync(0xffffffffu, conv);
+  const bool end = d0 && all1, cap = n + 1 > S->max_layers;
+  if (end || cap) {
+    if (lane == 0) S->n_layer = n + 1;
+    return decide_end(S, lane, end ? DMPT_OK : DMPT_ENOTCONV);
+  }
+  plan_layer(S, G, sh, n + 1, lane, conv);
+}
+
+// The decide step of one instance, run by one block of kDecideThreads
+// threads.  jobs: 1 + the response slots of the partials array.
+__device__ void decide_body(State* st, const double* __restrict__ partials, int64_t ptiles,
+                            int64_t entries, int jobs, int mode, DecideShared& sh) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid < kHeadWords) sh.head[tid] = reinterpret_cast<const unsigned*>(st)[tid];
+  if (tid >= kDecideThreads - 32) {
+    // the history entries the tests read, fetched while the sums are formed
+    const bool adj = mode == kDecideAdjInit || mode == kDecideAdjLayer || mode == kDecideAdjResume;
+    const bool fresh = mode == kDecideInit || mode == kDecideReplayInit;
+    const int n = fresh ? 0 : st->n_layer;   // the layer that has run
+    if (lane < kMaxK && !adj && n >= 2) sh.fe2[lane] = st->froerr1[lane][n - 2];
+    if (lane == 8 && !adj && n >= 1) sh.iderr1 = st->iderr[n - 1];
+    if (lane == 9 && !adj) sh.sig0 = st->sigma[n];
+    if (lane == 10 && !adj && n >= 1) sh.sig1 = st->sigma[n - 1];
+    if (lane == 11) {
+      int m = n + 1;
+      if (adj)
+        m = mode == kDecideAdjInit ? st->d0_updates
+                                   : (mode == kDecideAdjLayer ? st->adj_m - 1 : st->adj_m);
+      sh.sig_next = m >= 0 && m <= kMaxL ? st->sigma[m] : 0;
+    }
+  }
+  // per job: 256 strided sums, then the fixed binary tree over them (pairs
+  // 128, 64, ... 1 apart), one warp per quantity
+  const int grp = tid >> 8, t = tid & 255;
+  for (int j0 = 0; j0 < jobs; j0 += kDecideThreads / 256) {
+    const int job = j0 + grp;
+    double v[kNQ] = {0.0, 0.0, 0.0, 0.0};
+    if (job < jobs) {
+      for (int64_t e = t; e < entries; e += 256) {
+        const double2* p =
+            reinterpret_cast<const double2*>(partials + ((size_t)job * ptiles + e) * kNQ);
+        const double2 a = p[0], b = p[1];
+        v[0] += a.x;
+        v[1] += a.y;
+        v[2] += b.x;
+        v[3] += b.y;
+      }
+    }
+    if (j0 > 0) __syncthreads();
 #pragma unroll
-      for (int q = 0; q < kNQ; ++q) sums[job][q] = v[q];
+    for (int q = 0; q < kNQ; ++q) sh.red[grp][q][t] = v[q];
+    __syncthreads();
+    if (job < jobs && t < 32 * kNQ) {
+      const double* r = sh.red[grp][t >> 5];
+      const double a0 = r[lane] + r[lane + 128], a2 = r[lane + 64] + r[lane + 192];
+      const double a1 = r[lane + 32] + r[lane + 160], a3 = r[lane + 96] + r[lane + 224];
+      double x = (a0 + a2) + (a1 + a3);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane == 0) sh.sums[job][t >> 5] = x;
     }
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-
-  if (mode == kDecideReplayInit || mode == kDecideReplayLayer) {
-    // ---- response recursion replayed over the stored S0 states
-    if (st->timeout_flag) {
-      st->status = DMPT_ETIMEOUT;
-      st->done = 1;
-      return;
+  State* S = reinterpret_cast<State*>(sh.head);   // only the fields before the histories
+  if (tid < 32) {
+    if (lane == 0) {
+      S->round_ctr = 0u;    // for the next pair-kernel launch
+      S->ckpt_pending = 0;  // set again below when this step makes a checkpointed state
     }
-    double bad = 0.0;
-    for (int j = 0; j < k; ++j)
-      if (mode == kDecideReplayInit || st->plan_resp[j]) bad += sums[1 + j][kQBad];
-    if (bad > 0.0) {
-      st->status = DMPT_ENUMERIC;
-      st->done = 1;
-      return;
-    }
-    if (mode == kDecideReplayInit) {
-      for (int j = 0; j < k; ++j) {
-        st->cur1[j] = 0;
-        st->d1_conv[j] = 0;
-        st->d1_layer[j] = 0;
-        st->s1_fro2[j] = sums[1 + j][kQFroNew];
-        st->s1_exp_cur[j] = st->precision == DMPT_DUAL_FP16
-                                ? fp16_exponent_for(sqrt(st->s1_fro2[j]))
-                                : 0;
-      }
-      st->rp_lmax = st->layers_run;
-      st->rp_layers = 0;
-      plan_replay(st, 1);
-      return;
-    }
-    const int n = st->n_layer;
-    for (int j = 0; j < k; ++j) {
-      if (!st->plan_resp[j]) continue;
-      const double fe = sqrt(sums[1 + j][kQFroDiff]);
-      st->froerr1[j][n] = fe;
-      const bool fired = n - 2 >= st->d0_layer &&
-                         fe >= st->c_pt * st->froerr0 * st->froerr1[j][n - 2];
-      if (fired) {
-        st->d1_conv[j] = 1;
-        st->d1_layer[j] = n;
-      } else {
-        st->cur1[j] ^= 1;
-        st->s1_fro2[j] = sums[1 + j][kQFroNew];
-        st->s1_exp_cur[j] = st->s1_exp_next[j];
+    __syncwarp();
+    if (!S->done) {
+      switch (mode) {
+        case kDecideInit: decide_init(S, st, sh, lane); break;
+        case kDecideLayer: decide_layer(S, st, sh, lane); break;
+        case kDecideReplayInit:
+        case kDecideReplayLayer: decide_replay(S, st, sh, mode, lane); break;
+        default:
+          if (lane == 0) decide_adjoint(S, sh, mode);
       }
     }
-    st->rp_layers = n;
-    bool all1 = true;
-    for (int j = 0; j < k; ++j) all1 = all1 && st->d1_conv[j];
-    if (all1) {
-      st->status = DMPT_OK;
-      st->done = 1;
-      return;
-    }
-    if (n + 1 > st->max_layers) {
-      st->status = DMPT_ENOTCONV;
-      st->done = 1;
-      return;
-    }
-    plan_replay(st, n + 1);
-    return;
   }
-
-  if (adj) {
-    // ---- adjoint of the S0 recursion, run backwards over the stored states
-    if (st->timeout_flag) {
-      st->status = DMPT_ETIMEOUT;
-      st->done = 1;
-      return;
-    }
-    if (mode != kDecideAdjResume && sums[1][kQBad] > 0.0) {
-      st->status = DMPT_ENUMERIC;
-      st->done = 1;
-      return;
-    }
-    int m;
-    if (mode == kDecideAdjInit) {
-      st->k = 1;
-      st->cur1[0] = 0;
-      st->plan_square = 0;
-      st->plan_write0 = 0;
-      for (int j = 0; j < kMaxK; ++j) st->plan_resp[j] = 0;
-      st->s1_fro2[0] = sums[1][kQFroNew];
-      st->s1_exp_cur[0] = st->precision == DMPT_DUAL_FP16
-                              ? fp16_exponent_for(sqrt(st->s1_fro2[0]))
-                              : 0;
-      m = st->d0_updates;
-    } else if (mode == kDecideAdjLayer) {
-      st->cur1[0] ^= 1;
-      st->s1_fro2[0] = sums[1][kQFroNew];
-      st->s1_exp_cur[0] = st->s1_exp_next[0];
-      m = st->adj_m - 1;
-    } else {
-      m = st->adj_m;   // resume after the host reloaded the tape with an earlier segment
-    }
-    st->adj_m = m;
-    if (m <= 0) {
-      st->plan_resp[0] = 0;
-      st->status = DMPT_OK;
-      st->done = 1;
-      return;
-    }
-    if (m <= st->adj_seg_a) {
-      // S_{m-1} lies before the states in the tape (checkpointed run): the
-      // host recomputes the previous segment and resumes with layer m
-      st->plan_resp[0] = 0;
-      return;
-    }
-    // adjoint of layer m: Gbar <- sigma_m (S_{m-1} Gbar + Gbar S_{m-1}) + (1 - sigma_m) Gbar
-    // (the tape holds states adj_seg_a, adj_seg_a + 1, ...; 0 without checkpoints)
-    st->z0_cur = st->tape_base + 2 * (m - 1 - st->adj_seg_a);
-    st->sigma_cur = st->sigma[m];
-    st->plan_resp[0] = 1;
-    st->s1_exp_next[0] = st->precision == DMPT_DUAL_FP16
-                             ? fp16_exponent_for(4.5 * sqrt(st->s1_fro2[0]))
-                             : 0;
-    return;
-  }
-
-  if (mode == kDecideInit) {
-    if (!(st->epsN > st->eps1) || !isfinite(st->epsN) || !isfinite(st->eps1) ||
-        sums[0][kQBad] > 0.0) {
-      st->status = DMPT_ENUMERIC;
-      st->done = 1;
-      return;
-    }
-    st->NS = sums[0][kQTrace];
-    st->NX = sums[0][kQFroNew];
-    st->s0_exp = st->precision == DMPT_DUAL_FP16 ? kFp16TargetExp - 1 : 0;
-    st->cur0 = 0;
-    st->d0_updates = 0;
-    st->ckpt_pending = st->ckpt_k >= 2 ? 1 : 0;   // S_0 is checkpoint 0
-    st->z0_cur = st->tape ? st->tape_base : zslice(0, 0, 0, st->layout_k);
-    st->z0_next = st->tape ? st->tape_base + 2 : zslice(1, 0, 0, st->layout_k);
-    st->d0_conv = 0;
-    st->d0_layer = 0;
-    st->layers_run = 0;
-    st->froerr0 = 0.0;
-    for (int j = 0; j < k; ++j) {
-      st->cur1[j] = 0;
-      st->d1_conv[j] = 0;
-      st->d1_layer[j] = 0;
-      st->s1_fro2[j] = sums[1 + j][kQFroNew];
-      st->s1_exp_cur[j] = st->precision == DMPT_DUAL_FP16
-                              ? fp16_exponent_for(sqrt(st->s1_fro2[j]))
-                              : 0;
-    }
-    plan_layer(st, 1);
-    return;
-  }
-
-  // ---- a layer product has finished: apply its results
-  const int n = st->n_layer;
-  if (st->timeout_flag) {
-    st->status = DMPT_ETIMEOUT;
-    st->done = 1;
-    return;
-  }
-  double bad = 0.0;
-  if (st->plan_square) bad += sums[0][kQBad];
-  for (int j = 0; j < k; ++j)
-    if (st->plan_resp[j]) bad += sums[1 + j][kQBad];
-  if (bad > 0.0) {
-    st->status = DMPT_ENUMERIC;
-    st->done = 1;
-    return;
-  }
-  if (st->plan_square) {
-    if (st->plan_write0) {
-      st->NS = sums[0][kQTrace];    // Tr S_n      (N_S of Alg. 2)
-      st->NX = sums[0][kQFroNew];   // ||S_n||_F^2 = Tr S_n^2 (N_X of the next layer)
-      st->cur0 ^= 1;
-      st->d0_updates += 1;
-      if (st->ckpt_k >= 2 && st->d0_updates % st->ckpt_k == 0) st->ckpt_pending = 1;
-      if (st->tape) {
-        st->z0_cur = st->z0_next;
-        st->z0_next += 2;
-      } else {
-        st->z0_cur = zslice(st->cur0, 0, 0, st->layout_k);
-        st->z0_next = zslice(st->cur0 ^ 1, 0, 0, st->layout_k);
-      }
-    } else {
-      st->froerr0 = sqrt(sums[0][kQFroDiff]);  // FroErr^(0) of Alg. 2
-    }
-  }
-  for (int j = 0; j < k; ++j) {
-    if (!st->plan_resp[j]) continue;
-    const double fe = sqrt(sums[1 + j][kQFroDiff]);  // FroErr^(1)_n of Alg. 3
-    st->froerr1[j][n] = fe;
-    bool fired = false;
-    if (st->d0_conv && n - 2 >= st->d0_layer)
-      fired = fe >= st->c_pt * st->froerr0 * st->froerr1[j][n - 2];
-    if (fired) {
-      st->d1_conv[j] = 1;  // keep S1_{n-1}: the buffer written by this layer is dropped
-      st->d1_layer[j] = n;
-    } else {
-      st->cur1[j] ^= 1;
-      st->s1_fro2[j] = sums[1 + j][kQFroNew];
-      st->s1_exp_cur[j] = st->s1_exp_next[j];
-    }
-  }
-  st->layers_run = n;
-  bool all1 = true;
-  for (int j = 0; j < k; ++j) all1 = all1 && st->d1_conv[j];
-  if (st->d0_conv && all1) {
-    st->status = DMPT_OK;
-    st->done = 1;
-    st->n_layer = n + 1;
-    return;
-  }
-  if (n + 1 > st->max_layers) {
-    st->status = DMPT_ENOTCONV;
-    st->done = 1;
-    st->n_layer = n + 1;
-    return;
-  }
-  plan_layer(st, n + 1);
+  __syncthreads();
+  if (tid < kHeadWords) reinterpret_cast<unsigned*>(st)[tid] = sh.head[tid];
 }
 
-__global__ void __launch_bounds__(256) decide_kernel(State* st, const double* __restrict__ partials,
-                                                     int64_t ptiles, int64_t entries, int mode) {
-  __shared__ double red[kNQ * 256];
-  __shared__ double sums[kMaxK + 1][kNQ];
-  decide_body(st, partials, ptiles, entries, mode, red, sums);
+__global__ void __launch_bounds__(kDecideThreads)
+    decide_kernel(State* st, const double* __restrict__ partials, int64_t ptiles, int64_t entries,
+                  int jobs, int mode) {
+  __shared__ DecideShared sh;
+  decide_body(st, partials, ptiles, entries, jobs, mode, sh);
 }
 
 // Layer decide of every instance of a grouped launch, one block each.
-__global__ void __launch_bounds__(256) decide_group_kernel(const GroupDecide* __restrict__ args,
-                                                           const int* __restrict__ group_timeout,
-                                                           GroupQueue* queue) {
-  __shared__ double red[kNQ * 256];
-  __shared__ double sums[kMaxK + 1][kNQ];
+__global__ void __launch_bounds__(kDecideThreads)
+    decide_group_kernel(const GroupDecide* __restrict__ args, const int* __restrict__ group_timeout,
+                        GroupQueue* queue) {
+  __shared__ DecideShared sh;
   if (blockIdx.x == 0 && threadIdx.x == 0) {   // the next grouped launch starts a new queue
     queue->counter = 0u;
     queue->epoch += 1u;
   }
   const GroupDecide a = args[blockIdx.x];
-  if (threadIdx.x == 0 && *group_timeout && !a.st->done) a.st->timeout_flag = 1;
-  __syncthreads();
-  decide_body(a.st, a.partials, a.ptiles, a.entries, kDecideLayer, red, sums);
+  if (*group_timeout) {   // uniform across the grid
+    if (threadIdx.x == 0 && !a.st->done) a.st->timeout_flag = 1;
+    __syncthreads();
+  }
+  decide_body(a.st, a.partials, a.ptiles, a.entries, a.jobs, kDecideLayer, sh);
 }
 
 cudaError_t launch_decide_group(const GroupDecide* args, int count, const int* group_timeout,
                                 GroupQueue* queue, cudaStream_t s) {
   if (count < 1) return cudaSuccess;
-  decide_group_kernel<<<count, 256, 0, s>>>(args, group_timeout, queue);
+  decide_group_kernel<<<count, kDecideThreads, 0, s>>>(args, group_timeout, queue);
   return cudaGetLastError();
+}
+
+// Per-device one-time setup; thread-safe.  The decide kernel runs between
+// layer kernels that use nearly all of an SM's shared memory: with the same
+// split of L1 and shared memory the SM need not be reconfigured.
+static void decide_setup() {
+  constexpr int kDevices = 64;
+  static std::once_flag once[kDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return;
+  std::call_once(once[dev], [] {
+    cudaFuncSetAttribute(decide_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                         cudaSharedmemCarveoutMaxShared);
+  });
 }
 
 cudaError_t launch_decide(const Layout& L, void* ws, int mode, int64_t entries, cudaStream_t s) {
   char* base = (char*)ws;
-  decide_kernel<<<1, 256, 0, s>>>((State*)(base + L.off_state),
-                                  (const double*)(base + L.off_partials), L.partial_tiles,
-                                  entries, mode);
+  decide_setup();
+  decide_kernel<<<1, kDecideThreads, 0, s>>>((State*)(base + L.off_state),
+                                             (const double*)(base + L.off_partials),
+                                             L.partial_tiles, entries, 1 + L.k, mode);
   return cudaGetLastError();
 }
 
@@ -1609,11 +1664,11 @@ __global__ void __launch_bounds__(256) batch_init_kernel(const BatchInst* __rest
                b.partials, b.ptiles, u - first[i], kInitBlocks);
 }
 
-__global__ void __launch_bounds__(256) batch_decide_init_kernel(const BatchInst* __restrict__ bi) {
-  __shared__ double red[kNQ * 256];
-  __shared__ double sums[kMaxK + 1][kNQ];
+__global__ void __launch_bounds__(kDecideThreads)
+    batch_decide_init_kernel(const BatchInst* __restrict__ bi) {
+  __shared__ DecideShared sh;
   const BatchInst& b = bi[blockIdx.x];
-  decide_body(b.st, b.partials, b.ptiles, kInitBlocks, kDecideInit, red, sums);
+  decide_body(b.st, b.partials, b.ptiles, kInitBlocks, 1 + b.k, kDecideInit, sh);
 }
 
 // 16-bit split of matrices 0 .. layout k (as split_kernel), kBatchChunk
@@ -1690,7 +1745,7 @@ cudaError_t launch_batch_setup(const BatchInst* bi, const int64_t* first, int co
     batch_init_kernel<double><<<(unsigned)units[kBsInit], 256, 0, s>>>(bi, f_init, count);
   else
     batch_init_kernel<float><<<(unsigned)units[kBsInit], 256, 0, s>>>(bi, f_init, count);
-  batch_decide_init_kernel<<<count, 256, 0, s>>>(bi);
+  batch_decide_init_kernel<<<count, kDecideThreads, 0, s>>>(bi);
   if (dual && units[kBsSplit] > 0) {
     if (bf16)
       batch_split_kernel<__nv_bfloat16><<<(unsigned)units[kBsSplit], 256, 0, s>>>(bi, f_split,
