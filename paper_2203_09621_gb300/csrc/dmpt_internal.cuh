@@ -166,6 +166,13 @@ inline int64_t upper_tiles(int64_t Np, int bt) {
   return t * (t + 1) / 2;
 }
 
+// Tile edge of the FP64 form (see layer_fp64_kernel) and its upper tiles.
+inline int fp64_tile(int64_t n) { return n <= 400 ? 8 : (n <= 2048 ? 16 : 32); }
+inline int64_t fp64_tiles(int64_t n) {
+  const int64_t t = (n + fp64_tile(n) - 1) / fp64_tile(n);
+  return t * (t + 1) / 2;
+}
+
 // ---- launchers (kernels_simt.cu) ----
 cudaError_t launch_bounds(const double* H, int64_t n, int64_t ld, double* eps_out,
                           cudaStream_t s);
@@ -216,7 +223,6 @@ cudaError_t launch_finalize(const Layout& L, void* ws, double* P, double* P1,
 cudaError_t launch_mirror_upper(double* M, int64_t n, int64_t ld, int count, cudaStream_t s);
 cudaError_t launch_trivial(int64_t n, int k, int64_t ld, int full, double* P,
                            double* P1, cudaStream_t s);
-int simt_tile(int precision);
 
 // ---- tensor-core path (kernels_tc.cu) ----
 // round_align: the pair kernel's producers keep their rounds in step (a

@@ -29,10 +29,10 @@ Layout make_layout(int64_t n, int k, int precision, int tape_states, int ckpt_sl
   size_t off = 0;
   L.off_state = off;
   off = align256(off + sizeof(State));
-  // one partial entry per upper tile of the smallest product tile (64) or
-  // per block of the init kernel, whichever is larger
-  int64_t tiles = upper_tiles(L.Np, 64);
-  L.partial_tiles = tiles > 1024 ? tiles : 1024;
+  // one partial entry per upper tile of the smallest product tile (64; the
+  // FP64 form's own) or per block of the init kernel, whichever is larger
+  const int64_t tiles = precision == DMPT_FP64 ? fp64_tiles(n) : upper_tiles(L.Np, 64);
+  L.partial_tiles = tiles > kInitBlocks ? tiles : kInitBlocks;
   L.off_partials = off;
   off = align256(off + (size_t)(1 + k) * (size_t)L.partial_tiles * kNQ * sizeof(double));
   const size_t mat = (size_t)L.Np * (size_t)L.Np;
@@ -1088,7 +1088,236 @@ __global__ void __launch_bounds__(256, SimtBlocks<T>::value)
   }
 }
 
-int simt_tile(int precision) { return precision == DMPT_FP64 ? 64 : 128; }
+// ---------------------------------------------------------------------------
+// FP64 layer product with fused epilogue.
+//
+// The part runs two FP64 FMAs per clock and SM, so a warp's FMA holds the
+// SM's pipe for 16 clocks and everything else (shared-memory reads, copies,
+// indexing) hides behind it: what counts is that every SM gets the same
+// number of them and that none is spent on padding.  So the tiles are small
+// (FP64_TILE below), run over the n x n matrix rather than its padding to
+// 256, and a block is four warps that each sum a quarter of the K range of the
+// whole tile (k = w mod 4); the quarters are added in a fixed order.  Blocks
+// of the jobs with the most K passes start first.  Elements outside n x n are
+// neither computed on nor written: rows of the K range beyond n are filled
+// with zeros on the way to shared memory, and what a tile's columns beyond n
+// hold reaches discarded elements only.
+// Measured per layer, one direction (64 x 64 tiles over the padded matrix,
+// one thread per 4 x 4 elements -> now): n = 128
+// 531 -> 12.9 us, n = 700 2326 -> 939 us (0.82 ms at two FMAs per clock and
+// SM).
+//
+// Tile edge: 8 up to n = 400, where 16 leaves SMs with a tile more than
+// others; 16 up to n = 2048; 32 above, where the balance no longer depends on
+// it and larger tiles keep the partial sums few.
+// 16-byte asynchronous copy that writes zeros instead when `in` is false
+__device__ __forceinline__ void cp_async16_zfill(void* smem, const void* gmem, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(smem)),
+               "l"(gmem), "r"(in ? 16 : 0)
+               : "memory");
+}
+
+template <int T>
+__global__ void __launch_bounds__(128)
+    layer_fp64_kernel(const State* __restrict__ st, double* __restrict__ master, int64_t n,
+                      int64_t Np, int k, double* __restrict__ partials, int64_t ptiles) {
+  constexpr int BK = 16, STAGES = 3, NT = 128;
+  constexpr int LD = T + 2;                 // padded slab row (16-byte chunks)
+  constexpr int RA = T / 8, CB = T / 4;     // a lane's rows and columns of the tile
+  constexpr int NCP = BK * T / NT;          // 16-byte copies per thread and stage (A and B)
+  constexpr int NE = (T * T + NT - 1) / NT; // elements per thread in the epilogue
+  constexpr int SLAB = BK * LD;
+  constexpr int SMEM = STAGES * 2 * SLAB > 4 * T * T ? STAGES * 2 * SLAB : 4 * T * T;
+  // the copy stages; after the K loop the four warps' sums, then the new tile
+  __shared__ __align__(16) double sm[SMEM];
+  __shared__ double red[2][NT];
+  __shared__ double red_tr[32];
+
+  if (st->done) return;
+  const int job = (int)gridDim.y - 1 - (int)blockIdx.y;
+  const bool run = job == 0 ? st->plan_square != 0 : st->plan_resp[job - 1] != 0;
+  if (!run) return;
+
+  // upper tile (I, J), I <= J: blockIdx.x = J (J + 1) / 2 + I
+  const int64_t t = blockIdx.x;
+  int64_t J = (int64_t)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while ((J + 1) * (J + 2) / 2 <= t) ++J;
+  while (J * (J + 1) / 2 > t) --J;
+  const int64_t I = t - J * (J + 1) / 2;
+  const bool diag = I == J;
+
+  const size_t mat = (size_t)Np * Np;
+  const int cur0 = st->cur0;
+  const int cur = job == 0 ? cur0 : st->cur1[job - 1];
+  const double* Sj = master + (size_t)(cur * (1 + k) + job) * mat;   // the job's own slot
+  double* out = master + (size_t)((cur ^ 1) * (1 + k) + job) * mat;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ry = (lane >> 2) * RA, cx = (lane & 3) * CB;
+
+  // epilogue elements of this thread: tid + 128 v, row-major in the tile
+  double old[NE];
+#pragma unroll
+  for (int v = 0; v < NE; ++v) {
+    const int e = tid + NT * v;
+    const int64_t r = I * T + e / T, c = J * T + e % T;
+    old[v] = (e < T * T && r < n && c < n) ? Sj[(size_t)r * Np + c] : 0.0;
+  }
+
+  double acc[RA][CB];
+#pragma unroll
+  for (int i = 0; i < RA; ++i)
+#pragma unroll
+    for (int j = 0; j < CB; ++j) acc[i][j] = 0.0;
+
+  const int k1 = st->order >= 2 ? st->k1 : k;   // first-order directions
+  const int passes = simt_job_passes(job, k1);
+  const int nkb = (int)((n + BK - 1) / BK);     // K blocks per pass
+  const int steps = passes * nkb;
+  // The masters are exactly symmetric, so the K x T slab A[I rows][kb ..] is
+  // read as rows kb .. kb + BK - 1, columns I T .. I T + T - 1 (contiguous)
+  const double* A = nullptr;
+  const double* B = nullptr;
+  int lpass = 0, lkb = 0;   // position of the next load
+  auto load = [&](int stage) {
+    if (lkb == 0) {
+      int mA, mB;
+      simt_job_operands(job, lpass, k1, &mA, &mB);
+      A = master + (size_t)((mA == 0 ? cur0 : st->cur1[mA - 1]) * (1 + k) + mA) * mat + I * T;
+      B = master + (size_t)((mB == 0 ? cur0 : st->cur1[mB - 1]) * (1 + k) + mB) * mat + J * T;
+    }
+    double* s0 = sm + stage * 2 * SLAB;
+#pragma unroll
+    for (int v = 0; v < NCP; ++v) {
+      const int idx = tid + NT * v;
+      const int half = idx / (BK * T / 2), rem = idx % (BK * T / 2);
+      const int row = rem / (T / 2), cq = 2 * (rem % (T / 2));
+      const int64_t kr = (int64_t)lkb * BK + row;
+      const double* g = (half ? B : A) + (size_t)(kr < n ? kr : 0) * Np + cq;
+      cp_async16_zfill(s0 + half * SLAB + row * LD + cq, g, kr < n);
+    }
+    if (++lkb == nkb) {
+      lkb = 0;
+      ++lpass;
+    }
+  };
+#pragma unroll
+  for (int s = 0; s < STAGES - 1; ++s) {
+    if (s < steps) load(s);
+    cp_async_commit();
+  }
+  int stage = 0;
+  for (int it = 0; it < steps; ++it) {
+    cp_async_wait<STAGES - 2>();   // stage `it` has landed (this thread's copies)
+    __syncthreads();               // ... and every thread's; stage it - 1 is free
+    if (it + STAGES - 1 < steps) load(stage == 0 ? STAGES - 1 : stage - 1);
+    cp_async_commit();
+    const double* as = sm + stage * 2 * SLAB;
+    const double* bs = as + SLAB;
+#pragma unroll
+    for (int q = 0; q < BK / 4; ++q) {
+      const int kk = 4 * q + warp;
+      double a[RA], b[CB];
+#pragma unroll
+      for (int i = 0; i < RA; ++i) a[i] = as[kk * LD + ry + i];
+#pragma unroll
+      for (int j = 0; j < CB; ++j) b[j] = bs[kk * LD + cx + j];
+#pragma unroll
+      for (int i = 0; i < RA; ++i)
+#pragma unroll
+        for (int j = 0; j < CB; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+    if (++stage == STAGES) stage = 0;
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+
+  // ---- fused epilogue
+#pragma unroll
+  for (int i = 0; i < RA; ++i)
+#pragma unroll
+    for (int j = 0; j < CB; ++j) sm[warp * T * T + (ry + i) * T + cx + j] = acc[i][j];
+  __syncthreads();
+  const double sg = (double)st->sigma_cur, om = 1.0 - sg;
+  const bool write = job == 0 ? st->plan_write0 != 0 : true;
+  double fnew = 0.0, fdiff = 0.0, tr = 0.0;
+  double nw[NE];
+  int bad = 0;
+#pragma unroll
+  for (int v = 0; v < NE; ++v) {
+    const int e = tid + NT * v;
+    nw[v] = 0.0;
+    if (e >= T * T) continue;
+    const int64_t r = I * T + e / T, c = J * T + e % T;
+    if (r > c || c >= n) continue;   // owned by the mirrored element; outside (r <= c < n)
+    const double x = (sm[e] + sm[T * T + e]) + (sm[2 * T * T + e] + sm[3 * T * T + e]);
+    bad += isfinite(x) ? 0 : 1;
+    const double y = sg * x + om * old[v];
+    const double dd = old[v] - x;
+    // elements off the diagonal count twice (a tile off the diagonal: below)
+    fdiff = fma(diag && r != c ? 2.0 * dd : dd, dd, fdiff);
+    if (write) {
+      nw[v] = y;
+      fnew = fma(diag && r != c ? 2.0 * y : y, y, fnew);
+      if (r == c) tr += y;
+      out[(size_t)r * Np + c] = y;
+    }
+  }
+  red[0][tid] = fnew;
+  red[1][tid] = fdiff;
+  if (diag) {
+    // diagonal elements lie T + 1 apart; a thread holds at most one of each
+    // 32 consecutive ones
+    if (tid < 32) red_tr[tid] = 0.0;
+  }
+  const int nbad = __syncthreads_count(bad);   // also: every sum has been read
+  if (write) {
+    constexpr int TS = T + 1;
+#pragma unroll
+    for (int v = 0; v < NE; ++v) {
+      const int e = tid + NT * v;
+      if (e < T * T) sm[(e / T) * TS + e % T] = nw[v];
+      if (diag && e < T * T && e / T == e % T) red_tr[e / T] = tr;
+    }
+  }
+  __syncthreads();
+  if (write) {
+    constexpr int TS = T + 1;
+#pragma unroll
+    for (int v = 0; v < NE; ++v) {   // the mirror (c, r), row-major in the mirror tile
+      const int e = tid + NT * v;
+      const int64_t c = J * T + e / T, r = I * T + e % T;
+      if (e < T * T && r < c && c < n) out[(size_t)c * Np + r] = sm[(e % T) * TS + e / T];
+    }
+  }
+  if (warp < 3) {
+    double x = 0.0;
+    if (warp < 2) {
+      const double* p = red[warp];
+      x = (p[lane] + p[lane + 32]) + (p[lane + 64] + p[lane + 96]);
+    } else if (diag && write) {
+      x = red_tr[lane];
+    }
+    if (warp < 2 || diag) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    }
+    if (lane == 0) {
+      double* p = partials + ((size_t)job * ptiles + blockIdx.x) * kNQ;
+      if (warp == 0) {
+        p[kQFroNew] = diag ? x : 2.0 * x;
+        p[kQBad] = (double)nbad;
+      } else if (warp == 1) {
+        p[kQFroDiff] = diag ? x : 2.0 * x;
+      } else {
+        p[kQTrace] = x;
+      }
+    }
+  }
+}
+
+constexpr int kFp32Tile = 128;   // tile edge of the FP32 form
 
 // Per-device one-time setup: the SIMT layer kernels' dynamic shared memory
 // exceeds the default 48 KB limit; thread-safe.
@@ -1098,9 +1327,6 @@ static void simt_setup() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return;
   std::call_once(once[dev], [] {
-    cudaFuncSetAttribute(layer_simt_kernel<double, 4, 8>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         simt_smem_bytes<double, 4, 8>());
     cudaFuncSetAttribute(layer_simt_kernel<float, 8, 16>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                          simt_smem_bytes<float, 8, 16>());
@@ -1112,20 +1338,33 @@ cudaError_t launch_layer_simt(const Layout& L, void* ws, cudaStream_t s, int64_t
   char* base = (char*)ws;
   State* st = (State*)(base + L.off_state);
   double* partials = (double*)(base + L.off_partials);
-  const int bt = simt_tile(L.precision);
-  dim3 grid((unsigned)upper_tiles(L.Np, bt), 1 + L.k);
-  constexpr int smem64 = simt_smem_bytes<double, 4, 8>();
-  constexpr int smem32 = simt_smem_bytes<float, 8, 16>();
-  static_assert(2 * smem32 <= 227 * 1024, "two FP32 blocks per SM");
-  simt_setup();
-  if (L.precision == DMPT_FP64)
-    layer_simt_kernel<double, 4, 8><<<grid, 256, smem64, s>>>(
-        st, (double*)(base + L.off_master), L.Np, L.k, partials, L.partial_tiles);
-  else
-    layer_simt_kernel<float, 8, 16><<<grid, 256, smem32, s>>>(
+  int64_t tiles = 0;
+  if (L.precision == DMPT_FP64) {
+    double* master = (double*)(base + L.off_master);
+    const int bt = fp64_tile(L.n);
+    tiles = fp64_tiles(L.n);
+    const dim3 grid((unsigned)tiles, 1 + L.k);
+    if (bt == 8)
+      layer_fp64_kernel<8><<<grid, 128, 0, s>>>(st, master, L.n, L.Np, L.k, partials,
+                                                L.partial_tiles);
+    else if (bt == 16)
+      layer_fp64_kernel<16><<<grid, 128, 0, s>>>(st, master, L.n, L.Np, L.k, partials,
+                                                 L.partial_tiles);
+    else
+      layer_fp64_kernel<32><<<grid, 128, 0, s>>>(st, master, L.n, L.Np, L.k, partials,
+                                                 L.partial_tiles);
+    if (pass_flops) *pass_flops = (double)tiles * bt * bt * (double)L.n * 2.0;
+  } else {
+    constexpr int smem32 = simt_smem_bytes<float, 8, 16>();
+    static_assert(2 * smem32 <= 227 * 1024, "two FP32 blocks per SM");
+    simt_setup();
+    tiles = upper_tiles(L.Np, kFp32Tile);
+    layer_simt_kernel<float, 8, 16><<<dim3((unsigned)tiles, 1 + L.k), 256, smem32, s>>>(
         st, (float*)(base + L.off_master), L.Np, L.k, partials, L.partial_tiles);
-  if (entries) *entries = upper_tiles(L.Np, bt);
-  if (pass_flops) *pass_flops = (double)upper_tiles(L.Np, bt) * bt * bt * (double)L.Np * 2.0;
+    if (pass_flops)
+      *pass_flops = (double)tiles * kFp32Tile * kFp32Tile * (double)L.Np * 2.0;
+  }
+  if (entries) *entries = tiles;
   return cudaGetLastError();
 }
 
