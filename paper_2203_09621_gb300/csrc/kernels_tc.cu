@@ -64,12 +64,8 @@ constexpr int EPI_WARPS = 8;     // two per TMEM lane quadrant (column halves)
 constexpr int EPI_THREADS = 32 * EPI_WARPS;
 constexpr int EPI_WARP0 = 2;     // epilogue = warps 2 .. 9
 constexpr int NUM_THREADS = 64 + EPI_THREADS;
-// Epilogue scratch: a 2560-byte transpose buffer per epilogue warp (32 rows
-// of 20 words); it shares its space with the reduction array of the tile's
-// partial sums (EPI_THREADS x 4 doubles), which is used only after every
-// epilogue warp has left its tile epilogue.
-constexpr int EPI_SCRATCH = EPI_WARPS * 32 * 20 * 4;
-static_assert(EPI_SCRATCH >= EPI_THREADS * 4 * 8, "reduction array fits the scratch");
+// Epilogue scratch: the partial sums of a tile (tile_sums_out).
+constexpr int EPI_SCRATCH = 512;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* align */ + 1024 /* barriers etc */ +
                            EPI_SCRATCH;
 constexpr int DEFAULT_CHUNK_K = 256;  // K elements per tensor-memory accumulation chunk
@@ -224,12 +220,29 @@ struct Cvt<false> {
   using T = __half;
   static __device__ __forceinline__ T to(float x) { return __float2half_rn(x); }
   static __device__ __forceinline__ float from(T h) { return __half2float(h); }
+  static __device__ __forceinline__ uint32_t pack(float a, float b) {   // a in the low half
+    const __half2 v = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  static __device__ __forceinline__ void unpack(uint32_t v, float& a, float& b) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&v));
+    a = f.x;
+    b = f.y;
+  }
 };
 template <>
 struct Cvt<true> {
   using T = __nv_bfloat16;
   static __device__ __forceinline__ T to(float x) { return __float2bfloat16_rn(x); }
   static __device__ __forceinline__ float from(T h) { return __bfloat162float(h); }
+  static __device__ __forceinline__ uint32_t pack(float a, float b) {   // a in the low half
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  static __device__ __forceinline__ void unpack(uint32_t v, float& a, float& b) {
+    a = __uint_as_float(v << 16);
+    b = __uint_as_float(v & 0xffff0000u);
+  }
 };
 
 // AND of a predicate over the epilogue threads (named barrier 1).
@@ -335,105 +348,199 @@ __device__ __forceinline__ uint32_t h16_bits(H16 x) {
   return (uint32_t)(*reinterpret_cast<const uint16_t*>(&x));
 }
 
-// Rolled tile epilogue of one thread: its row r, columns c0 .. c0 + 127 of a
-// pair tile, whose sums the caller has written to tensor memory at ta_sum.
-// Forms S_new = sigma X + (1 - sigma) S_old (Eq. (eq:Sn) / Eq. (dB)), its
-// FP16/BF16 hi/lo split (Sec. II C), the partial sums (||S_new||_F^2 with
-// TwoSum compensation, ||S_old - X||_F^2, trace, non-finite count) and stores
-// each owned element (column >= row).  OFF: the tile is off the diagonal
-// (every column > every row).
+// Packed FP32 pairs (two elements per 64-bit register): fma / mul / add with
+// the rounding of the scalar instructions, at half their issue slots.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// (s, c) += (s2, c2): sums held as s + c, the rounding of s kept in c (TwoSum)
+__device__ __forceinline__ void ff_add(float& s, float& c, float s2, float c2) {
+  const float t = s + s2;
+  const float b = t - s;
+  c += c2 + ((s - (t - b)) + (s2 - b));
+  s = t;
+}
+
+// Partial sums of one thread's part of a tile: sums held as s + c pairs.
+struct TileSums {
+  float fn_s = 0.0f, fn_c = 0.0f;   // ||S_new||^2
+  float fd_s = 0.0f, fd_c = 0.0f;   // ||S_old - X||^2
+  float tr = 0.0f;                  // diagonal of S_new (at most one element per thread)
+  bool bad = false;                 // a non-finite X
+};
+
+// 32 bytes to a 32-byte aligned address (one store instruction)
+__device__ __forceinline__ void store32(void* p, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
+               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+
+// Rolled tile epilogue of one thread: its row r (lane = row of the warp's 32),
+// columns c0 .. c0 + 16 NG - 1 of a tile, whose sums the caller has written to
+// tensor memory at ta_sum.  Forms S_new = sigma X + (1 - sigma) S_old
+// (Eq. (eq:Sn) / Eq. (dB)), its FP16/BF16 hi/lo split (Sec. II C), the partial
+// sums and stores each owned element (column >= row).  `release` is called
+// when the sums have been read from tensor memory.
 //
-// Memory access pattern.  A warp holds 32 consecutive rows (one per lane)
-// and the same columns, so an access down a column (lane = row) is one
-// contiguous segment while an access along its rows touches 32 lines.
+// Sixteen columns at a time; a warp's group of 16 columns lies above its 32
+// rows (every element owned: the packed path), below them (nothing to do) or
+// across the diagonal (at most two or three groups of a warp).
+//
+// Memory access pattern.  A warp holds 32 consecutive rows (one per lane) and
+// the same columns, so an access down a column (lane = row) is one contiguous
+// segment while an access along the rows touches 32 lines.
 //  * The FP32 master is kept in one orientation only: element (r, c),
 //    c >= r, at (c, r) (the lower triangle with the diagonal), written and
-//    read down the columns.  S_old[r][c] is read there, 16 columns per batch
-//    of loads; the next batch is loaded while the current one is stored.
-//    The readers of a whole master (outputs, checkpoint reloads) take
-//    element (r, c) from (max(r, c), min(r, c)).
+//    read down the columns.  S_old[r][c] is read there; the next 16 columns
+//    are loaded while the current ones are stored.  The readers of a whole
+//    master (outputs, checkpoint reloads) take element (r, c) from
+//    (max(r, c), min(r, c)).
 //  * The 16-bit operand copies, which the tensor maps read as row panels,
-//    are stored in both orientations: the mirror (c, r) down the columns,
-//    and (r, c) through this warp's transpose buffer `xp` in shared memory
-//    (32 rows of XP_STRIDE words; 16 columns at a time): each lane writes
-//    its row, then the warp stores 4 rows x 32 B (hi, lo) per instruction.
-//    The row stride of 20 words keeps both the 16-byte row writes and the
-//    column-pair reads free of bank conflicts.
-// The sums run over the columns in ascending order, so every thread's
-// partial sums do not depend on the memory access pattern.
-constexpr int XP_STRIDE = 20;                       // words per buffer row
-constexpr int XP_WARP_BYTES = 32 * XP_STRIDE * 4;   // 2560 B per epilogue warp
-static_assert(EPI_WARPS * XP_WARP_BYTES == EPI_SCRATCH, "transpose buffers");
-template <class CV, bool OFF, int NG = 8>   // NG groups of 16 columns per thread row
+//    are stored in both orientations.  Along the rows each lane stores its
+//    16 columns as one whole 32-byte sector.  Down the columns two lanes
+//    exchange halves so that each stores two rows of one column as a word.
+// What bounds it: the instructions of the eight epilogue warps (about 9 K
+// clocks per 128 x 256 part of a tile) and its stores (384 KB, 12 K clocks at
+// the 32 B per clock an SM writes), which overlap in part.  With scalar
+// arithmetic, 16-bit mirror stores, a shared-memory transpose for the rows and
+// an FP64 tree for the partial sums a layer of n = 1000, k = 2 took 57 us and
+// one of n = 2048, k = 3 157 us; now 51 and 149 us.  Sixteen warps of half the
+// columns, or loads of S_old two groups ahead, do not change it.
+template <class CV, int NG, class Rel>
 __device__ __forceinline__ void rolled_tile_epilogue(
     const uint32_t ta_sum, const float* __restrict__ Sold, float* Snew, typename CV::T* hi_new,
-    typename CV::T* lo_new, uint32_t* xp, const int lane, const int64_t Np, const int r,
-    const int c0, const float sg, const float om, const float scale_new, const bool write,
-    float& fn_s, float& fn_c, float& fd, float& trf, int& bad) {
+    typename CV::T* lo_new, const int lane, const int64_t Np, const int r, const int c0,
+    const float sg, const float om, const float scale_new, const bool write, TileSums& ts,
+    Rel release) {
   const int r0 = r - lane;   // row of lane 0
   const int np = (int)Np;
-  // element (c, r) of the tile's columns at col_base + (c - c0) * np; element
-  // (r0 + i, c) at row_base + i * np + (c - c0)  (32-bit offsets)
+  // groups below the warp's rows come first, groups above them last
+  int g16 = (r0 - c0) >> 4;
+  g16 = g16 < 0 ? 0 : g16;
+  if (g16 >= NG) {
+    release();
+    return;
+  }
+  // element (c, r) of the tile's columns at (c - c0) * np past col_base
   const size_t col_base = (size_t)c0 * Np + r;
-  const size_t row_base = (size_t)r0 * Np + c0;
+  const size_t row_base = (size_t)r * Np + c0;
   const float* Sc = Sold + col_base;
   float* Snc = Snew + col_base;
   uint16_t* hic = reinterpret_cast<uint16_t*>(hi_new) + col_base;
   uint16_t* loc = reinterpret_cast<uint16_t*>(lo_new) + col_base;
   uint16_t* hir = reinterpret_cast<uint16_t*>(hi_new) + row_base;
   uint16_t* lor = reinterpret_cast<uint16_t*>(lo_new) + row_base;
+  // column pairs: even lanes store (rows r, r + 1) of the even column, odd
+  // lanes (rows r - 1, r) of the odd one
+  const int odd = lane & 1;
+  const uint32_t sel = odd ? 0x3276u : 0x5410u;
+  uint16_t* hip = hic + (odd ? np - 1 : 0);
+  uint16_t* lop = loc + (odd ? np - 1 : 0);
+  const f32x2 sg2 = pack2(sg, sg), om2 = pack2(om, om), sc2 = pack2(scale_new, scale_new);
+  const f32x2 neg2 = pack2(-1.0f, -1.0f), zero2 = pack2(0.0f, 0.0f);
+  f32x2 fs = zero2, fc = zero2, fd = zero2, z = zero2;
   float olds[16];   // S_old of the current 16 columns; the next 16 are loaded
                     // while the current ones are stored
 #pragma unroll
-  for (int q = 0; q < 16; ++q) olds[q] = __ldg(Sc + q * np);
+  for (int q = 0; q < 16; ++q) olds[q] = __ldg(Sc + (16 * g16 + q) * np);
 #pragma unroll 1
-  for (int g16 = 0; g16 < NG; ++g16) {
+  for (; g16 < NG; ++g16) {
     uint32_t xs[16];
     tmem_ld16(ta_sum + 16 * g16, xs);
+    if (g16 == NG - 1) release();
     const int cb16 = c0 + 16 * g16;
-    // the hi/lo bits stay in registers, packed in column pairs, until the
-    // group's values are formed
-    uint32_t hp[8], lp[8];
+    uint32_t hp[8], lp[8];   // hi / lo of the column pairs
+    if (cb16 >= r0 + 32) {   // every column right of every row
 #pragma unroll
-    for (int i = 0; i < 8; ++i) hp[i] = lp[i] = 0u;
-#pragma unroll
-    for (int gg = 0; gg < 4; ++gg) {
-      const int cb = cb16 + 4 * gg;
-      if (!OFF && r > cb + 3) continue;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int e = 4 * gg + i;
-        const float xv = __uint_as_float(xs[e]);
-        const int c = cb + i;
-        const bool own = OFF || c >= r;
-        const float w = (!OFF && c == r) ? 1.0f : 2.0f;
-        bad += (own && !isfinite(xv)) ? 1 : 0;
-        const float old = olds[e];
-        const float dd = old - xv;
-        fd = own ? fmaf(w * dd, dd, fd) : fd;
-        const float n1 = sg * xv + om * old;
-        if (own && write) {
-          const float p = w * n1 * n1;
-          const float ee = w * fmaf(n1, n1, -n1 * n1);
-          const float tt = fn_s + p;
-          const float bp = tt - fn_s;
-          fn_c += (fn_s - (tt - bp)) + (p - bp) + ee;
-          fn_s = tt;
-          if (!OFF && c == r) trf += n1;
+      for (int i = 0; i < 8; ++i) {
+        const f32x2 x = pack2(__uint_as_float(xs[2 * i]), __uint_as_float(xs[2 * i + 1]));
+        const f32x2 o = pack2(olds[2 * i], olds[2 * i + 1]);
+        z = fma2(x, zero2, z);               // becomes NaN with a non-finite x
+        const f32x2 d = fma2(x, neg2, o);
+        fd = fma2(d, d, fd);                 // each element counts twice: at the end
+        const f32x2 nw = fma2(sg2, x, mul2(om2, o));
+        // ||S_new||^2: the square as p + e (p = -np2), fs + p by TwoSum
+        const f32x2 np2 = mul2(nw, mul2(nw, neg2));
+        const f32x2 e = fma2(nw, nw, np2);
+        const f32x2 tt = fma2(np2, neg2, fs);
+        const f32x2 bp = fma2(fs, neg2, tt);
+        const f32x2 t2 = fma2(fma2(bp, neg2, tt), neg2, fs);
+        const f32x2 t3 = add2(np2, bp);
+        fc = add2(fc, add2(fma2(t3, neg2, t2), e));
+        fs = tt;
+        const f32x2 y = mul2(nw, sc2);
+        float y0, y1, n0, n1;
+        unpack2(y, y0, y1);
+        unpack2(nw, n0, n1);
+        float h0, h1;
+        hp[i] = CV::pack(y0, y1);
+        CV::unpack(hp[i], h0, h1);
+        float l0, l1;
+        unpack2(fma2(pack2(h0, h1), neg2, y), l0, l1);
+        lp[i] = CV::pack(l0, l1);
+        if (write) {
+          const int m = (16 * g16 + 2 * i) * np;
+          Snc[m] = n0;
+          Snc[m + np] = n1;
+          const uint32_t ho = __shfl_xor_sync(0xffffffffu, hp[i], 1);
+          const uint32_t lo = __shfl_xor_sync(0xffffffffu, lp[i], 1);
+          *reinterpret_cast<uint32_t*>(hip + m) = __byte_perm(hp[i], ho, sel);
+          *reinterpret_cast<uint32_t*>(lop + m) = __byte_perm(lp[i], lo, sel);
         }
+      }
+      if (write) {
+        store32(hir + 16 * g16, hp);
+        store32(lor + 16 * g16, lp);
+      }
+    } else {   // a group on the diagonal
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        const int c = cb16 + e;
+        if (c < r) continue;   // owned by the mirrored element
+        const float xv = __uint_as_float(xs[e]);
+        const float w = c == r ? 0.5f : 1.0f;
+        ts.bad = ts.bad || !isfinite(xv);
+        const float dd = olds[e] - xv;
+        ts.fd_s = fmaf(w * dd, dd, ts.fd_s);
+        if (!write) continue;
+        const float n1 = sg * xv + om * olds[e];
+        const float p = w * n1 * n1;
+        ff_add(ts.fn_s, ts.fn_c, p, fmaf(w * n1, n1, -p));
+        if (c == r) ts.tr = n1;
         const float y = n1 * scale_new;
         const typename CV::T h = CV::to(y);
-        const uint32_t hbits = h16_bits(h);
-        const uint32_t lbits = h16_bits(CV::to(y - CV::from(h)));
-        hp[e >> 1] |= hbits << (16 * (e & 1));
-        lp[e >> 1] |= lbits << (16 * (e & 1));
-        if (write && own) {   // (c, r), down the column
-          const int m = (c - c0) * np;
-          Snc[m] = n1;
-          if (OFF || c > r) {   // the 16-bit mirror; the diagonal goes with the rows
-            hic[m] = (uint16_t)hbits;
-            loc[m] = (uint16_t)lbits;
-          }
+        const uint16_t hb = (uint16_t)h16_bits(h);
+        const uint16_t lb = (uint16_t)h16_bits(CV::to(y - CV::from(h)));
+        const int m = (16 * g16 + e) * np;
+        Snc[m] = n1;
+        hir[16 * g16 + e] = hb;
+        lor[16 * g16 + e] = lb;
+        if (c > r) {
+          hic[m] = hb;
+          loc[m] = lb;
         }
       }
     }
@@ -441,33 +548,64 @@ __device__ __forceinline__ void rolled_tile_epilogue(
 #pragma unroll
       for (int q = 0; q < 16; ++q) olds[q] = __ldg(Sc + (16 * (g16 + 1) + q) * np);
     }
-    if (!write) continue;
-    // ---- 16-bit copies in the row direction (r, c) through the transpose buffer
-    uint4* xr4 = reinterpret_cast<uint4*>(xp + lane * XP_STRIDE);
-    xr4[0] = make_uint4(hp[0], hp[1], hp[2], hp[3]);
-    xr4[1] = make_uint4(hp[4], hp[5], hp[6], hp[7]);
-    xr4[2] = make_uint4(lp[0], lp[1], lp[2], lp[3]);
-    xr4[3] = make_uint4(lp[4], lp[5], lp[6], lp[7]);
-    __syncwarp();
-#pragma unroll
-    for (int sidx = 0; sidx < 8; ++sidx) {
-      const int i = 8 * (sidx >> 1) + (sidx & 1) + 2 * (lane >> 3);   // rows i, +2, +4, +6
-      const int m = lane & 7;                                           // column pair
-      const uint32_t vh = xp[i * XP_STRIDE + m];
-      const uint32_t vl = xp[i * XP_STRIDE + 8 + m];
-      const int rr = r0 + i, c = cb16 + 2 * m;
-      const int o = i * np + (c - c0);
-      if (OFF || c >= rr) {
-        *reinterpret_cast<uint32_t*>(hir + o) = vh;
-        *reinterpret_cast<uint32_t*>(lor + o) = vl;
-      } else if (c + 1 >= rr) {
-        hir[o + 1] = (uint16_t)(vh >> 16);
-        lor[o + 1] = (uint16_t)(vl >> 16);
-      }
-    }
-    __syncwarp();
   }
+  float a0, a1, b0, b1;
+  unpack2(fs, a0, a1);
+  unpack2(fc, b0, b1);
+  ff_add(ts.fn_s, ts.fn_c, a0, b0);
+  ff_add(ts.fn_s, ts.fn_c, a1, b1);
+  unpack2(fd, a0, a1);
+  ff_add(ts.fd_s, ts.fd_c, a0, 0.0f);
+  ff_add(ts.fd_s, ts.fd_c, a1, 0.0f);
+  unpack2(z, a0, a1);
+  ts.bad = ts.bad || !(a0 == 0.0f) || !(a1 == 0.0f);
 }
+
+// Partial sums of a CTA's part of a tile: each epilogue warp adds its lanes'
+// sums as s + c pairs and leaves them in `red` (two buffers, used by
+// successive items in turn); after one barrier the warp whose turn it is
+// (`seq` mod EPI_WARPS) adds the eight warps in FP64 and writes the entry,
+// while the others go on.  (Every thread's sums through an FP64 tree in
+// shared memory took ten barriers and about 5 K clocks per item.)
+constexpr int RED_FLOATS = 8;   // per warp: fn (s, c), fd (s, c), tr (s, c), bad, -
+static_assert(2 * EPI_WARPS * RED_FLOATS * 4 <= EPI_SCRATCH, "two buffers");
+__device__ __forceinline__ void tile_sums_out(TileSums ts, float* red, uint32_t seq, int ewarp,
+                                              int lane, double* entry) {
+  float tc = 0.0f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float ns = __shfl_down_sync(0xffffffffu, ts.fn_s, o);
+    const float nc = __shfl_down_sync(0xffffffffu, ts.fn_c, o);
+    const float ds = __shfl_down_sync(0xffffffffu, ts.fd_s, o);
+    const float dc = __shfl_down_sync(0xffffffffu, ts.fd_c, o);
+    const float t2 = __shfl_down_sync(0xffffffffu, ts.tr, o);
+    const float tc2 = __shfl_down_sync(0xffffffffu, tc, o);
+    ff_add(ts.fn_s, ts.fn_c, ns, nc);
+    ff_add(ts.fd_s, ts.fd_c, ds, dc);
+    ff_add(ts.tr, tc, t2, tc2);
+  }
+  const bool bad = __any_sync(0xffffffffu, ts.bad);
+  float* buf = red + (seq & 1u) * EPI_WARPS * RED_FLOATS;
+  if (lane == 0) {
+    float4* p = reinterpret_cast<float4*>(buf + ewarp * RED_FLOATS);
+    p[0] = make_float4(ts.fn_s, ts.fn_c, ts.fd_s, ts.fd_c);
+    p[1] = make_float4(ts.tr, tc, bad ? 1.0f : 0.0f, 0.0f);
+  }
+  epi_sync();
+  if (ewarp != (int)(seq % EPI_WARPS)) return;
+  // lane 4 w + q: quantity q of warp w (trace, fro_new, fro_diff, bad)
+  const int q = lane & 3, w = lane >> 2;
+  const float* p = buf + w * RED_FLOATS;
+  double v = q == 0 ? (double)p[4] + (double)p[5]
+                    : (q == 1 ? (double)p[0] + (double)p[1]
+                              : (q == 2 ? (double)p[2] + (double)p[3] : (double)p[6]));
+#pragma unroll
+  for (int o = 16; o >= 4; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  // elements off the diagonal count twice (and those on it were halved)
+  if (lane < 4) entry[lane] = (lane == kQFroNew || lane == kQFroDiff) ? 2.0 * v : v;
+}
+static_assert(kQTrace == 0 && kQFroNew == 1 && kQFroDiff == 2 && kQBad == 3 && EPI_WARPS == 8,
+              "lanes of tile_sums_out");
 
 template <bool BF16>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
@@ -511,7 +649,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const uint32_t bar_drain = bar_tempty + 8 * 2;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 128);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 136);
-  double* red = reinterpret_cast<double*>(misc + 1024);
+  float* red = reinterpret_cast<float*>(misc + 1024);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -676,12 +814,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int q = warp & 3;                 // TMEM lane quadrant of this warp
     const int half = (warp - EPI_WARP0) >> 2;  // column half: 0 -> 0..127, 1 -> 128..255
     const int rloc = 32 * q + lane;         // row within the tile
-    const int et = threadIdx.x - 32 * EPI_WARP0;  // 0..255
     const size_t mat = (size_t)Np * Np;
     const uint32_t tlane = (uint32_t)(32 * q) << 16;
     int ab = 0;
     uint32_t abphase = 0;
     bool alive = true;
+    uint32_t seq = 0;   // items done (tile_sums_out)
     const bool crev = false;   // this kernel always runs the passes forwards
     for (int64_t it = blockIdx.x; it < items && alive; it += gridDim.x) {
       const int job = job_at(jmask, (int)(it / tiles));
@@ -749,49 +887,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       H16* hi_new = reinterpret_cast<H16*>(ops) + (size_t)zh_new * mat;
       H16* lo_new = reinterpret_cast<H16*>(ops) + (size_t)(zh_new + 1) * mat;
 
-      // Partial norms in FP32 with compensation (GB300's FP64 rate is a small
-      // fraction of its FP32 rate): ||S_new||^2 feeds the Alg. 2 test, so its
-      // products are split exactly (FMA) and summed with TwoSum; the
-      // FroErr sums only enter ratio tests and use plain FP32.
-      float fn_s = 0.0f, fn_c = 0.0f, fd = 0.0f, trf = 0.0f;
-      int bad = 0;
-      uint32_t* xp = reinterpret_cast<uint32_t*>(misc + 1024) +
-                     (warp - EPI_WARP0) * (XP_WARP_BYTES / 4);
-      if (I * BM + BM - 1 < J * BN)   // every column of the tile above every row
-        rolled_tile_epilogue<CV, true>(ta_sum, Sold, Snew, hi_new, lo_new, xp, lane, Np, r, c0,
-                                       sg, om, scale_new, write, fn_s, fn_c, fd, trf, bad);
-      else
-        rolled_tile_epilogue<CV, false>(ta_sum, Sold, Snew, hi_new, lo_new, xp, lane, Np, r, c0,
-                                        sg, om, scale_new, write, fn_s, fn_c, fd, trf, bad);
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_tempty + 8 * ab);
+      TileSums ts;
+      auto release = [&]() {   // the accumulator goes back to the MMA
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_tempty + 8 * ab);
+      };
+      rolled_tile_epilogue<CV, 8>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
+                                   scale_new, write, ts, release);
       if (++ab == 2) {
         ab = 0;
         abphase ^= 1;
       }
-      epi_sync();   // the reduction array overlays the transpose buffers
-      // deterministic tile reduction over the 256 epilogue threads (FP64)
-      red[0 * EPI_THREADS + et] = (double)trf;
-      red[1 * EPI_THREADS + et] = (double)fn_s + (double)fn_c;
-      red[2 * EPI_THREADS + et] = (double)fd;
-      red[3 * EPI_THREADS + et] = (double)bad;
-      epi_sync();
-      for (int s = EPI_THREADS / 2; s > 0; s >>= 1) {
-        if (et < s) {
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) red[qq * EPI_THREADS + et] += red[qq * EPI_THREADS + et + s];
-        }
-        epi_sync();
-      }
-      if (et == 0) {
-        double* p = partials + ((size_t)job * ptiles + t) * kNQ;
-        p[kQTrace] = red[0];
-        p[kQFroNew] = red[EPI_THREADS];
-        p[kQFroDiff] = red[2 * EPI_THREADS];
-        p[kQBad] = red[3 * EPI_THREADS];
-      }
-      epi_sync();
+      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, partials + ((size_t)job * ptiles + t) * kNQ);
     }
   }
 
@@ -1116,7 +1224,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const uint32_t bar_drain = bar_tempty + 8 * 2;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 264);
-  double* red = reinterpret_cast<double*>(misc + 1024);
+  float* red = reinterpret_cast<float*>(misc + 1024);
   const uint32_t lead_full = map_to_rank(bar_full, 0);
   const uint32_t lead_tempty = map_to_rank(bar_tempty, 0);
 
@@ -1202,12 +1310,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     const int q = warp & 3;
     const int half = (warp - EPI_WARP0) >> 2;
     const int rloc = 32 * q + lane;
-    const int et = threadIdx.x - 32 * EPI_WARP0;
     const size_t mat = (size_t)Np * Np;
     const uint32_t tlane = (uint32_t)(32 * q) << 16;
     int ab = 0;
     uint32_t abphase = 0;
     bool alive = true;
+    uint32_t seq = 0;   // items done (tile_sums_out)
     int64_t eround = 0;
     for (int64_t v = pair; v < vbase + items && alive; v += npairs, ++eround) {
       if (v < vbase) continue;
@@ -1273,44 +1381,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       H16* hi_new = reinterpret_cast<H16*>(ops) + (size_t)zh_new * mat;
       H16* lo_new = reinterpret_cast<H16*>(ops) + (size_t)(zh_new + 1) * mat;
 
-      float fn_s = 0.0f, fn_c = 0.0f, fd = 0.0f, trf = 0.0f;
-      int bad = 0;
-      uint32_t* xp = reinterpret_cast<uint32_t*>(misc + 1024) +
-                     (warp - EPI_WARP0) * (XP_WARP_BYTES / 4);
-      if (I2 < J)
-        rolled_tile_epilogue<CV, true>(ta_sum, Sold, Snew, hi_new, lo_new, xp, lane, Np, r, c0,
-                                       sg, om, scale_new, write, fn_s, fn_c, fd, trf, bad);
-      else
-        rolled_tile_epilogue<CV, false>(ta_sum, Sold, Snew, hi_new, lo_new, xp, lane, Np, r, c0,
-                                        sg, om, scale_new, write, fn_s, fn_c, fd, trf, bad);
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab);
+      TileSums ts;
+      auto release = [&]() {   // the accumulator goes back to the MMA
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab);
+      };
+      rolled_tile_epilogue<CV, 8>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
+                                   scale_new, write, ts, release);
       if (++ab == 2) {
         ab = 0;
         abphase ^= 1;
       }
-      epi_sync();   // the reduction array overlays the transpose buffers
-      red[0 * EPI_THREADS + et] = (double)trf;
-      red[1 * EPI_THREADS + et] = (double)fn_s + (double)fn_c;
-      red[2 * EPI_THREADS + et] = (double)fd;
-      red[3 * EPI_THREADS + et] = (double)bad;
-      epi_sync();
-      for (int s2 = EPI_THREADS / 2; s2 > 0; s2 >>= 1) {
-        if (et < s2) {
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) red[qq * EPI_THREADS + et] += red[qq * EPI_THREADS + et + s2];
-        }
-        epi_sync();
-      }
-      if (et == 0) {
-        double* pp = partials + ((size_t)job * ptiles + 2 * t + rank) * kNQ;
-        pp[kQTrace] = red[0];
-        pp[kQFroNew] = red[EPI_THREADS];
-        pp[kQFroDiff] = red[2 * EPI_THREADS];
-        pp[kQBad] = red[3 * EPI_THREADS];
-      }
-      epi_sync();
+      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, partials + ((size_t)job * ptiles + 2 * t + rank) * kNQ);
     }
   }
 
@@ -1488,7 +1571,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const uint32_t bar_drain = bar_tempty + 8 * 2;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 264);
-  double* red = reinterpret_cast<double*>(misc + 1024);
+  float* red = reinterpret_cast<float*>(misc + 1024);
   const uint32_t lead_full = map_to_rank(bar_full, 0);
   const uint32_t lead_tempty = map_to_rank(bar_tempty, 0);
 
@@ -1576,11 +1659,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     const int q = warp & 3;
     const int half = (warp - EPI_WARP0) >> 2;
     const int rloc = 32 * q + lane;
-    const int et = threadIdx.x - 32 * EPI_WARP0;
     const uint32_t tlane = (uint32_t)(32 * q) << 16;
     int ab = 0;
     uint32_t abphase = 0;
     bool alive = true;
+    uint32_t seq = 0;   // items done (tile_sums_out)
     for (int64_t j = 0; alive; ++j) {
       // lane 0 of each warp reads the claim; every epilogue warp agrees on it
       uint32_t g = kNoItem;
@@ -1660,44 +1743,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       H16* hi_new = reinterpret_cast<H16*>(gi.ops) + (size_t)zh_new * mat;
       H16* lo_new = reinterpret_cast<H16*>(gi.ops) + (size_t)(zh_new + 1) * mat;
 
-      float fn_s = 0.0f, fn_c = 0.0f, fd = 0.0f, trf = 0.0f;
-      int bad = 0;
-      uint32_t* xp = reinterpret_cast<uint32_t*>(misc + 1024) +
-                     (warp - EPI_WARP0) * (XP_WARP_BYTES / 4);
-      if (I2 < J)
-        rolled_tile_epilogue<CV, true>(ta_sum, Sold, Snew, hi_new, lo_new, xp, lane, Np, r, c0,
-                                       sg, om, scale_new, write, fn_s, fn_c, fd, trf, bad);
-      else
-        rolled_tile_epilogue<CV, false>(ta_sum, Sold, Snew, hi_new, lo_new, xp, lane, Np, r, c0,
-                                        sg, om, scale_new, write, fn_s, fn_c, fd, trf, bad);
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab);
+      TileSums ts;
+      auto release = [&]() {   // the accumulator goes back to the MMA
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab);
+      };
+      rolled_tile_epilogue<CV, 8>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
+                                   scale_new, write, ts, release);
       if (++ab == 2) {
         ab = 0;
         abphase ^= 1;
       }
-      epi_sync();   // the reduction array overlays the transpose buffers
-      red[0 * EPI_THREADS + et] = (double)trf;
-      red[1 * EPI_THREADS + et] = (double)fn_s + (double)fn_c;
-      red[2 * EPI_THREADS + et] = (double)fd;
-      red[3 * EPI_THREADS + et] = (double)bad;
-      epi_sync();
-      for (int s2 = EPI_THREADS / 2; s2 > 0; s2 >>= 1) {
-        if (et < s2) {
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) red[qq * EPI_THREADS + et] += red[qq * EPI_THREADS + et + s2];
-        }
-        epi_sync();
-      }
-      if (et == 0) {
-        double* pp = gi.partials + ((size_t)job * gi.ptiles + 2 * itm.t + rank) * kNQ;
-        pp[kQTrace] = red[0];
-        pp[kQFroNew] = red[EPI_THREADS];
-        pp[kQFroDiff] = red[2 * EPI_THREADS];
-        pp[kQBad] = red[3 * EPI_THREADS];
-      }
-      epi_sync();
+      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, gi.partials + ((size_t)job * gi.ptiles + 2 * itm.t + rank) * kNQ);
     }
   }
 
@@ -1925,7 +1983,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   static_assert(8 * (2 * G_STAGES + 2 * G_ACC + 1) <= 256, "barriers below the TMEM slot");
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 264);
-  double* red = reinterpret_cast<double*>(misc + 1024);
+  float* red = reinterpret_cast<float*>(misc + 1024);
   const uint32_t lead_full = map_to_rank(bar_full, 0);
   const uint32_t lead_tempty = map_to_rank(bar_tempty, 0);
 
@@ -2014,10 +2072,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     const int q = warp & 3;
     const int half = (warp - EPI_WARP0) >> 2;
     const int rloc = 32 * q + lane;
-    const int et = threadIdx.x - 32 * EPI_WARP0;
     const uint32_t tlane = (uint32_t)(32 * q) << 16;
     RingPos ab;
     bool alive = true;
+    uint32_t seq = 0;   // items done (tile_sums_out)
     for (int64_t j = 0; alive; ++j) {
       uint32_t g = kNoItem;
       bool got = true;
@@ -2093,47 +2151,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       H16* hi_new = reinterpret_cast<H16*>(gi.ops) + (size_t)zh_new * mat;
       H16* lo_new = reinterpret_cast<H16*>(gi.ops) + (size_t)(zh_new + 1) * mat;
 
-      float fn_s = 0.0f, fn_c = 0.0f, fd = 0.0f, trf = 0.0f;
-      int bad = 0;
-      uint32_t* xp = reinterpret_cast<uint32_t*>(misc + 1024) +
-                     (warp - EPI_WARP0) * (XP_WARP_BYTES / 4);
+      TileSums ts;
+      auto release = [&]() {   // the accumulator goes back to the MMA
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab.idx);
+      };
       // rows past Np (a 256-row block over a matrix padded to 128): nothing to
       // store; the products there are zeros
-      if ((int64_t)row0 < Np) {
-        if (c0 >= row0 + BM)   // every column of this warp's block right of every row
-          rolled_tile_epilogue<CV, true, 4>(ta_sum, Sold, Snew, hi_new, lo_new, xp, lane, Np, r,
-                                            c0, sg, om, scale_new, write, fn_s, fn_c, fd, trf,
-                                            bad);
-        else
-          rolled_tile_epilogue<CV, false, 4>(ta_sum, Sold, Snew, hi_new, lo_new, xp, lane, Np, r,
-                                             c0, sg, om, scale_new, write, fn_s, fn_c, fd, trf,
-                                             bad);
-      }
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab.idx);
+      if ((int64_t)row0 < Np)
+        rolled_tile_epilogue<CV, 4>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
+                                     scale_new, write, ts, release);
+      else
+        release();
       ab.next(G_ACC);
-      epi_sync();   // the reduction array overlays the transpose buffers
-      red[0 * EPI_THREADS + et] = (double)trf;
-      red[1 * EPI_THREADS + et] = (double)fn_s + (double)fn_c;
-      red[2 * EPI_THREADS + et] = (double)fd;
-      red[3 * EPI_THREADS + et] = (double)bad;
-      epi_sync();
-      for (int s2 = EPI_THREADS / 2; s2 > 0; s2 >>= 1) {
-        if (et < s2) {
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) red[qq * EPI_THREADS + et] += red[qq * EPI_THREADS + et + s2];
-        }
-        epi_sync();
-      }
-      if (et == 0) {
-        double* pp = gi.partials + ((size_t)job * gi.ptiles + 2 * itm.t + rank) * kNQ;
-        pp[kQTrace] = red[0];
-        pp[kQFroNew] = red[EPI_THREADS];
-        pp[kQFroDiff] = red[2 * EPI_THREADS];
-        pp[kQBad] = red[3 * EPI_THREADS];
-      }
-      epi_sync();
+      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, gi.partials + ((size_t)job * gi.ptiles + 2 * itm.t + rank) * kNQ);
     }
   }
 
