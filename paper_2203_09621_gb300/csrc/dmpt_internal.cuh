@@ -190,7 +190,7 @@ cudaError_t launch_scc_mix(const double* P1, int64_t n, int64_t ld, double* q, i
 cudaError_t launch_decide(const Layout& L, void* ws, int mode, int64_t entries,
                           cudaStream_t s);
 // Layer-product launchers.  *entries: partial-sum entries per job (tiles);
-// *pass_flops: flops of one full-K, single-term pass over all tiles.
+// *pass_flops: flops of one single-term pass over all tiles and the K range.
 cudaError_t launch_layer_simt(const Layout& L, void* ws, cudaStream_t s, int64_t* entries,
                               double* pass_flops);
 // 16-bit copies of the current masters of jobs first_job .. first_job + jobs - 1
@@ -249,6 +249,7 @@ struct GroupInst {
   int64_t Np;
   int64_t ptiles;      // partial-sum entries per job
   int k;
+  int kblocks;         // K blocks of 32 that hold columns < n
   int npairs;          // CTA pairs a single-instance launch would use (K-snake rounds)
 };
 // Per-instance inputs of the batched decide kernel.
