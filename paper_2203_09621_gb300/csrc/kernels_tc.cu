@@ -144,6 +144,40 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
   }
 }
 
+// One lane of a converged warp, the same one each time.  Code under it stays
+// warp-uniform for the compiler, so the operands of the tensor-core and TMA
+// instructions need no per-lane handling (see mma_item).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
+// mbar_wait by a whole converged warp: every lane gets the same answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint64_t limit_ns,
+                                               volatile int* abort_smem, int* timeout_global) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const uint64_t t0 = gtimer();
+  uint32_t it = 0;
+  while (true) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((++it & 255) == 0) {
+      const bool late = gtimer() - t0 > limit_ns;
+      if (__any_sync(0xffffffffu, late || *abort_smem)) {
+        if (late) {
+          *abort_smem = 1;
+          atomicExch(timeout_global, 1);
+        }
+        return false;
+      }
+    }
+  }
+}
+
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y,
                                             int z, uint32_t bar) {
   asm volatile(
@@ -941,6 +975,23 @@ constexpr int P_STAGES = 6;
 constexpr int P_STAGE_BYTES = 2 * A_BYTES + 2 * A_BYTES;   // A hi/lo + B-half hi/lo: 32 KB
 constexpr int P_SMEM_BYTES = P_STAGES * P_STAGE_BYTES + 1024 + 1024 + EPI_SCRATCH;
 
+// Geometry of the pair kernels' tiles, 256 rows x NT columns: each CTA loads
+// its 128 A rows and NT / 2 B rows per stage, and tensor memory holds ACC
+// accumulators of NT columns.
+template <int NT>
+struct PairTile {
+  static constexpr int B_ROWS = NT / 2;
+  static constexpr int PB_BYTES = B_ROWS * BK * 2;
+  static constexpr int STAGE = 2 * A_BYTES + 2 * PB_BYTES;   // 32, 24, 20 KB
+  static constexpr int STAGES = P_STAGES * P_STAGE_BYTES / STAGE;
+  static constexpr int ACC = NT == 256 ? 2 : 4;
+  static constexpr int COLS = ACC * NT;                      // tensor-memory columns
+  static constexpr int SPLIT = BN / NT;                      // tiles per 256 x 256 tile
+};
+static_assert(8 * (2 * PairTile<64>::STAGES + 2 * PairTile<64>::ACC + 1) <= 256 &&
+                  8 * (2 * PairTile<128>::STAGES + 2 * PairTile<128>::ACC + 1) <= 256,
+              "barriers below the TMEM slot");
+
 __host__ __device__ inline int64_t num_pair_tiles(int64_t Np) {
   const int64_t tj = Np / BN;
   return tj * (tj + 1) / 2;
@@ -1033,9 +1084,9 @@ __device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
       " [%0], %1;" ::"r"(bar), "h"(mask)
       : "memory");
 }
-__host__ __device__ constexpr uint32_t make_idesc_m256(int ab_type) {
+__host__ __device__ constexpr uint32_t make_idesc_m256(int ab_type, int n) {
   return (1u << 4) | ((uint32_t)ab_type << 7) | ((uint32_t)ab_type << 10) |
-         ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+         ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 }
 
 // Position in the shared-memory stage ring (stage index and phase bit) or
@@ -1053,15 +1104,18 @@ struct RingPos {
 
 // TMA producer of a pair kernel, one work item: the item's passes over its
 // K blocks (backwards when `rev`), each stage the hi and lo halves of this
-// CTA's A rows and B rows, signalled on the pair leader's full barrier.
-// False when a bounded wait expired or the CTA aborted.
+// CTA's A rows (128-row map) and B rows (NT / 2-row map), signalled on the
+// pair leader's full barrier.  False when a bounded wait expired or the CTA
+// aborted.
+template <int NT>
 __device__ __forceinline__ bool produce_item(RingPos& rg, const CUtensorMap* map,
-                                             const State* st, int job, int passes, int k,
+                                             const CUtensorMap* mapB, const State* st, int job, int passes, int k,
                                              int k1, int cur0, int z0c, int rowA, int rowB,
                                              int kblocks, bool rev, bool leader, uint32_t ring,
                                              uint32_t bar_full, uint32_t bar_empty,
                                              uint32_t lead_full, uint64_t limit_ns,
                                              volatile int* abort_flag, int* timeout_global) {
+  using PT = PairTile<NT>;
   for (int pp = 0; pp < passes; ++pp) {
     const int pass = rev ? passes - 1 - pp : pp;
     int mA, mB;
@@ -1072,29 +1126,34 @@ __device__ __forceinline__ bool produce_item(RingPos& rg, const CUtensorMap* map
     const int zBh = zop(mB, bufB, 0, k, z0c), zBl = zop(mB, bufB, 1, k, z0c);
     for (int kq = 0; kq < kblocks; ++kq) {
       const int kb = rev ? kblocks - 1 - kq : kq;
-      if (!mbar_wait(bar_empty + 8 * rg.idx, rg.phase ^ 1, limit_ns, abort_flag, timeout_global))
+      if (!mbar_wait_warp(bar_empty + 8 * rg.idx, rg.phase ^ 1, limit_ns, abort_flag,
+                          timeout_global))
         return false;
-      const uint32_t sA = ring + rg.idx * P_STAGE_BYTES;
-      if (leader) mbar_expect_tx(bar_full + 8 * rg.idx, 2 * P_STAGE_BYTES);
+      const uint32_t sA = ring + rg.idx * PT::STAGE;
       const uint32_t fb = lead_full + 8 * rg.idx;
-      tma_load_3d_pair(sA, map, kb * BK, rowA, zAh, fb);
-      tma_load_3d_pair(sA + A_BYTES, map, kb * BK, rowA, zAl, fb);
-      tma_load_3d_pair(sA + 2 * A_BYTES, map, kb * BK, rowB, zBh, fb);
-      tma_load_3d_pair(sA + 3 * A_BYTES, map, kb * BK, rowB, zBl, fb);
-      rg.next(P_STAGES);
+      if (elect_one()) {
+        if (leader) mbar_expect_tx(bar_full + 8 * rg.idx, 2 * PT::STAGE);
+        tma_load_3d_pair(sA, map, kb * BK, rowA, zAh, fb);
+        tma_load_3d_pair(sA + A_BYTES, map, kb * BK, rowA, zAl, fb);
+        tma_load_3d_pair(sA + 2 * A_BYTES, mapB, kb * BK, rowB, zBh, fb);
+        tma_load_3d_pair(sA + 2 * A_BYTES + PT::PB_BYTES, mapB, kb * BK, rowB, zBl, fb);
+      }
+      __syncwarp();
+      rg.next(PT::STAGES);
     }
   }
   return true;
 }
 
 // Before a CTA exits, wait (bounded) for the copies it issued to land: the
-// last P_STAGES stages were released by MMA commits or are pending.
-__device__ __forceinline__ void producer_drain(RingPos rg, uint32_t bar_empty, uint64_t limit_ns) {
-  for (int i = 0; i < P_STAGES; ++i) {
+// last `stages` stages were released by MMA commits or are pending.
+__device__ __forceinline__ void producer_drain(RingPos rg, int stages, uint32_t bar_empty,
+                                               uint64_t limit_ns) {
+  for (int i = 0; i < stages; ++i) {
     const uint64_t t0 = gtimer();
     while (!mbar_try_wait(bar_empty + 8 * rg.idx, rg.phase ^ 1) && gtimer() - t0 < limit_ns) {
     }
-    rg.next(P_STAGES);
+    rg.next(stages);
   }
 }
 
@@ -1104,14 +1163,15 @@ __device__ __forceinline__ void producer_drain(RingPos rg, uint32_t bar_empty, u
 // stages and at the end of each K pass (so chunks never straddle a pass), the
 // first of a pass after chunk - cp0 stages, and is then published to both
 // CTAs.  False when a bounded wait expired.
-template <bool BF16>
+template <bool BF16, int NT>
 __device__ __forceinline__ bool mma_item(RingPos& rg, RingPos& tb, int nst, int kblocks,
                                          int chunk, int cp0, uint32_t tmem_base, uint32_t ring,
                                          uint32_t bar_full, uint32_t bar_empty,
                                          uint32_t bar_tfull, uint32_t bar_tempty,
                                          uint64_t limit_ns, volatile int* abort_flag,
                                          int* timeout_global) {
-  constexpr uint32_t idesc = make_idesc_m256(BF16 ? 1 : 0);
+  using PT = PairTile<NT>;
+  constexpr uint32_t idesc = make_idesc_m256(BF16 ? 1 : 0, NT);
   uint32_t d = 0, acc = 0;
   int sp = 0;   // stage within its K pass
   int cp = cp0;   // stage within its accumulation chunk
@@ -1119,33 +1179,38 @@ __device__ __forceinline__ bool mma_item(RingPos& rg, RingPos& tb, int nst, int 
   for (int si = 0; si < nst; ++si) {
     if (fresh) {
       fresh = false;
-      if (!mbar_wait(bar_tempty + 8 * tb.idx, tb.phase ^ 1, limit_ns, abort_flag, timeout_global))
+      if (!mbar_wait_warp(bar_tempty + 8 * tb.idx, tb.phase ^ 1, limit_ns, abort_flag,
+                          timeout_global))
         return false;
       fence_after();
-      d = tmem_base + (uint32_t)(tb.idx * BN);
+      d = tmem_base + (uint32_t)(tb.idx * NT);
       acc = 0;
     }
-    if (!mbar_wait(bar_full + 8 * rg.idx, rg.phase, limit_ns, abort_flag, timeout_global))
+    if (!mbar_wait_warp(bar_full + 8 * rg.idx, rg.phase, limit_ns, abort_flag, timeout_global))
       return false;
     fence_after();
-    const uint32_t sA = ring + rg.idx * P_STAGE_BYTES;
+    const uint32_t sA = ring + rg.idx * PT::STAGE;
     const uint64_t ah = sw64_desc(sA), al = sw64_desc(sA + A_BYTES);
     const uint64_t bh = sw64_desc(sA + 2 * A_BYTES);
-    const uint64_t bl = sw64_desc(sA + 3 * A_BYTES);
-#pragma unroll
-    for (int kk = 0; kk < BK / 16; ++kk) {
-      const uint64_t off = (uint64_t)((kk * 32) >> 4);
-      mma_f16_pair(d, ah + off, bh + off, idesc, acc);   // hi * hi
-      acc = 1;
-      mma_f16_pair(d, ah + off, bl + off, idesc, 1);     // hi * lo
-      mma_f16_pair(d, al + off, bh + off, idesc, 1);     // lo * hi
-    }
-    mma_commit_pair(bar_empty + 8 * rg.idx);   // frees the stage in both CTAs
-    rg.next(P_STAGES);
+    const uint64_t bl = sw64_desc(sA + 2 * A_BYTES + PT::PB_BYTES);
     const bool pass_end = ++sp == kblocks;
-    if (++cp == chunk || pass_end) {
-      mma_commit_pair(bar_tfull + 8 * tb.idx);    // chunk ready in both CTAs
-      tb.next(2);
+    const bool chunk_end = ++cp == chunk || pass_end;
+    if (elect_one()) {
+#pragma unroll
+      for (int kk = 0; kk < BK / 16; ++kk) {
+        const uint64_t off = (uint64_t)((kk * 32) >> 4);
+        mma_f16_pair(d, ah + off, bh + off, idesc, kk == 0 ? acc : 1u);   // hi * hi
+        mma_f16_pair(d, ah + off, bl + off, idesc, 1);                    // hi * lo
+        mma_f16_pair(d, al + off, bh + off, idesc, 1);                    // lo * hi
+      }
+      mma_commit_pair(bar_empty + 8 * rg.idx);   // frees the stage in both CTAs
+      if (chunk_end) mma_commit_pair(bar_tfull + 8 * tb.idx);   // chunk ready in both CTAs
+    }
+    __syncwarp();
+    acc = 1;
+    rg.next(PT::STAGES);
+    if (chunk_end) {
+      tb.next(PT::ACC);
       fresh = true;
       cp = pass_end ? cp0 : 0;
     }
@@ -1188,12 +1253,15 @@ __device__ __forceinline__ void round_start(unsigned* ctr, int64_t round, int64_
 // a time by rolled_tile_epilogue (no register spills, little code per tile);
 // the buffer returns to the MMA after that loop, so the MMA runs one chunk
 // ahead of the epilogue during it.
-template <bool BF16>
+template <bool BF16, int NT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
-    layer_tc2_kernel(const __grid_constant__ CUtensorMap mapA, State* st, float* __restrict__ master,
-                     uint16_t* __restrict__ ops, int64_t Np, int k, double* __restrict__ partials,
-                     int64_t ptiles, uint64_t limit_ns, int chunk, int k_snake, int band,
-                     int inject_stall, int round_align) {
+    layer_tc2_kernel(const __grid_constant__ CUtensorMap mapA,
+                     const __grid_constant__ CUtensorMap mapB, State* st,
+                     float* __restrict__ master, uint16_t* __restrict__ ops, int64_t Np, int k,
+                     double* __restrict__ partials, int64_t ptiles, uint64_t limit_ns, int chunk,
+                     int k_snake, int snake_pairs, int band, int inject_stall, int round_align) {
+  using PT = PairTile<NT>;
+  constexpr int SP = PT::SPLIT;
   using CV = Cvt<BF16>;
   using H16 = typename CV::T;
   extern __shared__ uint8_t smem_raw[];
@@ -1215,27 +1283,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   // a square alone: it then numbers the square's items as the forward launch
   // did, after its response items, so each tile keeps its round and K-snake
   // direction and the recomputed states are bit-identical)
-  const int64_t vbase = st->item_base;
+  const int64_t vbase = SP * st->item_base;
 
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
   const int64_t pair = blockIdx.x >> 1;
   const int64_t npairs = gridDim.x >> 1;
   const int64_t tiles = num_pair_tiles(Np);
-  const int64_t items = tiles * njobs;
+  const int64_t items = SP * tiles * njobs;
   const int kblocks = k_blocks(st->n);
 
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
   const uint32_t ring = base;
-  uint8_t* misc = gbase + P_STAGES * P_STAGE_BYTES;
+  uint8_t* misc = gbase + PT::STAGES * PT::STAGE;
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);
   const uint32_t bar_full = smem_u32(bars);
-  const uint32_t bar_empty = bar_full + 8 * P_STAGES;
-  const uint32_t bar_tfull = bar_empty + 8 * P_STAGES;
-  const uint32_t bar_tempty = bar_tfull + 8 * 2;
-  const uint32_t bar_drain = bar_tempty + 8 * 2;
+  const uint32_t bar_empty = bar_full + 8 * PT::STAGES;
+  const uint32_t bar_tfull = bar_empty + 8 * PT::STAGES;
+  const uint32_t bar_tempty = bar_tfull + 8 * PT::ACC;
+  const uint32_t bar_drain = bar_tempty + 8 * PT::ACC;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 264);
   float* red = reinterpret_cast<float*>(misc + 1024);
@@ -1246,11 +1314,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < P_STAGES; ++s) {
+    for (int s = 0; s < PT::STAGES; ++s) {
       mbar_init(bar_full + 8 * s, 1);
       mbar_init(bar_empty + 8 * s, 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < PT::ACC; ++b) {
       mbar_init(bar_tfull + 8 * b, 1);
       mbar_init(bar_tempty + 8 * b, 2 * EPI_WARPS);
     }
@@ -1261,7 +1329,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32((const void*)tmem_slot)),
-                 "r"(TMEM_COLS));
+                 "r"(PT::COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   fence_before();
@@ -1270,53 +1338,60 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
   int* timeout_global = &st->timeout_flag;
 
+  // All pairs move through their tiles' K ranges in near lockstep; in odd
+  // rounds of the 256 x 256 tiles the sweep runs backwards (passes and K
+  // blocks), so a round starts on the panel slices the previous round loaded
+  // last, which are still in L2.  Narrower tiles keep the direction of the
+  // 256 x 256 tile they are part of: an element's sums, and so the results,
+  // are the same bit for bit at every width.
+  auto item_rev = [&](int64_t v) { return k_snake && ((v / SP / snake_pairs) & 1); };
+
   if (warp == 0) {
     // ================= TMA producer (both CTAs load their own halves) ======
-    if (lane == 0) {
+    {
       RingPos rg;
       bool ok = true;
-      int64_t round = 0;
-      bool align = round_align != 0;
-      for (int64_t v = pair; v < vbase + items && ok; v += npairs, ++round) {
+      bool align = round_align != 0 && SP == 1;
+      for (int64_t v = pair; v < vbase + items && ok; v += npairs) {
         if (v < vbase) continue;
-        const int64_t it = v - vbase;
-        if (round > 0) round_start(&st->round_ctr, round, items, npairs, align);
+        const int64_t it = (v - vbase) / SP;
+        if (SP == 1 && v >= npairs) {
+          if (lane == 0) round_start(&st->round_ctr, v / npairs, items, npairs, align);
+          __syncwarp();
+        }
         const int job = job_at(jmask, (int)(it / tiles));
         int I2, J;
         pair_tile_banded(it % tiles, (int)(Np / BN), band, &I2, &J);
-        // all pairs move through their tiles' K ranges in near lockstep; in
-        // odd rounds the sweep runs backwards (passes and K blocks), so a
-        // round starts on the panel slices the previous round loaded last,
-        // which are still in L2
-        const bool rev = k_snake && (round & 1);
-        ok = produce_item(rg, &mapA, st, job, job_passes(job, k1), k, k1, cur0, z0c,
-                          I2 * 2 * BM + (int)rank * BM, J * BN + (int)rank * BM, kblocks, rev,
-                          leader, ring, bar_full, bar_empty, lead_full, limit_ns, abort_flag,
-                          timeout_global);
+        ok = produce_item<NT>(rg, &mapA, &mapB, st, job, job_passes(job, k1), k, k1, cur0, z0c,
+                              I2 * 2 * BM + (int)rank * BM,
+                              J * BN + (int)(v % SP) * NT + (int)rank * PT::B_ROWS, kblocks,
+                              item_rev(v), leader, ring, bar_full, bar_empty, lead_full, limit_ns,
+                              abort_flag, timeout_global);
       }
-      producer_drain(rg, bar_empty, limit_ns);
+      if (lane == 0) producer_drain(rg, PT::STAGES, bar_empty, limit_ns);
     }
   } else if (warp == 1) {
     // ================= MMA issuer (leader CTA only) =================
-    if (leader && lane == 0) {
+    if (leader) {
       RingPos rg, tb;
       // test hook (see the single-CTA kernel)
       bool ok = !(inject_stall &&
-                  !mbar_wait(bar_drain, 0, limit_ns, abort_flag, timeout_global));
+                  !mbar_wait_warp(bar_drain, 0, limit_ns, abort_flag, timeout_global));
       for (int64_t v = pair; v < vbase + items && ok; v += npairs) {
         if (v < vbase) continue;
-        const int64_t it = v - vbase;
+        const int64_t it = (v - vbase) / SP;
         const int job = job_at(jmask, (int)(it / tiles));
-        const bool rev = k_snake && ((v / npairs) & 1);   // same order as the producer
-        ok = mma_item<BF16>(rg, tb, job_passes(job, k1) * kblocks, kblocks, chunk,
-                            kchunk0(Np, kblocks, chunk, rev), tmem_base, ring,
-                            bar_full, bar_empty, bar_tfull, bar_tempty, limit_ns, abort_flag,
-                            timeout_global);
+        ok = mma_item<BF16, NT>(rg, tb, job_passes(job, k1) * kblocks, kblocks, chunk,
+                                kchunk0(Np, kblocks, chunk, item_rev(v)), tmem_base, ring,
+                                bar_full, bar_empty, bar_tfull, bar_tempty, limit_ns, abort_flag,
+                                timeout_global);
       }
-      asm volatile(
-          "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-              bar_drain)
-          : "memory");
+      if (elect_one())
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                bar_drain)
+            : "memory");
+      __syncwarp();
       const uint64_t t0 = gtimer();
       while (!mbar_try_wait(bar_drain, 0) && gtimer() - t0 < limit_ns) {
       }
@@ -1328,15 +1403,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     const int rloc = 32 * q + lane;
     const size_t mat = (size_t)Np * Np;
     const uint32_t tlane = (uint32_t)(32 * q) << 16;
-    int ab = 0;
-    uint32_t abphase = 0;
+    RingPos ab;
     bool alive = true;
     uint32_t seq = 0;   // items done (tile_sums_out)
-    int64_t eround = 0;
-    for (int64_t v = pair; v < vbase + items && alive; v += npairs, ++eround) {
+    for (int64_t v = pair; v < vbase + items && alive; v += npairs) {
       if (v < vbase) continue;
-      const int64_t it = v - vbase;
-      const bool crev = k_snake && (eround & 1);   // same order as the producer
+      const int64_t it = (v - vbase) / SP;
+      const bool crev = item_rev(v);
       const int job = job_at(jmask, (int)(it / tiles));
       const int passes = job_passes(job, k1);
       // chunks per pass
@@ -1345,22 +1418,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       // exact power-of-two unscale of the products of passes 0 and 1
       // (passes >= 2 of higher-order terms: cross_unscale)
       const float u01 = ldexpf(1.0f, -(s0e + (job == 0 ? s0e : st->s1_exp_cur[job - 1])));
-      float sum[128];
+      float sum[NT / 2];
 #pragma unroll
-      for (int i = 0; i < 128; ++i) sum[i] = 0.0f;
+      for (int i = 0; i < NT / 2; ++i) sum[i] = 0.0f;
       for (int ch = 0; ch < nchunks; ++ch) {
         const bool ok =
-            mbar_wait(bar_tfull + 8 * ab, abphase, limit_ns, abort_flag, timeout_global);
+            mbar_wait(bar_tfull + 8 * ab.idx, ab.phase, limit_ns, abort_flag, timeout_global);
         if (!epi_all(ok && !*abort_flag)) {
           alive = false;
           break;
         }
         fence_after();
-        const uint32_t ta = tmem_base + tlane + (uint32_t)(ab * BN + half * 128);
+        const uint32_t ta = tmem_base + tlane + (uint32_t)(ab.idx * NT + half * (NT / 2));
         const int pc = chunk_pass(ch, cpp, passes, crev);
         const float u = pc < 2 ? u01 : cross_unscale(st, job, pc, k1);
 #pragma unroll
-        for (int cc = 0; cc < 8; ++cc) {
+        for (int cc = 0; cc < NT / 32; ++cc) {
           uint32_t x[16];
           tmem_ld16(ta + 16 * cc, x);
 #pragma unroll
@@ -1369,17 +1442,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         if (ch + 1 == nchunks) break;   // keep the last chunk's buffer
         fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab);
-        if (++ab == 2) {
-          ab = 0;
-          abphase ^= 1;
-        }
+        if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab.idx);
+        ab.next(PT::ACC);
       }
       if (!alive) break;
       // the tile's sums go back into its last chunk's buffer
-      const uint32_t ta_sum = tmem_base + tlane + (uint32_t)(ab * BN + half * 128);
+      const uint32_t ta_sum = tmem_base + tlane + (uint32_t)(ab.idx * NT + half * (NT / 2));
 #pragma unroll
-      for (int cc = 0; cc < 8; ++cc) tmem_st16(ta_sum + 16 * cc, sum + 16 * cc);
+      for (int cc = 0; cc < NT / 32; ++cc) tmem_st16(ta_sum + 16 * cc, sum + 16 * cc);
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 
       const int64_t t = it % tiles;
@@ -1391,7 +1461,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       const float sg = (float)sigma, om = 1.0f - (float)sigma;
       const bool write = job != 0 || write0;
       const int r = I2 * 2 * BM + (int)rank * BM + rloc;
-      const int c0 = J * BN + half * 128;
+      const int c0 = J * BN + (int)(v % SP) * NT + half * (NT / 2);
       const float* Sold = master + (size_t)(curj * (1 + k) + job) * mat;
       float* Snew = master + (size_t)((curj ^ 1) * (1 + k) + job) * mat;
       const int zh_new = job == 0 ? z0n : zslice(curj ^ 1, job, 0, k);
@@ -1402,15 +1472,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       auto release = [&]() {   // the accumulator goes back to the MMA
         fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab);
+        if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab.idx);
       };
-      rolled_tile_epilogue<CV, 8>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
+      rolled_tile_epilogue<CV, NT / 32>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
                                    scale_new, write, ts, release);
-      if (++ab == 2) {
-        ab = 0;
-        abphase ^= 1;
-      }
-      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, partials + ((size_t)job * ptiles + 2 * t + rank) * kNQ);
+      ab.next(PT::ACC);
+      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, partials + ((size_t)job * ptiles + 2 * (SP * t + v % SP) + rank) * kNQ);
     }
   }
 
@@ -1421,7 +1488,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   fence_after();
   if (warp == 1) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
-                 "r"(TMEM_COLS));
+                 "r"(PT::COLS));
   }
 }
 
@@ -1624,16 +1691,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 
   if (warp == 0) {
     // ================= TMA producer (both CTAs load their own halves) ======
-    if (lane == 0) {
+    {
       RingPos rg;
       bool ok = true;
       int last_inst = -1;
       for (int64_t j = 0; ok; ++j) {
-        uint32_t g;
-        if (leader)
-          g = claim_next(gq, pair, j, epoch, items);
-        else if (!claim_wait(gq, pair, j, epoch, limit_ns, abort_flag, timeout_global, &g))
-          break;
+        uint32_t g = kNoItem;
+        if (lane == 0) {   // kNoItem as well when the wait fails
+          if (leader)
+            g = claim_next(gq, pair, j, epoch, items);
+          else if (!claim_wait(gq, pair, j, epoch, limit_ns, abort_flag, timeout_global, &g))
+            g = kNoItem;
+        }
+        g = __shfl_sync(0xffffffffu, g, 0);
         if (g == kNoItem) break;
         const GroupItem itm = group_item(inst, first, jmask, count, g, k_snake, chunk);
         const GroupInst& gi = inst[itm.inst];
@@ -1644,31 +1714,36 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         const State* sti = gi.st;
         int I2, J;
         pair_tile_banded(itm.t, (int)(gi.Np / BN), band, &I2, &J);
-        ok = produce_item(rg, &gi.map, sti, itm.job, itm.passes, gi.k, gi.k, sti->cur0,
+        ok = produce_item<BN>(rg, &gi.map, &gi.map, sti, itm.job, itm.passes, gi.k, gi.k, sti->cur0,
                           sti->z0_cur, I2 * 2 * BM + (int)rank * BM, J * BN + (int)rank * BM,
                           itm.kblocks, itm.rev, leader, ring, bar_full, bar_empty, lead_full,
                           limit_ns, abort_flag, timeout_global);
       }
-      producer_drain(rg, bar_empty, limit_ns);
+      if (lane == 0) producer_drain(rg, P_STAGES, bar_empty, limit_ns);
     }
   } else if (warp == 1) {
     // ================= MMA issuer (leader CTA only) =================
-    if (leader && lane == 0) {
+    if (leader) {
       RingPos rg, tb;
       bool ok = true;
       for (int64_t j = 0; ok; ++j) {
-        uint32_t g;
-        if (!claim_wait(gq, pair, j, epoch, limit_ns, abort_flag, timeout_global, &g)) break;
+        uint32_t g = kNoItem;
+        if (lane == 0 &&
+            !claim_wait(gq, pair, j, epoch, limit_ns, abort_flag, timeout_global, &g))
+          g = kNoItem;
+        g = __shfl_sync(0xffffffffu, g, 0);
         if (g == kNoItem) break;
         const GroupItem itm = group_item(inst, first, jmask, count, g, k_snake, chunk);
-        ok = mma_item<BF16>(rg, tb, itm.passes * itm.kblocks, itm.kblocks, chunk, itm.cp0,
+        ok = mma_item<BF16, BN>(rg, tb, itm.passes * itm.kblocks, itm.kblocks, chunk, itm.cp0,
                             tmem_base, ring, bar_full, bar_empty, bar_tfull, bar_tempty, limit_ns,
                             abort_flag, timeout_global);
       }
-      asm volatile(
-          "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-              bar_drain)
-          : "memory");
+      if (elect_one())
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                bar_drain)
+            : "memory");
+      __syncwarp();
       const uint64_t t0 = gtimer();
       while (!mbar_try_wait(bar_drain, 0) && gtimer() - t0 < limit_ns) {
       }
@@ -1808,19 +1883,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 // tile order differs from the 256 x 256 kernels, so results agree with them
 // to rounding, not bit for bit.
 constexpr int G_BN = 128;                                   // tile columns
-constexpr int G_BROWS = G_BN / 2;                           // B rows per CTA
-constexpr int G_B_BYTES = G_BROWS * BK * 2;                 // 4 KB
-constexpr int G_STAGES = 8;
-constexpr int G_STAGE_BYTES = 2 * A_BYTES + 2 * G_B_BYTES;  // 24 KB
-constexpr int G_ACC = 4;                                    // accumulators of G_BN columns
-static_assert(G_ACC * G_BN == TMEM_COLS, "accumulators fill the allocation");
-constexpr int G_SMEM_BYTES = G_STAGES * G_STAGE_BYTES + 1024 + 1024 + EPI_SCRATCH;
-static_assert(G_SMEM_BYTES == P_SMEM_BYTES, "same shared memory as the 256 x 256 kernel");
-
-__host__ __device__ constexpr uint32_t make_idesc_m256_n128(int ab_type) {
-  return (1u << 4) | ((uint32_t)ab_type << 7) | ((uint32_t)ab_type << 10) |
-         ((uint32_t)(G_BN >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
-}
+using GT = PairTile<G_BN>;
+static_assert(GT::COLS == TMEM_COLS, "accumulators fill the allocation");
 
 // 256 x 128 tiles holding some element with row <= col: 256-row block I2 and
 // 128-column block J' with J' >= 2 I2; row-major (I2, then J').
@@ -1859,98 +1923,6 @@ __device__ __forceinline__ GroupItem128 group_item128(const GroupInst* __restric
   return r;
 }
 
-// Producer of one 256 x 128 item: this CTA's 128 A rows (128-row map) and its
-// 64 B rows (64-row map) per stage, signalled on the leader's full barrier.
-__device__ __forceinline__ bool produce_item128(RingPos& rg, const CUtensorMap* map,
-                                                const CUtensorMap* map64, const State* st,
-                                                int job, int passes, int k, int cur0, int z0c,
-                                                int rowA, int rowB, int kblocks, bool leader,
-                                                uint32_t ring, uint32_t bar_full,
-                                                uint32_t bar_empty, uint32_t lead_full,
-                                                uint64_t limit_ns, volatile int* abort_flag,
-                                                int* timeout_global) {
-  for (int pass = 0; pass < passes; ++pass) {
-    int mA, mB;
-    job_operands(job, pass, k, &mA, &mB);
-    const int bufA = mA == 0 ? cur0 : st->cur1[mA - 1];
-    const int bufB = mB == 0 ? cur0 : st->cur1[mB - 1];
-    const int zAh = zop(mA, bufA, 0, k, z0c), zAl = zop(mA, bufA, 1, k, z0c);
-    const int zBh = zop(mB, bufB, 0, k, z0c), zBl = zop(mB, bufB, 1, k, z0c);
-    for (int kb = 0; kb < kblocks; ++kb) {
-      if (!mbar_wait(bar_empty + 8 * rg.idx, rg.phase ^ 1, limit_ns, abort_flag, timeout_global))
-        return false;
-      const uint32_t sA = ring + rg.idx * G_STAGE_BYTES;
-      if (leader) mbar_expect_tx(bar_full + 8 * rg.idx, 2 * G_STAGE_BYTES);
-      const uint32_t fb = lead_full + 8 * rg.idx;
-      tma_load_3d_pair(sA, map, kb * BK, rowA, zAh, fb);
-      tma_load_3d_pair(sA + A_BYTES, map, kb * BK, rowA, zAl, fb);
-      tma_load_3d_pair(sA + 2 * A_BYTES, map64, kb * BK, rowB, zBh, fb);
-      tma_load_3d_pair(sA + 2 * A_BYTES + G_B_BYTES, map64, kb * BK, rowB, zBl, fb);
-      rg.next(G_STAGES);
-    }
-  }
-  return true;
-}
-
-__device__ __forceinline__ void producer_drain128(RingPos rg, uint32_t bar_empty,
-                                                  uint64_t limit_ns) {
-  for (int i = 0; i < G_STAGES; ++i) {
-    const uint64_t t0 = gtimer();
-    while (!mbar_try_wait(bar_empty + 8 * rg.idx, rg.phase ^ 1) && gtimer() - t0 < limit_ns) {
-    }
-    rg.next(G_STAGES);
-  }
-}
-
-// MMA issuer of one 256 x 128 item (leader CTA, one thread): as mma_item,
-// with N = 128 and four accumulators.
-template <bool BF16>
-__device__ __forceinline__ bool mma_item128(RingPos& rg, RingPos& tb, int nst, int kblocks,
-                                            int chunk, uint32_t tmem_base, uint32_t ring,
-                                            uint32_t bar_full, uint32_t bar_empty,
-                                            uint32_t bar_tfull, uint32_t bar_tempty,
-                                            uint64_t limit_ns, volatile int* abort_flag,
-                                            int* timeout_global) {
-  constexpr uint32_t idesc = make_idesc_m256_n128(BF16 ? 1 : 0);
-  uint32_t d = 0, acc = 0;
-  int sp = 0;   // stage within its K pass
-  int cp = 0;   // stage within its accumulation chunk
-  for (int si = 0; si < nst; ++si) {
-    if (cp == 0) {
-      if (!mbar_wait(bar_tempty + 8 * tb.idx, tb.phase ^ 1, limit_ns, abort_flag, timeout_global))
-        return false;
-      fence_after();
-      d = tmem_base + (uint32_t)(tb.idx * G_BN);
-      acc = 0;
-    }
-    if (!mbar_wait(bar_full + 8 * rg.idx, rg.phase, limit_ns, abort_flag, timeout_global))
-      return false;
-    fence_after();
-    const uint32_t sA = ring + rg.idx * G_STAGE_BYTES;
-    const uint64_t ah = sw64_desc(sA), al = sw64_desc(sA + A_BYTES);
-    const uint64_t bh = sw64_desc(sA + 2 * A_BYTES);
-    const uint64_t bl = sw64_desc(sA + 2 * A_BYTES + G_B_BYTES);
-#pragma unroll
-    for (int kk = 0; kk < BK / 16; ++kk) {
-      const uint64_t off = (uint64_t)((kk * 32) >> 4);
-      mma_f16_pair(d, ah + off, bh + off, idesc, acc);   // hi * hi
-      acc = 1;
-      mma_f16_pair(d, ah + off, bl + off, idesc, 1);     // hi * lo
-      mma_f16_pair(d, al + off, bh + off, idesc, 1);     // lo * hi
-    }
-    mma_commit_pair(bar_empty + 8 * rg.idx);   // frees the stage in both CTAs
-    rg.next(G_STAGES);
-    const bool chunk_end = cp == chunk - 1 || sp == kblocks - 1;
-    if (++cp == chunk || sp == kblocks - 1) cp = 0;
-    if (++sp == kblocks) sp = 0;
-    if (chunk_end) {
-      mma_commit_pair(bar_tfull + 8 * tb.idx);    // chunk ready in both CTAs
-      tb.next(G_ACC);
-    }
-  }
-  return true;
-}
-
 template <bool BF16>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     layer_tc2_group128_kernel(const GroupInst* __restrict__ inst, int count, int* group_timeout,
@@ -1963,7 +1935,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
   const uint32_t ring = base;
-  uint8_t* misc = gbase + G_STAGES * G_STAGE_BYTES;
+  uint8_t* misc = gbase + GT::STAGES * GT::STAGE;
   int64_t* first = reinterpret_cast<int64_t*>(misc + 1024 + EPI_SCRATCH);
   uint32_t* jmask = reinterpret_cast<uint32_t*>(first + count + 1);
 
@@ -1995,11 +1967,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);
   const uint32_t bar_full = smem_u32(bars);
-  const uint32_t bar_empty = bar_full + 8 * G_STAGES;
-  const uint32_t bar_tfull = bar_empty + 8 * G_STAGES;
-  const uint32_t bar_tempty = bar_tfull + 8 * G_ACC;
-  const uint32_t bar_drain = bar_tempty + 8 * G_ACC;
-  static_assert(8 * (2 * G_STAGES + 2 * G_ACC + 1) <= 256, "barriers below the TMEM slot");
+  const uint32_t bar_empty = bar_full + 8 * GT::STAGES;
+  const uint32_t bar_tfull = bar_empty + 8 * GT::STAGES;
+  const uint32_t bar_tempty = bar_tfull + 8 * GT::ACC;
+  const uint32_t bar_drain = bar_tempty + 8 * GT::ACC;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 264);
   float* red = reinterpret_cast<float*>(misc + 1024);
@@ -2010,11 +1981,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < G_STAGES; ++s) {
+    for (int s = 0; s < GT::STAGES; ++s) {
       mbar_init(bar_full + 8 * s, 1);
       mbar_init(bar_empty + 8 * s, 1);
     }
-    for (int b = 0; b < G_ACC; ++b) {
+    for (int b = 0; b < GT::ACC; ++b) {
       mbar_init(bar_tfull + 8 * b, 1);
       mbar_init(bar_tempty + 8 * b, 2 * EPI_WARPS);
     }
@@ -2036,16 +2007,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 
   if (warp == 0) {
     // ================= TMA producer (both CTAs load their own rows) ======
-    if (lane == 0) {
+    {
       RingPos rg;
       bool ok = true;
       int last_inst = -1;
       for (int64_t j = 0; ok; ++j) {
-        uint32_t g;
-        if (leader)
-          g = claim_next(gq, pair, j, epoch, items);
-        else if (!claim_wait(gq, pair, j, epoch, limit_ns, abort_flag, timeout_global, &g))
-          break;
+        uint32_t g = kNoItem;
+        if (lane == 0) {   // kNoItem as well when the wait fails
+          if (leader)
+            g = claim_next(gq, pair, j, epoch, items);
+          else if (!claim_wait(gq, pair, j, epoch, limit_ns, abort_flag, timeout_global, &g))
+            g = kNoItem;
+        }
+        g = __shfl_sync(0xffffffffu, g, 0);
         if (g == kNoItem) break;
         const GroupItem128 itm = group_item128(inst, first, jmask, count, g);
         const GroupInst& gi = inst[itm.inst];
@@ -2057,31 +2031,37 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         const State* sti = gi.st;
         int I2, J;
         tile128_coords(itm.t, gi.Np, &I2, &J);
-        ok = produce_item128(rg, &gi.map, &gi.map64, sti, itm.job, itm.passes, gi.k, sti->cur0,
-                             sti->z0_cur, I2 * 2 * BM + (int)rank * BM,
-                             J * G_BN + (int)rank * G_BROWS, itm.kblocks, leader, ring, bar_full,
-                             bar_empty, lead_full, limit_ns, abort_flag, timeout_global);
+        ok = produce_item<G_BN>(rg, &gi.map, &gi.map64, sti, itm.job, itm.passes, gi.k, gi.k,
+                                sti->cur0, sti->z0_cur, I2 * 2 * BM + (int)rank * BM,
+                                J * G_BN + (int)rank * GT::B_ROWS, itm.kblocks, false, leader,
+                                ring, bar_full, bar_empty, lead_full, limit_ns, abort_flag,
+                                timeout_global);
       }
-      producer_drain128(rg, bar_empty, limit_ns);
+      if (lane == 0) producer_drain(rg, GT::STAGES, bar_empty, limit_ns);
     }
   } else if (warp == 1) {
     // ================= MMA issuer (leader CTA only) =================
-    if (leader && lane == 0) {
+    if (leader) {
       RingPos rg, tb;
       bool ok = true;
       for (int64_t j = 0; ok; ++j) {
-        uint32_t g;
-        if (!claim_wait(gq, pair, j, epoch, limit_ns, abort_flag, timeout_global, &g)) break;
+        uint32_t g = kNoItem;
+        if (lane == 0 &&
+            !claim_wait(gq, pair, j, epoch, limit_ns, abort_flag, timeout_global, &g))
+          g = kNoItem;
+        g = __shfl_sync(0xffffffffu, g, 0);
         if (g == kNoItem) break;
         const GroupItem128 itm = group_item128(inst, first, jmask, count, g);
-        ok = mma_item128<BF16>(rg, tb, itm.passes * itm.kblocks, itm.kblocks, chunk, tmem_base,
-                               ring, bar_full, bar_empty, bar_tfull, bar_tempty, limit_ns,
-                               abort_flag, timeout_global);
+        ok = mma_item<BF16, G_BN>(rg, tb, itm.passes * itm.kblocks, itm.kblocks, chunk, 0,
+                                  tmem_base, ring, bar_full, bar_empty, bar_tfull, bar_tempty,
+                                  limit_ns, abort_flag, timeout_global);
       }
-      asm volatile(
-          "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-              bar_drain)
-          : "memory");
+      if (elect_one())
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                bar_drain)
+            : "memory");
+      __syncwarp();
       const uint64_t t0 = gtimer();
       while (!mbar_try_wait(bar_drain, 0) && gtimer() - t0 < limit_ns) {
       }
@@ -2140,7 +2120,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab.idx);
-        ab.next(G_ACC);
+        ab.next(GT::ACC);
       }
       if (!alive) break;
       // the tile's sums go back into its last chunk's accumulator (rolled epilogue)
@@ -2183,7 +2163,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
                                      scale_new, write, ts, release);
       else
         release();
-      ab.next(G_ACC);
+      ab.next(GT::ACC);
       tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, gi.partials + ((size_t)job * gi.ptiles + 2 * itm.t + rank) * kNQ);
     }
   }
@@ -2202,6 +2182,38 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 
 // ---------------------------------------------------------------------------
 // Host side
+
+using PairKernel = decltype(&layer_tc2_kernel<false, BN>);
+PairKernel pair_kernel(bool bf16, int nt) {
+  if (nt == 64) return bf16 ? layer_tc2_kernel<true, 64> : layer_tc2_kernel<false, 64>;
+  if (nt == 128) return bf16 ? layer_tc2_kernel<true, 128> : layer_tc2_kernel<false, 128>;
+  return bf16 ? layer_tc2_kernel<true, BN> : layer_tc2_kernel<false, BN>;
+}
+
+// Tile width of the pair kernel for `tiles` 256 x 256 tiles of 1 + k jobs.
+// Measured time per layer in us of a whole solve, 256 / 128 / 64 wide:
+//   n = 128 k = 1   29 /  22 /  20       n = 2048 k = 1   84 /  74 / 106
+//   n = 768 k = 1   45 /  31 /  29       n = 2048 k = 3  155 / 150 / 224
+//   n = 768 k = 3   46 /  33 /  37       n = 2560 k = 3  270 / 285 / 397
+//   n = 1280 k = 3  64 /  66 /  86       n = 3072 k = 1  256 / 228 / 314
+// 64: while one round of the pairs holds every tile; the tile's own time (its
+// epilogue above all) is then what counts.  Above, the busiest pair's load
+// decides: a 128-wide tile takes 0.6 of the time of a 256-wide one per K block
+// (it loads 24 KB per 32-wide block for half the products, and its MMAs issue
+// no faster than 0.24 us per block against 0.4), and its last epilogue is
+// about 14 blocks shorter.  The pairs take the items round-robin, responses
+// (two K passes) first, so pair 0 has the largest load.
+int pair_tile_width(int64_t tiles, int k, int64_t kblocks, int pairs) {
+  const int64_t items = tiles * (1 + k);
+  if (BN / 64 * items <= pairs) return 64;
+  if (items > 8 * pairs) return BN;
+  auto load = [&](int split) {
+    int64_t passes = 0;
+    for (int64_t i = 0; i < split * items; i += pairs) passes += i < split * tiles * k ? 2 : 1;
+    return passes * kblocks;
+  };
+  return 3 * load(2) < 5 * (load(1) + 14) ? 128 : BN;
+}
 
 // Per-device one-time setup of the tensor-core kernels (their shared-memory
 // attribute is set in each device's context) and the device's SM count;
@@ -2222,10 +2234,10 @@ int device_setup() {
                          SMEM_BYTES);
     cudaFuncSetAttribute(layer_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          SMEM_BYTES);
-    cudaFuncSetAttribute(layer_tc2_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         P_SMEM_BYTES);
-    cudaFuncSetAttribute(layer_tc2_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         P_SMEM_BYTES);
+    for (bool bf16 : {false, true})
+      for (int nt : {256, 128, 64})
+        cudaFuncSetAttribute(pair_kernel(bf16, nt), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             P_SMEM_BYTES);
     constexpr int group_smem = P_SMEM_BYTES + (kGroupMax + 1) * (int)sizeof(int64_t) +
                                kGroupMax * (int)sizeof(uint32_t);
     static_assert(group_smem <= 227 * 1024, "grouped kernel shared memory");
@@ -2286,7 +2298,7 @@ bool make_group_inst(const Layout& L, void* ws, int sm_count, GroupInst* gi, boo
   const bool bf16 = L.precision == DMPT_DUAL_BF16;
   const int slices = 2 * (1 + L.k) * 2 + 2 * L.tape_states;
   if (!make_map(&gi->map, base + L.off_ops16, L.Np, slices, BM, bf16)) return false;
-  if (n128 && !make_map(&gi->map64, base + L.off_ops16, L.Np, slices, G_BROWS, bf16)) return false;
+  if (n128 && !make_map(&gi->map64, base + L.off_ops16, L.Np, slices, GT::B_ROWS, bf16)) return false;
   gi->st = (State*)(base + L.off_state);
   gi->master = (float*)(base + L.off_master);
   gi->ops = (uint16_t*)(base + L.off_ops16);
@@ -2343,11 +2355,14 @@ cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double ti
   const bool bf16 = L.precision == DMPT_DUAL_BF16;
   const int slices = 2 * (1 + L.k) * 2 + 2 * L.tape_states;
   CUtensorMap mA, mB;
-  if (!make_map(&mA, base + L.off_ops16, L.Np, slices, BM, bf16) ||
-      !make_map(&mB, base + L.off_ops16, L.Np, slices, BN, bf16))
-    return cudaErrorInvalidValue;
   const int sms = device_setup();
   if (sms == 0) return cudaErrorInvalidDevice;
+  // 256 x 256 tiles of every job (the jobs that run are only known on the device)
+  const int64_t ptiles = num_pair_tiles(L.Np), pitems = ptiles * (1 + L.k);
+  const int nt = pair_tile_width(ptiles, L.k, k_blocks(L.n), sms / 2);
+  if (!make_map(&mA, base + L.off_ops16, L.Np, slices, BM, bf16) ||
+      !make_map(&mB, base + L.off_ops16, L.Np, slices, cta_pair ? nt / 2 : BN, bf16))
+    return cudaErrorInvalidValue;
   const uint64_t limit_ns = (uint64_t)(timeout_s * 1e9);
   int ck = accum_chunk_k > 0 ? accum_chunk_k : DEFAULT_CHUNK_K;
   int chunk = ck / BK;
@@ -2357,17 +2372,15 @@ cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double ti
   uint16_t* ops = (uint16_t*)(base + L.off_ops16);
   double* partials = (double*)(base + L.off_partials);
   if (cta_pair) {
-    const int64_t tiles = num_pair_tiles(L.Np);
-    const int64_t max_items = tiles * (1 + L.k);
-    int64_t pairs = sms / 2;
-    if (pairs > max_items) pairs = max_items;
-    const int grid = (int)(2 * pairs);
-    auto kern = bf16 ? layer_tc2_kernel<true> : layer_tc2_kernel<false>;
-    kern<<<grid, NUM_THREADS, P_SMEM_BYTES, s>>>(
-        mA, st, master, ops, L.Np, L.k, partials, L.partial_tiles, limit_ns, chunk, k_snake, band,
-        inject_stall, round_align);
-    if (entries) *entries = 2 * tiles;
-    if (pass_flops) *pass_flops = (double)tiles * 2 * BM * BN * k_blocks(L.n) * BK * 2.0;
+    const int split = BN / nt;
+    const int64_t max_items = split * pitems;
+    const int pairs = (int)(max_items < sms / 2 ? max_items : sms / 2);
+    const int snake_pairs = (int)(pitems < sms / 2 ? pitems : sms / 2);
+    pair_kernel(bf16, nt)<<<2 * pairs, NUM_THREADS, P_SMEM_BYTES, s>>>(
+        mA, mB, st, master, ops, L.Np, L.k, partials, L.partial_tiles, limit_ns, chunk, k_snake,
+        snake_pairs, band, inject_stall, round_align);
+    if (entries) *entries = 2 * split * ptiles;
+    if (pass_flops) *pass_flops = (double)ptiles * 2 * BM * BN * k_blocks(L.n) * BK * 2.0;
     return cudaGetLastError();
   }
   const int64_t tiles = num_tiles(L.Np);
