@@ -10,6 +10,7 @@
 
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "dmpt.h"
@@ -89,6 +90,42 @@ struct State {
   double froerr1[kMaxK][kMaxL + 2];
   signed char sigma[kMaxL + 2];
 };
+
+// The control block's head (every field before the per-layer histories), in
+// 32-bit words.
+constexpr int kHeadWords = (int)(offsetof(State, iderr) / sizeof(unsigned));
+static_assert(offsetof(State, iderr) % sizeof(unsigned) == 0, "whole words");
+
+// Programmatic dependent launch.  The kernels of the layer loop are launched
+// with launch_pdl: a kernel may start while the one before it in the stream is
+// still running, sets itself up (barriers, tensor memory, tensor maps) and
+// waits in pdl_wait() until that kernel has completed and its writes are
+// visible; every thread calls it before its first access to device memory,
+// and reads what earlier kernels wrote past L1 or through plain loads only
+// (never ld.global.nc).  pdl_launch() lets the next kernel of the stream
+// start once every block has called it or ended.  The layer products call it
+// after pdl_wait(), so at most one layer and one decide step are ever waiting.
+// A solve of n = 128 took 38.7 instead of 44.2 us per layer with it, one of
+// n = 1000, k = 2 62.1 instead of 67.1 (256 x 256 tiles).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
 
 // Product options of a forward run, kept in its control block so that the
 // backward pass recomputes checkpointed states with the same launches.

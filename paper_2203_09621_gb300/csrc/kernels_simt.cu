@@ -406,9 +406,7 @@ __device__ int fp16_exponent_for(double bound) {
 // j.  Measured per step, n = 128 k = 1 / n = 2048 k = 3: 16.5 / 23.5 us
 // before, 5.8 / 7.0 us now (an empty launch takes 2 us).
 constexpr int kDecideThreads = 1024;
-constexpr int kHeadWords = (int)(offsetof(State, iderr) / sizeof(unsigned));
-static_assert(offsetof(State, iderr) % sizeof(unsigned) == 0 && kHeadWords <= kDecideThreads,
-              "one head word per thread");
+static_assert(kHeadWords <= kDecideThreads, "one head word per thread");
 
 struct DecideShared {
   alignas(16) unsigned head[kHeadWords + (kHeadWords & 1)];
@@ -687,10 +685,10 @@ __device__ void decide_layer(State* S, State* G, const DecideShared& sh, int lan
 
 // The decide step of one instance, run by one block of kDecideThreads
 // threads.  jobs: 1 + the response slots of the partials array.
-__device__ void decide_body(State* st, const double* __restrict__ partials, int64_t ptiles,
+__device__ void decide_body(State* st, const double* partials, int64_t ptiles,
                             int64_t entries, int jobs, int mode, DecideShared& sh) {
   const int tid = threadIdx.x, lane = tid & 31;
-  if (tid < kHeadWords) sh.head[tid] = reinterpret_cast<const unsigned*>(st)[tid];
+  if (tid < kHeadWords) sh.head[tid] = __ldcg(reinterpret_cast<const unsigned*>(st) + tid);
   if (tid >= kDecideThreads - 32) {
     // the history entries the tests read, fetched while the sums are formed
     const bool adj = mode == kDecideAdjInit || mode == kDecideAdjLayer || mode == kDecideAdjResume;
@@ -718,7 +716,7 @@ __device__ void decide_body(State* st, const double* __restrict__ partials, int6
       for (int64_t e = t; e < entries; e += 256) {
         const double2* p =
             reinterpret_cast<const double2*>(partials + ((size_t)job * ptiles + e) * kNQ);
-        const double2 a = p[0], b = p[1];
+        const double2 a = __ldcg(p), b = __ldcg(p + 1);
         v[0] += a.x;
         v[1] += a.y;
         v[2] += b.x;
@@ -763,9 +761,11 @@ __device__ void decide_body(State* st, const double* __restrict__ partials, int6
 }
 
 __global__ void __launch_bounds__(kDecideThreads)
-    decide_kernel(State* st, const double* __restrict__ partials, int64_t ptiles, int64_t entries,
+    decide_kernel(State* st, const double* partials, int64_t ptiles, int64_t entries,
                   int jobs, int mode) {
   __shared__ DecideShared sh;
+  pdl_launch();
+  pdl_wait();
   decide_body(st, partials, ptiles, entries, jobs, mode, sh);
 }
 
@@ -810,10 +810,9 @@ static void decide_setup() {
 cudaError_t launch_decide(const Layout& L, void* ws, int mode, int64_t entries, cudaStream_t s) {
   char* base = (char*)ws;
   decide_setup();
-  decide_kernel<<<1, kDecideThreads, 0, s>>>((State*)(base + L.off_state),
-                                             (const double*)(base + L.off_partials),
-                                             L.partial_tiles, entries, 1 + L.k, mode);
-  return cudaGetLastError();
+  return launch_pdl(decide_kernel, dim3(1), dim3(kDecideThreads), 0, s,
+                    (State*)(base + L.off_state), (const double*)(base + L.off_partials),
+                    L.partial_tiles, entries, 1 + L.k, mode);
 }
 
 // ---------------------------------------------------------------------------
@@ -928,6 +927,7 @@ __global__ void __launch_bounds__(256, SimtBlocks<T>::value)
   T* slabs = reinterpret_cast<T*>(simt_smem);
   double* red = reinterpret_cast<double*>(simt_smem + SIMT_STAGES * 2 * BK * LD * sizeof(T));
 
+  pdl_wait();   // no pdl_launch(): see layer_fp64_kernel
   if (st->done) return;
   const int job = blockIdx.y;
   const int run = job == 0 ? st->plan_square : st->plan_resp[job - 1];
@@ -1120,7 +1120,7 @@ __device__ __forceinline__ void cp_async16_zfill(void* smem, const void* gmem, b
 
 template <int T>
 __global__ void __launch_bounds__(128)
-    layer_fp64_kernel(const State* __restrict__ st, double* __restrict__ master, int64_t n,
+    layer_fp64_kernel(const State* st, double* master, int64_t n,
                       int64_t Np, int k, double* __restrict__ partials, int64_t ptiles) {
   constexpr int BK = 16, STAGES = 3, NT = 128;
   constexpr int LD = T + 2;                 // padded slab row (16-byte chunks)
@@ -1134,6 +1134,11 @@ __global__ void __launch_bounds__(128)
   __shared__ double red[2][NT];
   __shared__ double red_tr[32];
 
+  // The next kernel starts when this one's blocks have all ended (no
+  // pdl_launch() here): blocks of the next layer that come in while this one's
+  // last blocks run would fill the SMs that ended first and leave the layer
+  // unbalanced (FP64 form, n = 700: 39.1 ms against 37.2).
+  pdl_wait();
   if (st->done) return;
   const int job = (int)gridDim.y - 1 - (int)blockIdx.y;
   const bool run = job == 0 ? st->plan_square != 0 : st->plan_resp[job - 1] != 0;
@@ -1344,23 +1349,22 @@ cudaError_t launch_layer_simt(const Layout& L, void* ws, cudaStream_t s, int64_t
     const int bt = fp64_tile(L.n);
     tiles = fp64_tiles(L.n);
     const dim3 grid((unsigned)tiles, 1 + L.k);
-    if (bt == 8)
-      layer_fp64_kernel<8><<<grid, 128, 0, s>>>(st, master, L.n, L.Np, L.k, partials,
-                                                L.partial_tiles);
-    else if (bt == 16)
-      layer_fp64_kernel<16><<<grid, 128, 0, s>>>(st, master, L.n, L.Np, L.k, partials,
-                                                 L.partial_tiles);
-    else
-      layer_fp64_kernel<32><<<grid, 128, 0, s>>>(st, master, L.n, L.Np, L.k, partials,
-                                                 L.partial_tiles);
+    const auto kern = bt == 8 ? layer_fp64_kernel<8>
+                              : (bt == 16 ? layer_fp64_kernel<16> : layer_fp64_kernel<32>);
+    const cudaError_t e = launch_pdl(kern, grid, dim3(128), 0, s, st, master, L.n, L.Np, L.k,
+                                     partials, L.partial_tiles);
+    if (e != cudaSuccess) return e;
     if (pass_flops) *pass_flops = (double)tiles * bt * bt * (double)L.n * 2.0;
   } else {
     constexpr int smem32 = simt_smem_bytes<float, 8, 16>();
     static_assert(2 * smem32 <= 227 * 1024, "two FP32 blocks per SM");
     simt_setup();
     tiles = upper_tiles(L.Np, kFp32Tile);
-    layer_simt_kernel<float, 8, 16><<<dim3((unsigned)tiles, 1 + L.k), 256, smem32, s>>>(
-        st, (float*)(base + L.off_master), L.Np, L.k, partials, L.partial_tiles);
+    const cudaError_t e =
+        launch_pdl(layer_simt_kernel<float, 8, 16>, dim3((unsigned)tiles, 1 + L.k), dim3(256),
+                   smem32, s, st, (float*)(base + L.off_master), L.Np, L.k, partials,
+                   L.partial_tiles);
+    if (e != cudaSuccess) return e;
     if (pass_flops)
       *pass_flops = (double)tiles * kFp32Tile * kFp32Tile * (double)L.Np * 2.0;
   }

@@ -187,6 +187,10 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
+
 __device__ __forceinline__ void fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
@@ -509,7 +513,7 @@ __device__ __forceinline__ void rolled_tile_epilogue(
   float olds[16];   // S_old of the current 16 columns; the next 16 are loaded
                     // while the current ones are stored
 #pragma unroll
-  for (int q = 0; q < 16; ++q) olds[q] = __ldg(Sc + (16 * g16 + q) * np);
+  for (int q = 0; q < 16; ++q) olds[q] = __ldcg(Sc + (16 * g16 + q) * np);
 #pragma unroll 1
   for (; g16 < NG; ++g16) {
     uint32_t xs[16];
@@ -590,7 +594,7 @@ __device__ __forceinline__ void rolled_tile_epilogue(
     }
     if (g16 < NG - 1) {
 #pragma unroll
-      for (int q = 0; q < 16; ++q) olds[q] = __ldg(Sc + (16 * (g16 + 1) + q) * np);
+      for (int q = 0; q < 16; ++q) olds[q] = __ldcg(Sc + (16 * (g16 + 1) + q) * np);
     }
   }
   float a0, a1, b0, b1;
@@ -971,6 +975,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 //   tfull[b]  each CTA: leader's commit, multicast
 //   tempty[b] leader only: 16 arrivals (8 epilogue warps per CTA)
 
+static_assert(272 + 4 * kHeadWords <= 1024, "the control block's head below the partial sums");
+
 constexpr int P_STAGES = 6;
 constexpr int P_STAGE_BYTES = 2 * A_BYTES + 2 * A_BYTES;   // A hi/lo + B-half hi/lo: 32 KB
 constexpr int P_SMEM_BYTES = P_STAGES * P_STAGE_BYTES + 1024 + 1024 + EPI_SCRATCH;
@@ -1256,7 +1262,7 @@ __device__ __forceinline__ void round_start(unsigned* ctr, int64_t round, int64_
 template <bool BF16, int NT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     layer_tc2_kernel(const __grid_constant__ CUtensorMap mapA,
-                     const __grid_constant__ CUtensorMap mapB, State* st,
+                     const __grid_constant__ CUtensorMap mapB, State* gst,
                      float* __restrict__ master, uint16_t* __restrict__ ops, int64_t Np, int k,
                      double* __restrict__ partials, int64_t ptiles, uint64_t limit_ns, int chunk,
                      int k_snake, int snake_pairs, int band, int inject_stall, int round_align) {
@@ -1265,34 +1271,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   using CV = Cvt<BF16>;
   using H16 = typename CV::T;
   extern __shared__ uint8_t smem_raw[];
-  // every CTA takes the same early exits (state is read before any cluster
-  // barrier, and both CTAs of a pair see the same values)
-  if (st->done) return;
-  uint32_t jmask = st->plan_square ? 1u : 0u;
-  for (int j = 0; j < k; ++j)
-    if (st->plan_resp[j]) jmask |= 1u << (1 + j);
-  const int njobs = __popc(jmask);
-  if (njobs == 0) return;
-  const int cur0 = st->cur0;
-  const int sigma = st->sigma_cur;
-  const int write0 = st->plan_write0;
-  const int s0e = st->s0_exp;
-  const int z0c = st->z0_cur, z0n = st->z0_next;
-  const int k1 = st->order >= 2 ? st->k1 : k;   // first-order directions
-  // virtual index of the first item (0, except when the backward recomputes
-  // a square alone: it then numbers the square's items as the forward launch
-  // did, after its response items, so each tile keeps its round and K-snake
-  // direction and the recomputed states are bit-identical)
-  const int64_t vbase = SP * st->item_base;
-
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
-  const int64_t pair = blockIdx.x >> 1;
-  const int64_t npairs = gridDim.x >> 1;
-  const int64_t tiles = num_pair_tiles(Np);
-  const int64_t items = SP * tiles * njobs;
-  const int kblocks = k_blocks(st->n);
-
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
@@ -1332,11 +1312,50 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
                  "r"(PT::COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
+  if (warp == 0 && elect_one()) {
+    prefetch_tensormap(&mapA);
+    prefetch_tensormap(&mapB);
+  }
   fence_before();
   cluster_sync_all();   // barriers of both CTAs initialised, TMEM allocated
   fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  int* timeout_global = &st->timeout_flag;
+
+  // ---- everything above ran while the previous kernels of the stream finished
+  pdl_wait();
+  pdl_launch();
+  State* st = reinterpret_cast<State*>(misc + 272);   // the control block's head
+  for (int i = threadIdx.x; i < kHeadWords; i += NUM_THREADS)
+    reinterpret_cast<unsigned*>(st)[i] = __ldcg(reinterpret_cast<const unsigned*>(gst) + i);
+  __syncthreads();
+
+  // ---- plan of this layer (the same in every CTA)
+  uint32_t jmask = 0;
+  if (!st->done) {
+    jmask = st->plan_square ? 1u : 0u;
+    for (int j = 0; j < k; ++j)
+      if (st->plan_resp[j]) jmask |= 1u << (1 + j);
+  }
+  const int njobs = __popc(jmask);
+  const int cur0 = st->cur0;
+  const int sigma = st->sigma_cur;
+  const int write0 = st->plan_write0;
+  const int s0e = st->s0_exp;
+  const int z0c = st->z0_cur, z0n = st->z0_next;
+  const int k1 = st->order >= 2 ? st->k1 : k;   // first-order directions
+  // virtual index of the first item (0, except when the backward recomputes
+  // a square alone: it then numbers the square's items as the forward launch
+  // did, after its response items, so each tile keeps its round and K-snake
+  // direction and the recomputed states are bit-identical)
+  const int64_t vbase = SP * st->item_base;
+
+  const int64_t pair = blockIdx.x >> 1;
+  const int64_t npairs = gridDim.x >> 1;
+  const int64_t tiles = num_pair_tiles(Np);
+  const int64_t items = SP * tiles * njobs;
+  const int kblocks = k_blocks(st->n);
+
+  int* timeout_global = &gst->timeout_flag;
 
   // All pairs move through their tiles' K ranges in near lockstep; in odd
   // rounds of the 256 x 256 tiles the sweep runs backwards (passes and K
@@ -1346,7 +1365,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   // are the same bit for bit at every width.
   auto item_rev = [&](int64_t v) { return k_snake && ((v / SP / snake_pairs) & 1); };
 
-  if (warp == 0) {
+  if (njobs == 0) {
+    // nothing to do in this launch
+  } else if (warp == 0) {
     // ================= TMA producer (both CTAs load their own halves) ======
     {
       RingPos rg;
@@ -1356,7 +1377,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         if (v < vbase) continue;
         const int64_t it = (v - vbase) / SP;
         if (SP == 1 && v >= npairs) {
-          if (lane == 0) round_start(&st->round_ctr, v / npairs, items, npairs, align);
+          if (lane == 0) round_start(&gst->round_ctr, v / npairs, items, npairs, align);
           __syncwarp();
         }
         const int job = job_at(jmask, (int)(it / tiles));
@@ -2376,9 +2397,11 @@ cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double ti
     const int64_t max_items = split * pitems;
     const int pairs = (int)(max_items < sms / 2 ? max_items : sms / 2);
     const int snake_pairs = (int)(pitems < sms / 2 ? pitems : sms / 2);
-    pair_kernel(bf16, nt)<<<2 * pairs, NUM_THREADS, P_SMEM_BYTES, s>>>(
-        mA, mB, st, master, ops, L.Np, L.k, partials, L.partial_tiles, limit_ns, chunk, k_snake,
-        snake_pairs, band, inject_stall, round_align);
+    const cudaError_t e = launch_pdl(
+        pair_kernel(bf16, nt), dim3(2 * pairs), dim3(NUM_THREADS), P_SMEM_BYTES, s, mA, mB, st,
+        master, ops, L.Np, L.k, partials, L.partial_tiles, limit_ns, chunk, k_snake, snake_pairs,
+        band, inject_stall, round_align);
+    if (e != cudaSuccess) return e;
     if (entries) *entries = 2 * split * ptiles;
     if (pass_flops) *pass_flops = (double)ptiles * 2 * BM * BN * k_blocks(L.n) * BK * 2.0;
     return cudaGetLastError();
