@@ -81,8 +81,9 @@ typedef struct {
   double c_d0;          /* factor of the Alg. 2 test (default 4.5)            */
   int operand_scaling;  /* 1: exact power-of-two scaling of the 16-bit halves
                            (FP16 range); 0: none (default 1)                  */
-  int sync_every;       /* layers issued between host polls of the device
-                           state (default 4)                                  */
+  int sync_every;       /* batches: layers issued between host polls of the
+                           device state; single solves: most layers issued
+                           ahead of the device (at most 2) (default 4)        */
   int timing;           /* 1: time every layer-product launch with CUDA events
                            on `stream` and report it in dmpt_info             */
   double timeout_s;     /* limit of any device-side spin wait, in seconds,
@@ -223,9 +224,10 @@ dmpt_status dmpt_bounds(dmpt_handle h, const double* H, int64_t n, int64_t ld,
  *   P1     device, k blocks n x n (ld) outputs.
  *   info   host pointer, may be NULL.
  *   workspace / ws_bytes: caller scratch of dmpt_workspace_size() bytes.
- * The call issues all work on `stream` and synchronises that stream every
- * o->sync_every layers to read the convergence flag; it returns when the
- * outputs are written.  Returns DMPT_ENOTCONV (outputs = last iterate) when
+ * The call issues all work on `stream`, at most two layers ahead of the
+ * device (it follows the run through a word of mapped host memory that the
+ * handle owns), and synchronises that stream; it returns when the outputs are
+ * written.  Returns DMPT_ENOTCONV (outputs = last iterate) when
  * max_layers is reached, DMPT_ENUMERIC on non-finite values or
  * eps_N <= eps_1 for 0 < n_occ < n.  With o->ckpt_every = 1 the workspace
  * (sized by dmpt_workspace_size with the same options) also keeps every S0

@@ -224,8 +224,10 @@ cudaError_t launch_scc_potential(const double* gamma, int64_t n, int64_t ld, con
                                  double* v, int k, cudaStream_t s);
 cudaError_t launch_scc_mix(const double* P1, int64_t n, int64_t ld, double* q, int k,
                            double alpha, double* red, cudaStream_t s);
+// progress (device address of mapped host memory; may be NULL): the step
+// writes `code` there, with bit 0 set when the run has ended.
 cudaError_t launch_decide(const Layout& L, void* ws, int mode, int64_t entries,
-                          cudaStream_t s);
+                          cudaStream_t s, unsigned* progress = nullptr, unsigned code = 0);
 // Layer-product launchers.  *entries: partial-sum entries per job (tiles);
 // *pass_flops: flops of one single-term pass over all tiles and the K range.
 cudaError_t launch_layer_simt(const Layout& L, void* ws, cudaStream_t s, int64_t* entries,

@@ -762,11 +762,13 @@ __device__ void decide_body(State* st, const double* partials, int64_t ptiles,
 
 __global__ void __launch_bounds__(kDecideThreads)
     decide_kernel(State* st, const double* partials, int64_t ptiles, int64_t entries,
-                  int jobs, int mode) {
+                  int jobs, int mode, volatile unsigned* progress, unsigned code) {
   __shared__ DecideShared sh;
   pdl_launch();
   pdl_wait();
   decide_body(st, partials, ptiles, entries, jobs, mode, sh);
+  if (progress && threadIdx.x == 0)
+    *progress = code | (reinterpret_cast<const State*>(sh.head)->done ? 1u : 0u);
 }
 
 // Layer decide of every instance of a grouped launch, one block each.
@@ -807,12 +809,13 @@ static void decide_setup() {
   });
 }
 
-cudaError_t launch_decide(const Layout& L, void* ws, int mode, int64_t entries, cudaStream_t s) {
+cudaError_t launch_decide(const Layout& L, void* ws, int mode, int64_t entries, cudaStream_t s,
+                          unsigned* progress, unsigned code) {
   char* base = (char*)ws;
   decide_setup();
   return launch_pdl(decide_kernel, dim3(1), dim3(kDecideThreads), 0, s,
                     (State*)(base + L.off_state), (const double*)(base + L.off_partials),
-                    L.partial_tiles, entries, 1 + L.k, mode);
+                    L.partial_tiles, entries, 1 + L.k, mode, progress, code);
 }
 
 // ---------------------------------------------------------------------------
