@@ -210,6 +210,18 @@ __device__ __forceinline__ uint64_t sw64_desc(uint32_t addr) {
   return d;
 }
 
+// The same with 128-byte swizzle: rows of 128 B, 8-row groups 1024 B apart,
+// layout 2.
+__device__ __forceinline__ uint64_t sw128_desc(uint32_t addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;             // LBO (unused for swizzled K-major)
+  d |= (uint64_t)(1024 >> 4) << 32;   // SBO
+  d |= (uint64_t)1 << 46;             // descriptor version
+  d |= (uint64_t)2 << 61;             // SWIZZLE_128B
+  return d;
+}
+
 // Instruction descriptor, kind::f16: D = F32, A/B = F16 (0) or BF16 (1),
 // both K-major, N = 256, M = 128.
 __host__ __device__ constexpr uint32_t make_idesc(int ab_type) {
@@ -368,7 +380,7 @@ __device__ __forceinline__ float cross_unscale(const State* st, int job, int pas
 }
 // K range of the products: the 32-wide K blocks that hold columns < n.  The
 // blocks of the padding to Np hold zeros on both sides and are left out
-// (n = 5904: 185 of 192 blocks, layer 1288 -> KTRIM us).  The accumulation
+// (n = 5904: 185 of 192 blocks, solve 57.4 -> 54.4 ms).  The accumulation
 // chunks keep the boundaries they have over all Np / 32 blocks, so results do
 // not change: a backwards sweep starts `kchunk0` stages into its first chunk.
 __host__ __device__ __forceinline__ int k_blocks(int64_t n) { return (int)((n + BK - 1) / BK); }
@@ -977,26 +989,26 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 
 static_assert(272 + 4 * kHeadWords <= 1024, "the control block's head below the partial sums");
 
-constexpr int P_STAGES = 6;
-constexpr int P_STAGE_BYTES = 2 * A_BYTES + 2 * A_BYTES;   // A hi/lo + B-half hi/lo: 32 KB
-constexpr int P_SMEM_BYTES = P_STAGES * P_STAGE_BYTES + 1024 + 1024 + EPI_SCRATCH;
-
 // Geometry of the pair kernels' tiles, 256 rows x NT columns: each CTA loads
-// its 128 A rows and NT / 2 B rows per stage, and tensor memory holds ACC
-// accumulators of NT columns.
+// its 128 A rows and NT / 2 B rows, SK columns wide, per stage, and tensor
+// memory holds ACC accumulators of NT columns.  A stage is one 128-byte swizzle
+// span of K: with 64-byte rows and stages of 32 columns the 256 x 256 tiles
+// waited for operands (n = 8192 k = 3 solve 295.7 ms, now 290.7; n = 4096
+// k = 1 layer 432 -> 411 us).
 template <int NT>
 struct PairTile {
+  static constexpr int SK = 64;                                 // K elements per stage
   static constexpr int B_ROWS = NT / 2;
-  static constexpr int PB_BYTES = B_ROWS * BK * 2;
-  static constexpr int STAGE = 2 * A_BYTES + 2 * PB_BYTES;   // 32, 24, 20 KB
-  static constexpr int STAGES = P_STAGES * P_STAGE_BYTES / STAGE;
+  static constexpr int PA_BYTES = BM * SK * 2;
+  static constexpr int PB_BYTES = B_ROWS * SK * 2;
+  static constexpr int STAGE = 2 * PA_BYTES + 2 * PB_BYTES;     // 64, 48, 40 KB
+  static constexpr int STAGES = 200 * 1024 / STAGE;             // 3, 4, 5
   static constexpr int ACC = NT == 256 ? 2 : 4;
-  static constexpr int COLS = ACC * NT;                      // tensor-memory columns
-  static constexpr int SPLIT = BN / NT;                      // tiles per 256 x 256 tile
+  static constexpr int COLS = ACC * NT;                         // tensor-memory columns
+  static constexpr int SPLIT = BN / NT;                         // tiles per 256 x 256 tile
+  static constexpr int SMEM = STAGES * STAGE + 1024 + 1024 + EPI_SCRATCH;
+  static_assert(8 * (2 * STAGES + 2 * ACC + 1) <= 256, "barriers below the TMEM slot");
 };
-static_assert(8 * (2 * PairTile<64>::STAGES + 2 * PairTile<64>::ACC + 1) <= 256 &&
-                  8 * (2 * PairTile<128>::STAGES + 2 * PairTile<128>::ACC + 1) <= 256,
-              "barriers below the TMEM slot");
 
 __host__ __device__ inline int64_t num_pair_tiles(int64_t Np) {
   const int64_t tj = Np / BN;
@@ -1130,8 +1142,9 @@ __device__ __forceinline__ bool produce_item(RingPos& rg, const CUtensorMap* map
     const int bufB = mB == 0 ? cur0 : st->cur1[mB - 1];
     const int zAh = zop(mA, bufA, 0, k, z0c), zAl = zop(mA, bufA, 1, k, z0c);
     const int zBh = zop(mB, bufB, 0, k, z0c), zBl = zop(mB, bufB, 1, k, z0c);
-    for (int kq = 0; kq < kblocks; ++kq) {
-      const int kb = rev ? kblocks - 1 - kq : kq;
+    const int nst = (kblocks * BK + PT::SK - 1) / PT::SK;
+    for (int kq = 0; kq < nst; ++kq) {
+      const int x = (rev ? nst - 1 - kq : kq) * PT::SK;
       if (!mbar_wait_warp(bar_empty + 8 * rg.idx, rg.phase ^ 1, limit_ns, abort_flag,
                           timeout_global))
         return false;
@@ -1139,10 +1152,10 @@ __device__ __forceinline__ bool produce_item(RingPos& rg, const CUtensorMap* map
       const uint32_t fb = lead_full + 8 * rg.idx;
       if (elect_one()) {
         if (leader) mbar_expect_tx(bar_full + 8 * rg.idx, 2 * PT::STAGE);
-        tma_load_3d_pair(sA, map, kb * BK, rowA, zAh, fb);
-        tma_load_3d_pair(sA + A_BYTES, map, kb * BK, rowA, zAl, fb);
-        tma_load_3d_pair(sA + 2 * A_BYTES, mapB, kb * BK, rowB, zBh, fb);
-        tma_load_3d_pair(sA + 2 * A_BYTES + PT::PB_BYTES, mapB, kb * BK, rowB, zBl, fb);
+        tma_load_3d_pair(sA, map, x, rowA, zAh, fb);
+        tma_load_3d_pair(sA + PT::PA_BYTES, map, x, rowA, zAl, fb);
+        tma_load_3d_pair(sA + 2 * PT::PA_BYTES, mapB, x, rowB, zBh, fb);
+        tma_load_3d_pair(sA + 2 * PT::PA_BYTES + PT::PB_BYTES, mapB, x, rowB, zBl, fb);
       }
       __syncwarp();
       rg.next(PT::STAGES);
@@ -1163,64 +1176,75 @@ __device__ __forceinline__ void producer_drain(RingPos rg, int stages, uint32_t 
   }
 }
 
-// MMA issuer of a pair kernel (leader CTA, one thread), one work item of
-// `nst` stages: per stage the three products hi*hi, hi*lo, lo*hi for two K16
-// steps into the current accumulation chunk; a chunk ends every `chunk`
-// stages and at the end of each K pass (so chunks never straddle a pass), the
-// first of a pass after chunk - cp0 stages, and is then published to both
-// CTAs.  False when a bounded wait expired.
+// MMA issuer of a pair kernel (leader CTA, one warp), one work item: per K
+// block of 32 the three products hi*hi, hi*lo, lo*hi for two K16 steps into
+// the current accumulation chunk; a chunk ends every `chunk` blocks and at the
+// end of each K pass (so chunks never straddle a pass), the first of a pass
+// after chunk - cp0 blocks, and is then published to both CTAs.  False when a
+// bounded wait expired.
+//
+// The whole warp runs the loop and one elected lane issues: what bounds a
+// narrow tile is the issue of its MMAs, and with the loop under `lane == 0`
+// the compiler handles each instruction's operands per lane.  Per 32-wide
+// block at N = 64 / 128 that took 0.39 / 0.41 us, with the elected lane 0.24 us
+// each.
 template <bool BF16, int NT>
-__device__ __forceinline__ bool mma_item(RingPos& rg, RingPos& tb, int nst, int kblocks,
-                                         int chunk, int cp0, uint32_t tmem_base, uint32_t ring,
-                                         uint32_t bar_full, uint32_t bar_empty,
+__device__ __forceinline__ bool mma_item(RingPos& rg, RingPos& tb, int passes, int kblocks,
+                                         int chunk, int cp0, bool rev, uint32_t tmem_base,
+                                         uint32_t ring, uint32_t bar_full, uint32_t bar_empty,
                                          uint32_t bar_tfull, uint32_t bar_tempty,
                                          uint64_t limit_ns, volatile int* abort_flag,
                                          int* timeout_global) {
   using PT = PairTile<NT>;
   constexpr uint32_t idesc = make_idesc_m256(BF16 ? 1 : 0, NT);
-  uint32_t d = 0, acc = 0;
-  int sp = 0;   // stage within its K pass
-  int cp = cp0;   // stage within its accumulation chunk
-  bool fresh = true;
-  for (int si = 0; si < nst; ++si) {
-    if (fresh) {
-      fresh = false;
-      if (!mbar_wait_warp(bar_tempty + 8 * tb.idx, tb.phase ^ 1, limit_ns, abort_flag,
-                          timeout_global))
+  constexpr int H = PT::SK / BK;   // blocks per stage
+  const int nst = (kblocks + H - 1) / H;
+  for (int pass = 0; pass < passes; ++pass) {
+    uint32_t d = 0;
+    int cp = cp0;   // block within its accumulation chunk
+    bool fresh = true;
+    for (int sq = 0; sq < nst; ++sq) {
+      if (!mbar_wait_warp(bar_full + 8 * rg.idx, rg.phase, limit_ns, abort_flag, timeout_global))
         return false;
-      fence_after();
-      d = tmem_base + (uint32_t)(tb.idx * NT);
-      acc = 0;
-    }
-    if (!mbar_wait_warp(bar_full + 8 * rg.idx, rg.phase, limit_ns, abort_flag, timeout_global))
-      return false;
-    fence_after();
-    const uint32_t sA = ring + rg.idx * PT::STAGE;
-    const uint64_t ah = sw64_desc(sA), al = sw64_desc(sA + A_BYTES);
-    const uint64_t bh = sw64_desc(sA + 2 * A_BYTES);
-    const uint64_t bl = sw64_desc(sA + 2 * A_BYTES + PT::PB_BYTES);
-    const bool pass_end = ++sp == kblocks;
-    const bool chunk_end = ++cp == chunk || pass_end;
-    if (elect_one()) {
+      const uint32_t sA = ring + rg.idx * PT::STAGE;
+      const uint64_t ah = sw128_desc(sA), al = sw128_desc(sA + PT::PA_BYTES);
+      const uint64_t bh = sw128_desc(sA + 2 * PT::PA_BYTES);
+      const uint64_t bl = sw128_desc(sA + 2 * PT::PA_BYTES + PT::PB_BYTES);
 #pragma unroll
-      for (int kk = 0; kk < BK / 16; ++kk) {
-        const uint64_t off = (uint64_t)((kk * 32) >> 4);
-        mma_f16_pair(d, ah + off, bh + off, idesc, kk == 0 ? acc : 1u);   // hi * hi
-        mma_f16_pair(d, ah + off, bl + off, idesc, 1);                    // hi * lo
-        mma_f16_pair(d, al + off, bh + off, idesc, 1);                    // lo * hi
+      for (int hq = 0; hq < H; ++hq) {
+        const int h = rev ? H - 1 - hq : hq;
+        const int blk = (rev ? nst - 1 - sq : sq) * H + h;
+        if (blk >= kblocks) continue;   // the padding half of the last stage
+        uint32_t acc = 1;
+        if (fresh) {
+          if (!mbar_wait_warp(bar_tempty + 8 * tb.idx, tb.phase ^ 1, limit_ns, abort_flag,
+                              timeout_global))
+            return false;
+          d = tmem_base + (uint32_t)(tb.idx * NT);
+          acc = 0;
+        }
+        fence_after();
+        fresh = ++cp == chunk || blk == (rev ? 0 : kblocks - 1);   // the chunk's last block
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            const uint64_t off = (uint64_t)((h * BK * 2 + kk * 32) >> 4);
+            mma_f16_pair(d, ah + off, bh + off, idesc, kk == 0 ? acc : 1u);   // hi * hi
+            mma_f16_pair(d, ah + off, bl + off, idesc, 1);                    // hi * lo
+            mma_f16_pair(d, al + off, bh + off, idesc, 1);                    // lo * hi
+          }
+          if (fresh) mma_commit_pair(bar_tfull + 8 * tb.idx);   // chunk ready in both CTAs
+        }
+        __syncwarp();
+        if (fresh) {
+          tb.next(PT::ACC);
+          cp = 0;
+        }
       }
-      mma_commit_pair(bar_empty + 8 * rg.idx);   // frees the stage in both CTAs
-      if (chunk_end) mma_commit_pair(bar_tfull + 8 * tb.idx);   // chunk ready in both CTAs
+      if (elect_one()) mma_commit_pair(bar_empty + 8 * rg.idx);   // frees the stage in both CTAs
+      __syncwarp();
+      rg.next(PT::STAGES);
     }
-    __syncwarp();
-    acc = 1;
-    rg.next(PT::STAGES);
-    if (chunk_end) {
-      tb.next(PT::ACC);
-      fresh = true;
-      cp = pass_end ? cp0 : 0;
-    }
-    if (pass_end) sp = 0;
   }
   return true;
 }
@@ -1402,8 +1426,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         if (v < vbase) continue;
         const int64_t it = (v - vbase) / SP;
         const int job = job_at(jmask, (int)(it / tiles));
-        ok = mma_item<BF16, NT>(rg, tb, job_passes(job, k1) * kblocks, kblocks, chunk,
-                                kchunk0(Np, kblocks, chunk, item_rev(v)), tmem_base, ring,
+        ok = mma_item<BF16, NT>(rg, tb, job_passes(job, k1), kblocks, chunk,
+                                kchunk0(Np, kblocks, chunk, item_rev(v)), item_rev(v), tmem_base, ring,
                                 bar_full, bar_empty, bar_tfull, bar_tempty, limit_ns, abort_flag,
                                 timeout_global);
       }
@@ -1632,6 +1656,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     layer_tc2_group_kernel(const GroupInst* __restrict__ inst, int count, int* group_timeout,
                            GroupQueue* gq, uint64_t limit_ns, int chunk, int k_snake, int band) {
   using CV = Cvt<BF16>;
+  using PT = PairTile<BN>;
   using H16 = typename CV::T;
   extern __shared__ uint8_t smem_raw[];
 
@@ -1639,7 +1664,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
   const uint32_t ring = base;
-  uint8_t* misc = gbase + P_STAGES * P_STAGE_BYTES;
+  uint8_t* misc = gbase + PT::STAGES * PT::STAGE;
   int64_t* first = reinterpret_cast<int64_t*>(misc + 1024 + EPI_SCRATCH);
   uint32_t* jmask = reinterpret_cast<uint32_t*>(first + count + 1);
 
@@ -1672,8 +1697,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);
   const uint32_t bar_full = smem_u32(bars);
-  const uint32_t bar_empty = bar_full + 8 * P_STAGES;
-  const uint32_t bar_tfull = bar_empty + 8 * P_STAGES;
+  const uint32_t bar_empty = bar_full + 8 * PT::STAGES;
+  const uint32_t bar_tfull = bar_empty + 8 * PT::STAGES;
   const uint32_t bar_tempty = bar_tfull + 8 * 2;
   const uint32_t bar_drain = bar_tempty + 8 * 2;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 256);
@@ -1686,7 +1711,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < P_STAGES; ++s) {
+    for (int s = 0; s < PT::STAGES; ++s) {
       mbar_init(bar_full + 8 * s, 1);
       mbar_init(bar_empty + 8 * s, 1);
     }
@@ -1740,7 +1765,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
                           itm.kblocks, itm.rev, leader, ring, bar_full, bar_empty, lead_full,
                           limit_ns, abort_flag, timeout_global);
       }
-      if (lane == 0) producer_drain(rg, P_STAGES, bar_empty, limit_ns);
+      if (lane == 0) producer_drain(rg, PT::STAGES, bar_empty, limit_ns);
     }
   } else if (warp == 1) {
     // ================= MMA issuer (leader CTA only) =================
@@ -1755,7 +1780,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g == kNoItem) break;
         const GroupItem itm = group_item(inst, first, jmask, count, g, k_snake, chunk);
-        ok = mma_item<BF16, BN>(rg, tb, itm.passes * itm.kblocks, itm.kblocks, chunk, itm.cp0,
+        ok = mma_item<BF16, BN>(rg, tb, itm.passes, itm.kblocks, chunk, itm.cp0, itm.rev,
                             tmem_base, ring, bar_full, bar_empty, bar_tfull, bar_tempty, limit_ns,
                             abort_flag, timeout_global);
       }
@@ -2073,7 +2098,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g == kNoItem) break;
         const GroupItem128 itm = group_item128(inst, first, jmask, count, g);
-        ok = mma_item<BF16, G_BN>(rg, tb, itm.passes * itm.kblocks, itm.kblocks, chunk, 0,
+        ok = mma_item<BF16, G_BN>(rg, tb, itm.passes, itm.kblocks, chunk, 0, false,
                                   tmem_base, ring, bar_full, bar_empty, bar_tfull, bar_tempty,
                                   limit_ns, abort_flag, timeout_global);
       }
@@ -2211,6 +2236,10 @@ PairKernel pair_kernel(bool bf16, int nt) {
   return bf16 ? layer_tc2_kernel<true, BN> : layer_tc2_kernel<false, BN>;
 }
 
+int pair_smem(int nt) {
+  return nt == 64 ? PairTile<64>::SMEM : (nt == 128 ? PairTile<128>::SMEM : PairTile<BN>::SMEM);
+}
+
 // Tile width of the pair kernel for `tiles` 256 x 256 tiles of 1 + k jobs.
 // Measured time per layer in us of a whole solve, 256 / 128 / 64 wide:
 //   n = 128 k = 1   29 /  22 /  20       n = 2048 k = 1   84 /  74 / 106
@@ -2258,8 +2287,10 @@ int device_setup() {
     for (bool bf16 : {false, true})
       for (int nt : {256, 128, 64})
         cudaFuncSetAttribute(pair_kernel(bf16, nt), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             P_SMEM_BYTES);
-    constexpr int group_smem = P_SMEM_BYTES + (kGroupMax + 1) * (int)sizeof(int64_t) +
+                             pair_smem(nt));
+    constexpr int ring_smem =
+        PairTile<BN>::SMEM > GT::SMEM ? PairTile<BN>::SMEM : GT::SMEM;
+    constexpr int group_smem = ring_smem + (kGroupMax + 1) * (int)sizeof(int64_t) +
                                kGroupMax * (int)sizeof(uint32_t);
     static_assert(group_smem <= 227 * 1024, "grouped kernel shared memory");
     cudaFuncSetAttribute(layer_tc2_group_kernel<false>,
@@ -2288,16 +2319,18 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
   return fn;
 }
 
-bool make_map(CUtensorMap* map, void* base, int64_t Np, int slices, int box_rows, bool bf16) {
+// sk: K elements per box (32 or 64: 64- or 128-byte swizzle)
+bool make_map(CUtensorMap* map, void* base, int64_t Np, int slices, int box_rows, bool bf16,
+              int sk) {
   auto enc = get_encoder();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)Np, (cuuint64_t)Np, (cuuint64_t)slices};
   cuuint64_t strides[2] = {(cuuint64_t)Np * 2, (cuuint64_t)Np * Np * 2};
-  cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)sk, (cuuint32_t)box_rows, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
                    3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   sk == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
@@ -2318,8 +2351,9 @@ bool make_group_inst(const Layout& L, void* ws, int sm_count, GroupInst* gi, boo
   char* base = (char*)ws;
   const bool bf16 = L.precision == DMPT_DUAL_BF16;
   const int slices = 2 * (1 + L.k) * 2 + 2 * L.tape_states;
-  if (!make_map(&gi->map, base + L.off_ops16, L.Np, slices, BM, bf16)) return false;
-  if (n128 && !make_map(&gi->map64, base + L.off_ops16, L.Np, slices, GT::B_ROWS, bf16)) return false;
+  if (!make_map(&gi->map, base + L.off_ops16, L.Np, slices, BM, bf16, GT::SK)) return false;
+  if (n128 && !make_map(&gi->map64, base + L.off_ops16, L.Np, slices, GT::B_ROWS, bf16, GT::SK))
+    return false;
   gi->st = (State*)(base + L.off_state);
   gi->master = (float*)(base + L.off_master);
   gi->ops = (uint16_t*)(base + L.off_ops16);
@@ -2343,7 +2377,7 @@ cudaError_t launch_layer_tc_group(const GroupInst* inst, int count, bool bf16, i
   if (count < 1 || count > kGroupMax || !queue || sm_count / 2 > kQueuePairs)
     return cudaErrorInvalidValue;
   const int smem =
-      P_SMEM_BYTES + (count + 1) * (int)sizeof(int64_t) + count * (int)sizeof(uint32_t);
+      (n128 ? GT::SMEM : PairTile<BN>::SMEM) + (count + 1) * (int)sizeof(int64_t) + count * (int)sizeof(uint32_t);
   if (device_setup() == 0) return cudaErrorInvalidDevice;
   const uint64_t limit_ns = (uint64_t)(timeout_s * 1e9);
   const int ck = accum_chunk_k > 0 ? accum_chunk_k : DEFAULT_CHUNK_K;
@@ -2381,8 +2415,9 @@ cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double ti
   // 256 x 256 tiles of every job (the jobs that run are only known on the device)
   const int64_t ptiles = num_pair_tiles(L.Np), pitems = ptiles * (1 + L.k);
   const int nt = pair_tile_width(ptiles, L.k, k_blocks(L.n), sms / 2);
-  if (!make_map(&mA, base + L.off_ops16, L.Np, slices, BM, bf16) ||
-      !make_map(&mB, base + L.off_ops16, L.Np, slices, cta_pair ? nt / 2 : BN, bf16))
+  const int sk = cta_pair ? PairTile<BN>::SK : BK;
+  if (!make_map(&mA, base + L.off_ops16, L.Np, slices, BM, bf16, sk) ||
+      !make_map(&mB, base + L.off_ops16, L.Np, slices, cta_pair ? nt / 2 : BN, bf16, sk))
     return cudaErrorInvalidValue;
   const uint64_t limit_ns = (uint64_t)(timeout_s * 1e9);
   int ck = accum_chunk_k > 0 ? accum_chunk_k : DEFAULT_CHUNK_K;
@@ -2398,7 +2433,7 @@ cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double ti
     const int pairs = (int)(max_items < sms / 2 ? max_items : sms / 2);
     const int snake_pairs = (int)(pitems < sms / 2 ? pitems : sms / 2);
     const cudaError_t e = launch_pdl(
-        pair_kernel(bf16, nt), dim3(2 * pairs), dim3(NUM_THREADS), P_SMEM_BYTES, s, mA, mB, st,
+        pair_kernel(bf16, nt), dim3(2 * pairs), dim3(NUM_THREADS), pair_smem(nt), s, mA, mB, st,
         master, ops, L.Np, L.k, partials, L.partial_tiles, limit_ns, chunk, k_snake, snake_pairs,
         band, inject_stall, round_align);
     if (e != cudaSuccess) return e;
