@@ -64,8 +64,11 @@ constexpr int EPI_WARPS = 8;     // two per TMEM lane quadrant (column halves)
 constexpr int EPI_THREADS = 32 * EPI_WARPS;
 constexpr int EPI_WARP0 = 2;     // epilogue = warps 2 .. 9
 constexpr int NUM_THREADS = 64 + EPI_THREADS;
-// Epilogue scratch: the partial sums of a tile (tile_sums_out).
-constexpr int EPI_SCRATCH = 512;
+// Epilogue scratch: the partial sums of a tile (tile_sums_out), then one
+// 32 x 32 block of 16-bit values per epilogue warp, its rows padded to DLD.
+constexpr int EPI_SUMS = 512;
+constexpr int DLD = 34;
+constexpr int EPI_SCRATCH = EPI_SUMS + EPI_WARPS * 32 * DLD * 2;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* align */ + 1024 /* barriers etc */ +
                            EPI_SCRATCH;
 constexpr int DEFAULT_CHUNK_K = 256;  // K elements per tensor-memory accumulation chunk
@@ -467,7 +470,7 @@ __device__ __forceinline__ void store32(void* p, const uint32_t (&v)[8]) {
 //
 // Sixteen columns at a time; a warp's group of 16 columns lies above its 32
 // rows (every element owned: the packed path), below them (nothing to do) or
-// across the diagonal (at most two or three groups of a warp).
+// across the diagonal (two groups, the 32 x 32 block at the warp's rows).
 //
 // Memory access pattern.  A warp holds 32 consecutive rows (one per lane) and
 // the same columns, so an access down a column (lane = row) is one contiguous
@@ -489,17 +492,36 @@ __device__ __forceinline__ void store32(void* p, const uint32_t (&v)[8]) {
 // an FP64 tree for the partial sums a layer of n = 1000, k = 2 took 57 us and
 // one of n = 2048, k = 3 157 us; now 51 and 149 us.  Sixteen warps of half the
 // columns, or loads of S_old two groups ahead, do not change it.
-template <class CV, int NG, class Rel>
+//
+// First 16-column group of a warp (rows from r0, columns from c0) that holds
+// an owned element; its S_old values (element (c, r) at Sc + (c - c0) np).
+__device__ __forceinline__ int epi_first_group(int r0, int c0) {
+  return r0 > c0 ? (r0 - c0) >> 4 : 0;
+}
+__device__ __forceinline__ void epi_load_old(float (&olds)[16], const float* Sc, int np, int g16) {
+#pragma unroll
+  for (int q = 0; q < 16; ++q) olds[q] = __ldcg(Sc + (16 * g16 + q) * np);
+}
+
+// The calling epilogue warp's scratch block, after the partial sums at `red`.
+__device__ __forceinline__ uint16_t* epi_block(float* red) {
+  return reinterpret_cast<uint16_t*>(red + EPI_SUMS / 4) +
+         ((threadIdx.x >> 5) - EPI_WARP0) * (32 * DLD);
+}
+
+// PRE: `olds` holds the first group's S_old on entry (read while the products
+// still ran: tiles of up to 128 columns have the registers); dbuf: this warp's
+// 32 x 32 block of scratch.
+template <class CV, int NG, bool PRE, class Rel>
 __device__ __forceinline__ void rolled_tile_epilogue(
     const uint32_t ta_sum, const float* __restrict__ Sold, float* Snew, typename CV::T* hi_new,
     typename CV::T* lo_new, const int lane, const int64_t Np, const int r, const int c0,
-    const float sg, const float om, const float scale_new, const bool write, TileSums& ts,
-    Rel release) {
+    const float sg, const float om, const float scale_new, const bool write, float (&olds)[16],
+    uint16_t* dbuf, TileSums& ts, Rel release) {
   const int r0 = r - lane;   // row of lane 0
   const int np = (int)Np;
   // groups below the warp's rows come first, groups above them last
-  int g16 = (r0 - c0) >> 4;
-  g16 = g16 < 0 ? 0 : g16;
+  int g16 = epi_first_group(r0, c0);
   if (g16 >= NG) {
     release();
     return;
@@ -522,92 +544,123 @@ __device__ __forceinline__ void rolled_tile_epilogue(
   const f32x2 sg2 = pack2(sg, sg), om2 = pack2(om, om), sc2 = pack2(scale_new, scale_new);
   const f32x2 neg2 = pack2(-1.0f, -1.0f), zero2 = pack2(0.0f, 0.0f);
   f32x2 fs = zero2, fc = zero2, fd = zero2, z = zero2;
-  float olds[16];   // S_old of the current 16 columns; the next 16 are loaded
-                    // while the current ones are stored
-#pragma unroll
-  for (int q = 0; q < 16; ++q) olds[q] = __ldcg(Sc + (16 * g16 + q) * np);
+  if constexpr (!PRE) epi_load_old(olds, Sc, np, g16);
 #pragma unroll 1
   for (; g16 < NG; ++g16) {
     uint32_t xs[16];
     tmem_ld16(ta_sum + 16 * g16, xs);
     if (g16 == NG - 1) release();
-    const int cb16 = c0 + 16 * g16;
-    uint32_t hp[8], lp[8];   // hi / lo of the column pairs
-    if (cb16 >= r0 + 32) {   // every column right of every row
+    const int d = c0 + 16 * g16 - r0;   // < 32: a group on the diagonal
+    if (d < 32) {
+      // elements below the diagonal belong to their mirror elements; the one on
+      // it counts half (the sums are doubled at the end)
+      float xd = 0.0f, od = 0.0f;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const f32x2 x = pack2(__uint_as_float(xs[2 * i]), __uint_as_float(xs[2 * i + 1]));
-        const f32x2 o = pack2(olds[2 * i], olds[2 * i + 1]);
-        z = fma2(x, zero2, z);               // becomes NaN with a non-finite x
-        const f32x2 d = fma2(x, neg2, o);
-        fd = fma2(d, d, fd);                 // each element counts twice: at the end
-        const f32x2 nw = fma2(sg2, x, mul2(om2, o));
-        // ||S_new||^2: the square as p + e (p = -np2), fs + p by TwoSum
-        const f32x2 np2 = mul2(nw, mul2(nw, neg2));
-        const f32x2 e = fma2(nw, nw, np2);
-        const f32x2 tt = fma2(np2, neg2, fs);
-        const f32x2 bp = fma2(fs, neg2, tt);
-        const f32x2 t2 = fma2(fma2(bp, neg2, tt), neg2, fs);
-        const f32x2 t3 = add2(np2, bp);
-        fc = add2(fc, add2(fma2(t3, neg2, t2), e));
-        fs = tt;
-        const f32x2 y = mul2(nw, sc2);
-        float y0, y1, n0, n1;
-        unpack2(y, y0, y1);
-        unpack2(nw, n0, n1);
-        float h0, h1;
-        hp[i] = CV::pack(y0, y1);
-        CV::unpack(hp[i], h0, h1);
-        float l0, l1;
-        unpack2(fma2(pack2(h0, h1), neg2, y), l0, l1);
-        lp[i] = CV::pack(l0, l1);
-        if (write) {
-          const int m = (16 * g16 + 2 * i) * np;
+      for (int e = 0; e < 16; ++e) {
+        if (d + e == lane) {
+          xd = __uint_as_float(xs[e]);
+          od = olds[e];
+        }
+        if (d + e < lane) xs[e] = 0u;
+        if (d + e < lane) olds[e] = 0.0f;
+      }
+      const float dd = od - xd, n1 = sg * xd + om * od;
+      ts.fd_s = fmaf(-0.5f * dd, dd, ts.fd_s);
+      const float p = -0.5f * n1 * n1;
+      ff_add(ts.fn_s, ts.fn_c, p, fmaf(-0.5f * n1, n1, -p));
+      if (write) ts.tr += n1;
+    }
+    uint32_t hp[8], lp[8];   // hi / lo of the column pairs
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const f32x2 x = pack2(__uint_as_float(xs[2 * i]), __uint_as_float(xs[2 * i + 1]));
+      const f32x2 o = pack2(olds[2 * i], olds[2 * i + 1]);
+      z = fma2(x, zero2, z);               // becomes NaN with a non-finite x
+      const f32x2 dx = fma2(x, neg2, o);
+      fd = fma2(dx, dx, fd);               // each element counts twice: at the end
+      const f32x2 nw = fma2(sg2, x, mul2(om2, o));
+      // ||S_new||^2: the square as p + e (p = -np2), fs + p by TwoSum
+      const f32x2 np2 = mul2(nw, mul2(nw, neg2));
+      const f32x2 e = fma2(nw, nw, np2);
+      const f32x2 tt = fma2(np2, neg2, fs);
+      const f32x2 bp = fma2(fs, neg2, tt);
+      const f32x2 t2 = fma2(fma2(bp, neg2, tt), neg2, fs);
+      const f32x2 t3 = add2(np2, bp);
+      fc = add2(fc, add2(fma2(t3, neg2, t2), e));
+      fs = tt;
+      const f32x2 y = mul2(nw, sc2);
+      float y0, y1, n0, n1;
+      unpack2(y, y0, y1);
+      unpack2(nw, n0, n1);
+      float h0, h1;
+      hp[i] = CV::pack(y0, y1);
+      CV::unpack(hp[i], h0, h1);
+      float l0, l1;
+      unpack2(fma2(pack2(h0, h1), neg2, y), l0, l1);
+      lp[i] = CV::pack(l0, l1);
+      if (write) {
+        const int m = (16 * g16 + 2 * i) * np;
+        if (d >= 32) {
           Snc[m] = n0;
           Snc[m + np] = n1;
           const uint32_t ho = __shfl_xor_sync(0xffffffffu, hp[i], 1);
           const uint32_t lo = __shfl_xor_sync(0xffffffffu, lp[i], 1);
           *reinterpret_cast<uint32_t*>(hip + m) = __byte_perm(hp[i], ho, sel);
           *reinterpret_cast<uint32_t*>(lop + m) = __byte_perm(lp[i], lo, sel);
+        } else {
+          if (d + 2 * i >= lane) Snc[m] = n0;
+          if (d + 2 * i + 1 >= lane) Snc[m + np] = n1;
         }
       }
-      if (write) {
+    }
+    if (write) {
+      if (d >= 32) {
         store32(hir + 16 * g16, hp);
         store32(lor + 16 * g16, lp);
-      }
-    } else {   // a group on the diagonal
+      } else {
+        // Both triangles of the 32 x 32 block on the diagonal (r0 and c0 are
+        // multiples of 32) go through the warp's scratch block, whose finished
+        // rows are stored whole: after the first group columns 0 .. 15 of rows
+        // 0 .. 15, after the second the rest.  (Stored one by one, 16-bit
+        // elements of every row went to 32 lines per instruction: 6.2 us of
+        // epilogue in the layers of n = 128.)
 #pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const int c = cb16 + e;
-        if (c < r) continue;   // owned by the mirrored element
-        const float xv = __uint_as_float(xs[e]);
-        const float w = c == r ? 0.5f : 1.0f;
-        ts.bad = ts.bad || !isfinite(xv);
-        const float dd = olds[e] - xv;
-        ts.fd_s = fmaf(w * dd, dd, ts.fd_s);
-        if (!write) continue;
-        const float n1 = sg * xv + om * olds[e];
-        const float p = w * n1 * n1;
-        ff_add(ts.fn_s, ts.fn_c, p, fmaf(w * n1, n1, -p));
-        if (c == r) ts.tr = n1;
-        const float y = n1 * scale_new;
-        const typename CV::T h = CV::to(y);
-        const uint16_t hb = (uint16_t)h16_bits(h);
-        const uint16_t lb = (uint16_t)h16_bits(CV::to(y - CV::from(h)));
-        const int m = (16 * g16 + e) * np;
-        Snc[m] = n1;
-        hir[16 * g16 + e] = hb;
-        lor[16 * g16 + e] = lb;
-        if (c > r) {
-          hic[m] = hb;
-          loc[m] = lb;
+        for (int part = 0; part < 2; ++part) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const uint32_t v = part ? lp[i] : hp[i];
+            const int cl = d + 2 * i;   // column within the block
+            if (cl >= lane) {
+              dbuf[lane * DLD + cl] = (uint16_t)v;
+              dbuf[cl * DLD + lane] = (uint16_t)v;
+            }
+            if (cl + 1 >= lane) {
+              dbuf[lane * DLD + cl + 1] = (uint16_t)(v >> 16);
+              dbuf[(cl + 1) * DLD + lane] = (uint16_t)(v >> 16);
+            }
+          }
+          __syncwarp();
+          // the columns left of this group belong to the block as well in the
+          // second group's new rows (lanes 16 .. 31)
+          uint16_t* row = (part ? lor : hir) + 16 * g16;
+          const uint32_t* src = reinterpret_cast<const uint32_t*>(dbuf + lane * DLD + d);
+          if (d == 16 || lane < 16) {
+            uint32_t v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = src[i];
+            store32(row, v);
+          }
+          if (d == 16 && lane >= 16) {
+            uint32_t v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = src[i - 8];
+            store32(row - 16, v);
+          }
+          __syncwarp();
         }
       }
     }
-    if (g16 < NG - 1) {
-#pragma unroll
-      for (int q = 0; q < 16; ++q) olds[q] = __ldcg(Sc + (16 * (g16 + 1) + q) * np);
-    }
+    if (g16 < NG - 1) epi_load_old(olds, Sc, np, g16 + 1);
   }
   float a0, a1, b0, b1;
   unpack2(fs, a0, a1);
@@ -628,7 +681,7 @@ __device__ __forceinline__ void rolled_tile_epilogue(
 // while the others go on.  (Every thread's sums through an FP64 tree in
 // shared memory took ten barriers and about 5 K clocks per item.)
 constexpr int RED_FLOATS = 8;   // per warp: fn (s, c), fd (s, c), tr (s, c), bad, -
-static_assert(2 * EPI_WARPS * RED_FLOATS * 4 <= EPI_SCRATCH, "two buffers");
+static_assert(2 * EPI_WARPS * RED_FLOATS * 4 <= EPI_SUMS, "two buffers");
 __device__ __forceinline__ void tile_sums_out(TileSums ts, float* red, uint32_t seq, int ewarp,
                                               int lane, double* entry) {
   float tc = 0.0f;
@@ -947,14 +1000,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       H16* hi_new = reinterpret_cast<H16*>(ops) + (size_t)zh_new * mat;
       H16* lo_new = reinterpret_cast<H16*>(ops) + (size_t)(zh_new + 1) * mat;
 
+      float olds[16];
       TileSums ts;
       auto release = [&]() {   // the accumulator goes back to the MMA
         fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty + 8 * ab);
       };
-      rolled_tile_epilogue<CV, 8>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
-                                   scale_new, write, ts, release);
+      rolled_tile_epilogue<CV, 8, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
+                                   scale_new, write, olds, epi_block(red), ts, release);
       if (++ab == 2) {
         ab = 0;
         abphase ^= 1;
@@ -1015,41 +1069,42 @@ __host__ __device__ inline int64_t num_pair_tiles(int64_t Np) {
   return tj * (tj + 1) / 2;
 }
 // pair tile t -> (I2, J), I2 <= J, J-major
-__device__ __forceinline__ void pair_tile_coords(int64_t t, int* I2, int* J) {
-  int j = (int)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-  while ((int64_t)(j + 1) * (j + 2) / 2 <= t) ++j;
-  while ((int64_t)j * (j + 1) / 2 > t) --j;
-  *J = j;
-  *I2 = (int)(t - (int64_t)j * (j + 1) / 2);
+__device__ __forceinline__ void pair_tile_coords(unsigned t, int* I2, int* J) {
+  unsigned j = (unsigned)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while ((j + 1) * (j + 2) / 2 <= t) ++j;
+  while (j * (j + 1) / 2 > t) --j;
+  *J = (int)j;
+  *I2 = (int)(t - j * (j + 1) / 2);
 }
 
 // Banded order of the pair tiles (I2 <= J): column blocks are grouped into
 // bands of `band` blocks; inside a band the tiles run I2-major, so the pairs
 // working at the same time cover a compact block of rows and columns and
 // share their operand panels in L2.  band <= 0 keeps the plain J-major order.
-__device__ __forceinline__ void pair_tile_banded(int64_t t, int tj, int band, int* I2, int* J) {
+// (Tile indexes fit 32 bits: a matrix of 2^31 tiles would not fit any memory.)
+__device__ __forceinline__ void pair_tile_banded(unsigned t, int tj, int band, int* I2, int* J) {
   if (band <= 0) {
     pair_tile_coords(t, I2, J);
     return;
   }
-  int J0 = 0;
+  unsigned J0 = 0;
   while (true) {
-    const int w = tj - J0 < band ? tj - J0 : band;
-    const int64_t cnt = (int64_t)J0 * w + (int64_t)w * (w + 1) / 2;   // tiles in this band
-    if (t < cnt || J0 + w >= tj) {
-      if (t < (int64_t)J0 * w) {          // rows above the band's diagonal block
+    const unsigned w = tj - J0 < (unsigned)band ? tj - J0 : band;
+    const unsigned cnt = J0 * w + w * (w + 1) / 2;   // tiles in this band
+    if (t < cnt || J0 + w >= (unsigned)tj) {
+      if (t < J0 * w) {          // rows above the band's diagonal block
         *I2 = (int)(t / w);
-        *J = J0 + (int)(t % w);
+        *J = (int)(J0 + t % w);
         return;
       }
-      int64_t u = t - (int64_t)J0 * w;    // upper triangle of the w x w diagonal block
-      int r = 0;
+      unsigned u = t - J0 * w;    // upper triangle of the w x w diagonal block
+      unsigned r = 0;
       while (u >= w - r) {
         u -= w - r;
         ++r;
       }
-      *I2 = J0 + r;
-      *J = J0 + r + (int)u;
+      *I2 = (int)(J0 + r);
+      *J = (int)(J0 + r + u);
       return;
     }
     t -= cnt;
@@ -1371,12 +1426,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   // a square alone: it then numbers the square's items as the forward launch
   // did, after its response items, so each tile keeps its round and K-snake
   // direction and the recomputed states are bit-identical)
-  const int64_t vbase = SP * st->item_base;
+  const unsigned vbase = SP * (unsigned)st->item_base;
 
-  const int64_t pair = blockIdx.x >> 1;
-  const int64_t npairs = gridDim.x >> 1;
-  const int64_t tiles = num_pair_tiles(Np);
-  const int64_t items = SP * tiles * njobs;
+  const unsigned pair = blockIdx.x >> 1;
+  const unsigned npairs = gridDim.x >> 1;
+  const unsigned tiles = (unsigned)num_pair_tiles(Np);
+  const unsigned items = SP * tiles * (unsigned)njobs;
   const int kblocks = k_blocks(st->n);
 
   int* timeout_global = &gst->timeout_flag;
@@ -1387,7 +1442,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   // last, which are still in L2.  Narrower tiles keep the direction of the
   // 256 x 256 tile they are part of: an element's sums, and so the results,
   // are the same bit for bit at every width.
-  auto item_rev = [&](int64_t v) { return k_snake && ((v / SP / snake_pairs) & 1); };
+  auto item_rev = [&](unsigned v) {
+    return k_snake && ((v / SP / (unsigned)snake_pairs) & 1u);
+  };
 
   if (njobs == 0) {
     // nothing to do in this launch
@@ -1397,9 +1454,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       RingPos rg;
       bool ok = true;
       bool align = round_align != 0 && SP == 1;
-      for (int64_t v = pair; v < vbase + items && ok; v += npairs) {
+      for (unsigned v = pair; v < vbase + items && ok; v += npairs) {
         if (v < vbase) continue;
-        const int64_t it = (v - vbase) / SP;
+        const unsigned it = (v - vbase) / SP;
         if (SP == 1 && v >= npairs) {
           if (lane == 0) round_start(&gst->round_ctr, v / npairs, items, npairs, align);
           __syncwarp();
@@ -1422,9 +1479,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       // test hook (see the single-CTA kernel)
       bool ok = !(inject_stall &&
                   !mbar_wait_warp(bar_drain, 0, limit_ns, abort_flag, timeout_global));
-      for (int64_t v = pair; v < vbase + items && ok; v += npairs) {
+      for (unsigned v = pair; v < vbase + items && ok; v += npairs) {
         if (v < vbase) continue;
-        const int64_t it = (v - vbase) / SP;
+        const unsigned it = (v - vbase) / SP;
         const int job = job_at(jmask, (int)(it / tiles));
         ok = mma_item<BF16, NT>(rg, tb, job_passes(job, k1), kblocks, chunk,
                                 kchunk0(Np, kblocks, chunk, item_rev(v)), item_rev(v), tmem_base, ring,
@@ -1451,9 +1508,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     RingPos ab;
     bool alive = true;
     uint32_t seq = 0;   // items done (tile_sums_out)
-    for (int64_t v = pair; v < vbase + items && alive; v += npairs) {
+    for (unsigned v = pair; v < vbase + items && alive; v += npairs) {
       if (v < vbase) continue;
-      const int64_t it = (v - vbase) / SP;
+      const unsigned it = (v - vbase) / SP;
       const bool crev = item_rev(v);
       const int job = job_at(jmask, (int)(it / tiles));
       const int passes = job_passes(job, k1);
@@ -1463,6 +1520,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       // exact power-of-two unscale of the products of passes 0 and 1
       // (passes >= 2 of higher-order terms: cross_unscale)
       const float u01 = ldexpf(1.0f, -(s0e + (job == 0 ? s0e : st->s1_exp_cur[job - 1])));
+      // S_old of this thread's first columns: narrow tiles have the registers to
+      // read them while the products run
+      float olds[16];
+      auto first_old = [&]() {
+        int I2, J;
+        pair_tile_banded(it % tiles, (int)(Np / BN), band, &I2, &J);
+        const int r = I2 * 2 * BM + (int)rank * BM + rloc;
+        const int c0 = J * BN + (int)(v % SP) * NT + half * (NT / 2);
+        const int g0 = epi_first_group(r - lane, c0);
+        const int curj = job == 0 ? cur0 : st->cur1[job - 1];
+        const float* Sc = master + (size_t)(curj * (1 + k) + job) * mat + (size_t)c0 * Np + r;
+        if (g0 < NT / 32) epi_load_old(olds, Sc, (int)Np, g0);
+      };
+      if constexpr (NT < BN) first_old();
       float sum[NT / 2];
 #pragma unroll
       for (int i = 0; i < NT / 2; ++i) sum[i] = 0.0f;
@@ -1497,7 +1568,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       for (int cc = 0; cc < NT / 32; ++cc) tmem_st16(ta_sum + 16 * cc, sum + 16 * cc);
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 
-      const int64_t t = it % tiles;
+      const unsigned t = it % tiles;
       int I2, J;
       pair_tile_banded(t, (int)(Np / BN), band, &I2, &J);
       const int curj = job == 0 ? cur0 : st->cur1[job - 1];
@@ -1519,10 +1590,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab.idx);
       };
-      rolled_tile_epilogue<CV, NT / 32>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
-                                   scale_new, write, ts, release);
+      rolled_tile_epilogue<CV, NT / 32, NT < BN>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
+                                   scale_new, write, olds, epi_block(red), ts, release);
       ab.next(PT::ACC);
-      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, partials + ((size_t)job * ptiles + 2 * (SP * t + v % SP) + rank) * kNQ);
+      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane,
+                    partials + ((size_t)job * ptiles + 2 * (SP * (size_t)t + v % SP) + rank) * kNQ);
     }
   }
 
@@ -1759,7 +1831,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         }
         const State* sti = gi.st;
         int I2, J;
-        pair_tile_banded(itm.t, (int)(gi.Np / BN), band, &I2, &J);
+        pair_tile_banded((unsigned)itm.t, (int)(gi.Np / BN), band, &I2, &J);
         ok = produce_item<BN>(rg, &gi.map, &gi.map, sti, itm.job, itm.passes, gi.k, gi.k, sti->cur0,
                           sti->z0_cur, I2 * 2 * BM + (int)rank * BM, J * BN + (int)rank * BM,
                           itm.kblocks, itm.rev, leader, ring, bar_full, bar_empty, lead_full,
@@ -1866,7 +1938,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       const int64_t Np = gi.Np;
       const size_t mat = (size_t)Np * Np;
       int I2, J;
-      pair_tile_banded(itm.t, (int)(Np / BN), band, &I2, &J);
+      pair_tile_banded((unsigned)itm.t, (int)(Np / BN), band, &I2, &J);
       const int cur0 = sti->cur0;
       const int curj = job == 0 ? cur0 : sti->cur1[job - 1];
       const int e_new = job == 0 ? s0e : sti->s1_exp_next[job - 1];
@@ -1883,14 +1955,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       H16* hi_new = reinterpret_cast<H16*>(gi.ops) + (size_t)zh_new * mat;
       H16* lo_new = reinterpret_cast<H16*>(gi.ops) + (size_t)(zh_new + 1) * mat;
 
+      float olds[16];
       TileSums ts;
       auto release = [&]() {   // the accumulator goes back to the MMA
         fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab);
       };
-      rolled_tile_epilogue<CV, 8>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
-                                   scale_new, write, ts, release);
+      rolled_tile_epilogue<CV, 8, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
+                                   scale_new, write, olds, epi_block(red), ts, release);
       if (++ab == 2) {
         ab = 0;
         abphase ^= 1;
@@ -2196,6 +2269,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       H16* hi_new = reinterpret_cast<H16*>(gi.ops) + (size_t)zh_new * mat;
       H16* lo_new = reinterpret_cast<H16*>(gi.ops) + (size_t)(zh_new + 1) * mat;
 
+      float olds[16];
       TileSums ts;
       auto release = [&]() {   // the accumulator goes back to the MMA
         fence_before();
@@ -2205,8 +2279,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       // rows past Np (a 256-row block over a matrix padded to 128): nothing to
       // store; the products there are zeros
       if ((int64_t)row0 < Np)
-        rolled_tile_epilogue<CV, 4>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
-                                     scale_new, write, ts, release);
+        rolled_tile_epilogue<CV, 4, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
+                                     scale_new, write, olds, epi_block(red), ts, release);
       else
         release();
       ab.next(GT::ACC);
