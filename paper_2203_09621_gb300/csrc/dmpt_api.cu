@@ -183,16 +183,6 @@ Layout layout_for(int64_t n, int k, const dmpt_options* o, int pad = kPad) {
   return make_layout(n, slots, o->precision, tape_states, ckpt_slots, pad);
 }
 
-// The forward's product options, kept for the states the backward recomputes.
-__global__ void state_init_kernel(State* st, int k, int max_layers, int precision, double n_occ,
-                                  double c_pt, double c_d0, int tape, int tape_base,
-                                  int tape_states, int layout_k, int64_t n, int order = 1,
-                                  int k1 = 0, FwdOpts fo = FwdOpts{0, 0, 0, 1, 1, 8},
-                                  int hole = 0) {
-  state_init_fields(st, k, max_layers, precision, n_occ, c_pt, c_d0, tape, tape_base,
-                    tape_states, layout_k, n, order, k1, fo, hole);
-}
-
 // Re-open a finished forward state for the adjoint run (keeps sigma, the
 // bounds, the tape geometry and the number of S0 updates).
 __global__ void adj_state_reset_kernel(State* st) {
@@ -239,7 +229,7 @@ dmpt_status replay_run(dmpt_handle h, const Layout& L, const double* H1, const d
                        void* workspace, cudaStream_t s) {
   State* st = (State*)workspace;
   cudaError_t e;
-  const int blocks = kInitBlocks;
+  const int blocks = init_blocks(L.Np);
   replay_reset_kernel<<<1, 1, 0, s>>>(st, k);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(h, e, "replay reset");
   if ((e = launch_init(L, workspace, nullptr, H1, ld, k, blocks, s, 1, shift)) != cudaSuccess)
@@ -504,23 +494,19 @@ static dmpt_status forward_impl(dmpt_handle h, const double* H, const double* H1
     return fail(h, DMPT_EWORKSPACE, "dmpt_sp2_response: workspace too small%s");
   const bool dual = o->precision >= DMPT_DUAL_FP16;
 
-  char* base = (char*)workspace;
-  State* st = (State*)(base + L.off_state);
-  cudaError_t e = cudaMemsetAsync(st, 0, sizeof(State), s);
-  if (e != cudaSuccess) return cuda_fail(h, e, "state reset");
+  State* st = (State*)((char*)workspace + L.off_state);
   const FwdOpts fo{o->ckpt_every >= 2 ? o->ckpt_every : 0, L.ckpt_slots, o->accum_chunk,
                    o->cta_pair, o->k_snake, o->tile_band};
-  state_init_kernel<<<1, 1, 0, s>>>(st, order >= 2 ? order * k : k, o->max_layers, o->precision,
-                                    (double)n_occ, o->c_pt, o->c_d0, o->ckpt_every == 1 ? 1 : 0,
-                                    4 * (1 + L.k), L.tape_states, L.k, n, order, k, fo,
-                                    use_hole_form(o, n, n_occ));
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(h, e, "state init");
-  if ((e = launch_bounds(H, n, ld, &st->eps1, s)) != cudaSuccess) return cuda_fail(h, e, "bounds");
-  const int init_blocks = kInitBlocks;
-  if ((e = launch_init(L, workspace, H, H1, ld, k, init_blocks, s, 0, nullptr,
+  cudaError_t e = launch_forward_setup(L, workspace, H, ld, order >= 2 ? order * k : k,
+                                       o->max_layers, (double)n_occ, o->c_pt, o->c_d0,
+                                       o->ckpt_every == 1 ? 1 : 0, order, k, fo,
+                                       use_hole_form(o, n, n_occ), s);
+  if (e != cudaSuccess) return cuda_fail(h, e, "set-up");
+  const int iblocks = init_blocks(L.Np);
+  if ((e = launch_init(L, workspace, H, H1, ld, k, iblocks, s, 0, nullptr,
                        (order - 1) * k)) != cudaSuccess)
     return cuda_fail(h, e, "init");
-  if ((e = launch_decide(L, workspace, kDecideInit, init_blocks, s)) != cudaSuccess)
+  if ((e = launch_decide(L, workspace, kDecideInit, iblocks, s)) != cudaSuccess)
     return cuda_fail(h, e, "decide(init)");
   const bool ckpt = o->ckpt_every >= 2;
   if (ckpt && (e = launch_ckpt_store(L, workspace, s)) != cudaSuccess)

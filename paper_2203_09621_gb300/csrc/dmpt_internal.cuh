@@ -213,6 +213,13 @@ inline int64_t fp64_tiles(int64_t n) {
 // ---- launchers (kernels_simt.cu) ----
 cudaError_t launch_bounds(const double* H, int64_t n, int64_t ld, double* eps_out,
                           cudaStream_t s);
+// The start of a forward run: its fresh control block and the bounds of H in
+// it, in two launches.
+cudaError_t launch_forward_setup(const Layout& L, void* ws, const double* H, int64_t ld, int slots,
+                                 int max_layers, double n_occ, double c_pt, double c_d0, int tape,
+                                 int order, int k1, FwdOpts fo, int hole, cudaStream_t s);
+// Blocks (partial-sum entries) of the initial layer of a matrix padded to Np.
+int init_blocks(int64_t Np);
 // first_m = 0: S0 and S1_1..k; first_m = 1: S1 only (response replay), each
 // S1_j = -(H1_j + diag(shift_j)) / (eps_N - eps_1) (shift: k x n or NULL).
 cudaError_t launch_init(const Layout& L, void* ws, const double* H, const double* H1,

@@ -95,9 +95,13 @@ __global__ void bounds_init_kernel(long long* key) {
   key[1] = dkey(-INFINITY);
 }
 
-// one warp per row; row r: centre H_rr, radius sum_{j != r} |H_rj|
+// one warp per row; row r: centre H_rr, radius sum_{j != r} |H_rj|.  With a
+// counter (zero on entry and on return) the last block to finish turns the
+// keys into the bounds.
 __global__ void bounds_rows_kernel(const double* __restrict__ H, int64_t n, int64_t ld,
-                                   long long* key) {
+                                   long long* key, unsigned* counter) {
+  pdl_wait();
+  pdl_launch();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -117,6 +121,19 @@ __global__ void bounds_rows_kernel(const double* __restrict__ H, int64_t n, int6
     atomicMin(&key[0], dkey(lo));
     atomicMax(&key[1], dkey(hi));
   }
+  if (counter == nullptr) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(counter, 1u) == gridDim.x - 1) {
+      __threadfence();
+      double* out = reinterpret_cast<double*>(key);
+      const double b0 = dkey_inv(__ldcg(&key[0])), b1 = dkey_inv(__ldcg(&key[1]));
+      out[0] = b0;
+      out[1] = b1;
+      *counter = 0u;
+    }
+  }
 }
 
 __global__ void bounds_fin_kernel(long long* key) {
@@ -127,15 +144,51 @@ __global__ void bounds_fin_kernel(long long* key) {
   out[1] = hi;
 }
 
+static int bounds_blocks(int64_t n) {
+  const int64_t warps = n < 152 * 64 ? n : 152 * 64;
+  return (int)((warps * 32 + 255) / 256);
+}
+
 cudaError_t launch_bounds(const double* H, int64_t n, int64_t ld, double* eps_out,
                           cudaStream_t s) {
   long long* key = reinterpret_cast<long long*>(eps_out);
   bounds_init_kernel<<<1, 1, 0, s>>>(key);
-  int64_t warps = n < 152 * 64 ? n : 152 * 64;
-  int blocks = (int)((warps * 32 + 255) / 256);
-  bounds_rows_kernel<<<blocks, 256, 0, s>>>(H, n, ld, key);
+  bounds_rows_kernel<<<bounds_blocks(n), 256, 0, s>>>(H, n, ld, key, nullptr);
   bounds_fin_kernel<<<1, 1, 0, s>>>(key);
   return cudaGetLastError();
+}
+
+// A fresh control block of a forward run (zeroed, then its fields) with the
+// keys of the bounds.
+__global__ void __launch_bounds__(256)
+    forward_setup_kernel(State* st, int k, int max_layers, int precision, double n_occ,
+                         double c_pt, double c_d0, int tape, int tape_base, int tape_states,
+                         int layout_k, int64_t n, int order, int k1, FwdOpts fo, int hole) {
+  static_assert(sizeof(State) % 4 == 0, "State zeroed as words");
+  pdl_launch();
+  unsigned* w = reinterpret_cast<unsigned*>(st);
+  for (int i = threadIdx.x; i < (int)(sizeof(State) / 4); i += blockDim.x) w[i] = 0u;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    state_init_fields(st, k, max_layers, precision, n_occ, c_pt, c_d0, tape, tape_base,
+                      tape_states, layout_k, n, order, k1, fo, hole);
+    long long* key = reinterpret_cast<long long*>(&st->eps1);
+    key[0] = dkey(INFINITY);
+    key[1] = dkey(-INFINITY);
+  }
+}
+
+cudaError_t launch_forward_setup(const Layout& L, void* ws, const double* H, int64_t ld, int slots,
+                                 int max_layers, double n_occ, double c_pt, double c_d0, int tape,
+                                 int order, int k1, FwdOpts fo, int hole, cudaStream_t s) {
+  State* st = (State*)((char*)ws + L.off_state);
+  forward_setup_kernel<<<1, 256, 0, s>>>(st, slots, max_layers, L.precision, n_occ, c_pt, c_d0,
+                                         tape, 4 * (1 + L.k), L.tape_states, L.k, L.n, order, k1,
+                                         fo, hole);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_pdl(bounds_rows_kernel, dim3(bounds_blocks(L.n)), dim3(256), 0, s, H, L.n, ld,
+                    reinterpret_cast<long long*>(&st->eps1), &st->round_ctr);
 }
 
 // ---------------------------------------------------------------------------
@@ -305,8 +358,15 @@ __global__ void __launch_bounds__(256) init_kernel(State* st, T* master, const d
                                                    int64_t Np, int64_t ld, int k, int first_m,
                                                    const double* __restrict__ shift, int k_zero,
                                                    double* partials, int64_t ptiles) {
+  pdl_wait();
+  pdl_launch();
   init_body<T>(st, master, H, H1, n, Np, ld, k, first_m, shift, k_zero, partials, ptiles,
                blockIdx.x, gridDim.x);
+}
+
+int init_blocks(int64_t Np) {
+  const int64_t tb = Np / kInitTile, pairs = tb * (tb + 1) / 2;
+  return (int)(pairs < kInitBlocks ? pairs : kInitBlocks);
 }
 
 cudaError_t launch_init(const Layout& L, void* ws, const double* H, const double* H1,
@@ -316,14 +376,12 @@ cudaError_t launch_init(const Layout& L, void* ws, const double* H, const double
   State* st = (State*)(base + L.off_state);
   double* partials = (double*)(base + L.off_partials);
   if (L.precision == DMPT_FP64)
-    init_kernel<double><<<blocks, 256, 0, s>>>(st, (double*)(base + L.off_master), H, H1, L.n,
-                                               L.Np, ld, k, first_m, shift, k_zero, partials,
-                                               L.partial_tiles);
-  else
-    init_kernel<float><<<blocks, 256, 0, s>>>(st, (float*)(base + L.off_master), H, H1, L.n,
-                                              L.Np, ld, k, first_m, shift, k_zero, partials,
-                                              L.partial_tiles);
-  return cudaGetLastError();
+    return launch_pdl(init_kernel<double>, dim3(blocks), dim3(256), 0, s, st,
+                      (double*)(base + L.off_master), H, H1, L.n, L.Np, ld, k, first_m, shift,
+                      k_zero, partials, L.partial_tiles);
+  return launch_pdl(init_kernel<float>, dim3(blocks), dim3(256), 0, s, st,
+                    (float*)(base + L.off_master), H, H1, L.n, L.Np, ld, k, first_m, shift, k_zero,
+                    partials, L.partial_tiles);
 }
 
 // ---------------------------------------------------------------------------
@@ -400,18 +458,21 @@ __device__ int fp16_exponent_for(double bound) {
 // per-layer histories) in shared memory.  What bounds it is latency, not work:
 // one thread walking the block in device memory took 9-35 us per layer (a
 // dependent access costs about 0.4 us, an FP64 square root or divide as much).
-// Here the head, the partial sums of every job and the few history entries the
-// tests read are fetched at the same time, 256 threads per job (four jobs at
-// once), and one warp then takes the decisions, lane j those of response slot
-// j.  Measured per step, n = 128 k = 1 / n = 2048 k = 3: 16.5 / 23.5 us
-// before, 5.8 / 7.0 us now (an empty launch takes 2 us).
+// Here the head and the few history entries the tests read are fetched while
+// the layer product still runs, the partial sums of four jobs are added at once
+// by 256 threads each, their square roots are taken in parallel, and one warp
+// then takes the decisions, lane j those of response slot j.  Measured from the
+// end of the layer to the end of the step, n = 128 k = 1: 16.5 us by one
+// thread, 4.0 us with every read after the layer's end and a 256-wide FP64
+// tree per quantity, 3.0 us now.
 constexpr int kDecideThreads = 1024;
 static_assert(kHeadWords <= kDecideThreads, "one head word per thread");
 
 struct DecideShared {
   alignas(16) unsigned head[kHeadWords + (kHeadWords & 1)];
-  double red[kDecideThreads / 256][kNQ][256];
+  double red[kDecideThreads / 256][8][kNQ];
   double sums[kMaxK + 1][kNQ];   // per job, as summed from the partials
+  double roots[kMaxK + 1][kNQ];  // their square roots, taken in parallel
   double fe2[kMaxK];             // FroErr^(1)_{n-2} of the layer that has run
   double iderr1;                 // IdErr_{n-1}
   int sig0, sig1, sig_next;      // sigma_n, sigma_{n-1}; sigma of the layer to plan
@@ -419,8 +480,9 @@ struct DecideShared {
 
 // Plan layer n (Alg. 1: branch choice; Alg. 2: D0 stopping tests).  One warp;
 // S: head in shared memory, G: control block, conv: slot `lane` has stopped.
+// root: sqrt(s1_fro2) of slot `lane`.
 __device__ void plan_layer(State* S, State* G, const DecideShared& sh, int n, int lane,
-                           bool conv) {
+                           bool conv, double root) {
   if (lane == 0) {
     int sigma;
     if (!S->d0_conv) {
@@ -459,7 +521,7 @@ __device__ void plan_layer(State* S, State* G, const DecideShared& sh, int n, in
     //            <= 4.5 ||S1_{n-1}||_F   (spectrum of S0 within [-0.25, 1.25]);
     // an order-o slot (o >= 2) adds sum_{a=1}^{o-1} ||S_a S_{o-a}||_2
     // <= sum ||S_a||_F ||S_{o-a}||_F (twice, for 2 S - S^2)
-    double bound = 4.5 * sqrt(S->s1_fro2[lane]);
+    double bound = 4.5 * root;
     if (S->order >= 2 && lane >= S->k1) {
       const int o = 1 + lane / S->k1, d = lane % S->k1;
       double cross = 0.0;
@@ -475,7 +537,7 @@ __device__ void plan_layer(State* S, State* G, const DecideShared& sh, int n, in
 // min(m - 1, U), the forward's sigma_m (continued by flips past the forward's
 // last layer), responses of the directions still running.
 __device__ void plan_replay(State* S, State* G, const DecideShared& sh, int m, int lane,
-                            bool conv) {
+                            bool conv, double root) {
   if (lane == 0) {
     const int U = S->d0_updates;
     S->z0_cur = S->tape_base + 2 * (m - 1 < U ? m - 1 : U);
@@ -491,9 +553,8 @@ __device__ void plan_replay(State* S, State* G, const DecideShared& sh, int m, i
   }
   if (lane < S->k) {
     S->plan_resp[lane] = !conv;
-    S->s1_exp_next[lane] = S->precision == DMPT_DUAL_FP16
-                               ? fp16_exponent_for(4.5 * sqrt(S->s1_fro2[lane]))
-                               : 0;
+    S->s1_exp_next[lane] =
+        S->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(4.5 * root) : 0;
   }
 }
 
@@ -514,6 +575,7 @@ __device__ void decide_replay(State* S, State* G, const DecideShared& sh, int mo
   if (S->timeout_flag) return decide_end(S, lane, DMPT_ETIMEOUT);
   if (bad) return decide_end(S, lane, DMPT_ENUMERIC);
   bool conv = true;
+  double root = 0.0;   // sqrt(s1_fro2) of this lane's slot
   if (init) {
     if (lane < k) {
       S->cur1[lane] = 0;
@@ -521,7 +583,8 @@ __device__ void decide_replay(State* S, State* G, const DecideShared& sh, int mo
       S->d1_layer[lane] = 0;
       const double f = sh.sums[1 + lane][kQFroNew];
       S->s1_fro2[lane] = f;
-      S->s1_exp_cur[lane] = S->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(sqrt(f)) : 0;
+      root = sh.roots[1 + lane][kQFroNew];
+      S->s1_exp_cur[lane] = S->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(root) : 0;
       conv = false;
     }
     if (lane == 0) {
@@ -529,11 +592,11 @@ __device__ void decide_replay(State* S, State* G, const DecideShared& sh, int mo
       S->rp_layers = 0;
     }
     __syncwarp();
-    return plan_replay(S, G, sh, 1, lane, conv);
+    return plan_replay(S, G, sh, 1, lane, conv, root);
   }
   if (lane < k) conv = S->d1_conv[lane] != 0;
   if (ran) {
-    const double fe = sqrt(sh.sums[1 + lane][kQFroDiff]);
+    const double fe = sh.roots[1 + lane][kQFroDiff];
     G->froerr1[lane][n] = fe;
     const bool fired = n - 2 >= S->d0_layer && fe >= S->c_pt * S->froerr0 * sh.fe2[lane];
     if (fired) {
@@ -543,14 +606,16 @@ __device__ void decide_replay(State* S, State* G, const DecideShared& sh, int mo
     } else {
       S->cur1[lane] ^= 1;
       S->s1_fro2[lane] = sh.sums[1 + lane][kQFroNew];
+      root = sh.roots[1 + lane][kQFroNew];
       S->s1_exp_cur[lane] = S->s1_exp_next[lane];
     }
   }
+  if (lane < k && conv) root = sqrt(S->s1_fro2[lane]);
   if (lane == 0) S->rp_layers = n;
   const bool all1 = __all_sync(0xffffffffu, conv);
   if (all1) return decide_end(S, lane, DMPT_OK);
   if (n + 1 > S->max_layers) return decide_end(S, lane, DMPT_ENOTCONV);
-  plan_replay(S, G, sh, n + 1, lane, conv);
+  plan_replay(S, G, sh, n + 1, lane, conv, root);
 }
 
 // Adjoint of the S0 recursion, run backwards over the stored states (lane 0).
@@ -616,16 +681,17 @@ __device__ void decide_init(State* S, State* G, const DecideShared& sh, int lane
     S->layers_run = 0;
     S->froerr0 = 0.0;
   }
+  double root = 0.0;
   if (lane < S->k) {
     S->cur1[lane] = 0;
     S->d1_conv[lane] = 0;
     S->d1_layer[lane] = 0;
-    const double f = sh.sums[1 + lane][kQFroNew];
-    S->s1_fro2[lane] = f;
-    S->s1_exp_cur[lane] = S->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(sqrt(f)) : 0;
+    S->s1_fro2[lane] = sh.sums[1 + lane][kQFroNew];
+    root = sh.roots[1 + lane][kQFroNew];
+    S->s1_exp_cur[lane] = S->precision == DMPT_DUAL_FP16 ? fp16_exponent_for(root) : 0;
   }
   __syncwarp();
-  plan_layer(S, G, sh, 1, lane, false);
+  plan_layer(S, G, sh, 1, lane, false, root);
 }
 
 // A layer product has finished: apply its results (one warp).
@@ -639,6 +705,7 @@ __device__ void decide_layer(State* S, State* G, const DecideShared& sh, int lan
   if (S->timeout_flag) return decide_end(S, lane, DMPT_ETIMEOUT);
   if (bad) return decide_end(S, lane, DMPT_ENUMERIC);
   bool conv = lane < k ? S->d1_conv[lane] != 0 : true;
+  double root = 0.0;   // sqrt(s1_fro2) of this lane's slot
   if (square && lane == 0) {
     if (wrote) {
       S->NS = sh.sums[0][kQTrace];    // Tr S_n      (N_S of Alg. 2)
@@ -654,12 +721,12 @@ __device__ void decide_layer(State* S, State* G, const DecideShared& sh, int lan
         S->z0_next = zslice(S->cur0 ^ 1, 0, 0, S->layout_k);
       }
     } else {
-      S->froerr0 = sqrt(sh.sums[0][kQFroDiff]);  // FroErr^(0) of Alg. 2
+      S->froerr0 = sh.roots[0][kQFroDiff];  // FroErr^(0) of Alg. 2
     }
   }
   __syncwarp();
   if (ran) {
-    const double fe = sqrt(sh.sums[1 + lane][kQFroDiff]);  // FroErr^(1)_n of Alg. 3
+    const double fe = sh.roots[1 + lane][kQFroDiff];  // FroErr^(1)_n of Alg. 3
     G->froerr1[lane][n] = fe;
     bool fired = false;
     if (d0 && n - 2 >= S->d0_layer) fired = fe >= S->c_pt * S->froerr0 * sh.fe2[lane];
@@ -670,9 +737,11 @@ __device__ void decide_layer(State* S, State* G, const DecideShared& sh, int lan
     } else {
       S->cur1[lane] ^= 1;
       S->s1_fro2[lane] = sh.sums[1 + lane][kQFroNew];
+      root = sh.roots[1 + lane][kQFroNew];
       S->s1_exp_cur[lane] = S->s1_exp_next[lane];
     }
   }
+  if (lane < k && conv) root = sqrt(S->s1_fro2[lane]);
   if (lane == 0) S->layers_run = n;
   const bool all1 = __all_sync(0xffffffffu, conv);
   const bool end = d0 && all1, cap = n + 1 > S->max_layers;
@@ -680,11 +749,16 @@ __device__ void decide_layer(State* S, State* G, const DecideShared& sh, int lan
     if (lane == 0) S->n_layer = n + 1;
     return decide_end(S, lane, end ? DMPT_OK : DMPT_ENOTCONV);
   }
-  plan_layer(S, G, sh, n + 1, lane, conv);
+  plan_layer(S, G, sh, n + 1, lane, conv, root);
 }
 
 // The decide step of one instance, run by one block of kDecideThreads
 // threads.  jobs: 1 + the response slots of the partials array.
+// Pdl: launched while the layer product may still run.  That product writes
+// nothing of the control block but timeout_flag (and round_ctr, reset here),
+// and it started after the previous decide step had finished, so the rest of
+// the block is read before pdl_wait().
+template <bool Pdl>
 __device__ void decide_body(State* st, const double* partials, int64_t ptiles,
                             int64_t entries, int jobs, int mode, DecideShared& sh) {
   const int tid = threadIdx.x, lane = tid & 31;
@@ -693,51 +767,56 @@ __device__ void decide_body(State* st, const double* partials, int64_t ptiles,
     // the history entries the tests read, fetched while the sums are formed
     const bool adj = mode == kDecideAdjInit || mode == kDecideAdjLayer || mode == kDecideAdjResume;
     const bool fresh = mode == kDecideInit || mode == kDecideReplayInit;
-    const int n = fresh ? 0 : st->n_layer;   // the layer that has run
-    if (lane < kMaxK && !adj && n >= 2) sh.fe2[lane] = st->froerr1[lane][n - 2];
-    if (lane == 8 && !adj && n >= 1) sh.iderr1 = st->iderr[n - 1];
-    if (lane == 9 && !adj) sh.sig0 = st->sigma[n];
-    if (lane == 10 && !adj && n >= 1) sh.sig1 = st->sigma[n - 1];
+    const int n = fresh ? 0 : __ldcg(&st->n_layer);   // the layer that has run
+    if (lane < kMaxK && !adj && n >= 2) sh.fe2[lane] = __ldcg(&st->froerr1[lane][n - 2]);
+    if (lane == 8 && !adj && n >= 1) sh.iderr1 = __ldcg(&st->iderr[n - 1]);
+    if (lane == 9 && !adj) sh.sig0 = __ldcg(&st->sigma[n]);
+    if (lane == 10 && !adj && n >= 1) sh.sig1 = __ldcg(&st->sigma[n - 1]);
     if (lane == 11) {
       int m = n + 1;
       if (adj)
-        m = mode == kDecideAdjInit ? st->d0_updates
-                                   : (mode == kDecideAdjLayer ? st->adj_m - 1 : st->adj_m);
-      sh.sig_next = m >= 0 && m <= kMaxL ? st->sigma[m] : 0;
+        m = mode == kDecideAdjInit
+                ? __ldcg(&st->d0_updates)
+                : __ldcg(&st->adj_m) - (mode == kDecideAdjLayer ? 1 : 0);
+      sh.sig_next = m >= 0 && m <= kMaxL ? __ldcg(&st->sigma[m]) : 0;
     }
   }
-  // per job: 256 strided sums, then the fixed binary tree over them (pairs
-  // 128, 64, ... 1 apart), one warp per quantity
-  const int grp = tid >> 8, t = tid & 255;
+  if constexpr (Pdl) {
+    pdl_wait();
+    constexpr int kTimeoutWord = (int)(offsetof(State, timeout_flag) / sizeof(unsigned));
+    if (tid == kTimeoutWord) sh.head[tid] = __ldcg(reinterpret_cast<const unsigned*>(st) + tid);
+  }
+  // Sums of the partials, four jobs at once, in a fixed order: lane 4 u + q of
+  // warp w of a job adds quantity q of the entries 8 w + u (mod 64), three
+  // shuffles add a warp's eight, and one warp adds the job's eight warps and
+  // takes the square roots.  The part runs two FP64 operations per clock and
+  // SM, so a warp's addition holds the pipe for 16 clocks: their number counts.
+  const int grp = tid >> 8, w = (tid >> 5) & 7, q = lane & 3;
   for (int j0 = 0; j0 < jobs; j0 += kDecideThreads / 256) {
     const int job = j0 + grp;
-    double v[kNQ] = {0.0, 0.0, 0.0, 0.0};
     if (job < jobs) {
-      for (int64_t e = t; e < entries; e += 256) {
-        const double2* p =
-            reinterpret_cast<const double2*>(partials + ((size_t)job * ptiles + e) * kNQ);
-        const double2 a = __ldcg(p), b = __ldcg(p + 1);
-        v[0] += a.x;
-        v[1] += a.y;
-        v[2] += b.x;
-        v[3] += b.y;
+      double v = 0.0;
+      const double* p = partials + ((size_t)job * ptiles + 8 * w + (lane >> 2)) * kNQ + q;
+#pragma unroll 4
+      for (int64_t e = 8 * w + (lane >> 2); e < entries; e += 64, p += 64 * kNQ) v += __ldcg(p);
+      if (8 * w < entries) {
+#pragma unroll
+        for (int o = 16; o >= 4; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      }
+      if (lane < 4) sh.red[grp][w][lane] = v;
+    }
+    __syncthreads();
+    if (job < jobs && w == 0) {
+      double x = sh.red[grp][lane >> 2][q];
+#pragma unroll
+      for (int o = 16; o >= 4; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane < 4) {
+        sh.sums[job][lane] = x;
+        sh.roots[job][lane] = sqrt(x);
       }
     }
-    if (j0 > 0) __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kNQ; ++q) sh.red[grp][q][t] = v[q];
     __syncthreads();
-    if (job < jobs && t < 32 * kNQ) {
-      const double* r = sh.red[grp][t >> 5];
-      const double a0 = r[lane] + r[lane + 128], a2 = r[lane + 64] + r[lane + 192];
-      const double a1 = r[lane + 32] + r[lane + 160], a3 = r[lane + 96] + r[lane + 224];
-      double x = (a0 + a2) + (a1 + a3);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-      if (lane == 0) sh.sums[job][t >> 5] = x;
-    }
   }
-  __syncthreads();
   State* S = reinterpret_cast<State*>(sh.head);   // only the fields before the histories
   if (tid < 32) {
     if (lane == 0) {
@@ -765,8 +844,7 @@ __global__ void __launch_bounds__(kDecideThreads)
                   int jobs, int mode, volatile unsigned* progress, unsigned code) {
   __shared__ DecideShared sh;
   pdl_launch();
-  pdl_wait();
-  decide_body(st, partials, ptiles, entries, jobs, mode, sh);
+  decide_body<true>(st, partials, ptiles, entries, jobs, mode, sh);
   if (progress && threadIdx.x == 0)
     *progress = code | (reinterpret_cast<const State*>(sh.head)->done ? 1u : 0u);
 }
@@ -785,7 +863,7 @@ __global__ void __launch_bounds__(kDecideThreads)
     if (threadIdx.x == 0 && !a.st->done) a.st->timeout_flag = 1;
     __syncthreads();
   }
-  decide_body(a.st, a.partials, a.ptiles, a.entries, a.jobs, kDecideLayer, sh);
+  decide_body<false>(a.st, a.partials, a.ptiles, a.entries, a.jobs, kDecideLayer, sh);
 }
 
 cudaError_t launch_decide_group(const GroupDecide* args, int count, const int* group_timeout,
@@ -1402,7 +1480,7 @@ __device__ __forceinline__ unsigned short bits16(__nv_bfloat16 x) {
 template <typename H16>
 __device__ __forceinline__ void split4(const float* __restrict__ src, unsigned short* hi,
                                        unsigned short* lo, size_t idx, int e) {
-  const float4 v = *reinterpret_cast<const float4*>(src + idx);
+  const float4 v = __ldcg(reinterpret_cast<const float4*>(src + idx));
   const float x[4] = {ldexpf(v.x, e), ldexpf(v.y, e), ldexpf(v.z, e), ldexpf(v.w, e)};
   unsigned short hb[4], lb[4];
 #pragma unroll
@@ -1420,6 +1498,8 @@ __device__ __forceinline__ void split4(const float* __restrict__ src, unsigned s
 template <typename H16>
 __global__ void split_kernel(const State* st, const float* __restrict__ master,
                              unsigned short* ops, int64_t Np, int k, int first_job) {
+  pdl_wait();
+  pdl_launch();
   const size_t mat = (size_t)Np * Np;   // a multiple of 4
   const int m = first_job + blockIdx.y;  // matrix: 0 = S0, 1 + j = S1_j
   const int cur = m == 0 ? st->cur0 : st->cur1[m - 1];
@@ -1436,16 +1516,12 @@ __global__ void split_kernel(const State* st, const float* __restrict__ master,
 cudaError_t launch_split(const Layout& L, void* ws, int first_job, cudaStream_t s, int jobs) {
   char* base = (char*)ws;
   const State* st = (const State*)(base + L.off_state);
-  dim3 grid(152 * 4, jobs < 0 ? 1 + L.k - first_job : jobs);
-  if (L.precision == DMPT_DUAL_FP16)
-    split_kernel<__half><<<grid, 256, 0, s>>>(st, (const float*)(base + L.off_master),
-                                              (unsigned short*)(base + L.off_ops16), L.Np, L.k,
-                                              first_job);
-  else
-    split_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(st, (const float*)(base + L.off_master),
-                                                     (unsigned short*)(base + L.off_ops16),
-                                                     L.Np, L.k, first_job);
-  return cudaGetLastError();
+  const int64_t bx = L.Np * L.Np / 1024;   // 4 elements per thread
+  const dim3 grid((unsigned)(bx < 152 * 4 ? bx : 152 * 4), jobs < 0 ? 1 + L.k - first_job : jobs);
+  return launch_pdl(L.precision == DMPT_DUAL_FP16 ? split_kernel<__half>
+                                                  : split_kernel<__nv_bfloat16>,
+                    grid, dim3(256), 0, s, st, (const float*)(base + L.off_master),
+                    (unsigned short*)(base + L.off_ops16), L.Np, L.k, first_job);
 }
 
 // ---------------------------------------------------------------------------
@@ -1466,7 +1542,7 @@ __device__ __forceinline__ void sym_tile(const T* __restrict__ src, int64_t Np, 
   const int64_t lr = TS * (bi > bj ? bi : bj), lc = TS * (bi > bj ? bj : bi);
   T v[RPT];
 #pragma unroll
-  for (int j = 0; j < RPT; ++j) v[j] = src[(lr + ty + RS * j) * Np + lc + tx];
+  for (int j = 0; j < RPT; ++j) v[j] = __ldcg(&src[(lr + ty + RS * j) * Np + lc + tx]);
 #pragma unroll
   for (int j = 0; j < RPT; ++j) t[ty + RS * j][tx] = v[j];
   __syncthreads();
@@ -1731,6 +1807,8 @@ __global__ void __launch_bounds__(256) finalize_kernel(const State* st,
   __shared__ T t[kSymTile][kSymTile + 1];
   const size_t mat = (size_t)Np * Np;
   const int y = blockIdx.y;
+  pdl_wait();
+  pdl_launch();
   if (y == 0 && P == nullptr) return;
   const int m = y == 0 ? 0 : slot0 + y - 1;
   const int cur = m == 0 ? st->cur0 : st->cur1[m - 1];
@@ -1748,14 +1826,13 @@ cudaError_t launch_finalize(const Layout& L, void* ws, double* P, double* P1, in
                             int k_out, cudaStream_t s, int slot0) {
   char* base = (char*)ws;
   const State* st = (const State*)(base + L.off_state);
-  dim3 grid(152 * 16, 1 + k_out);
+  const int64_t tb = (L.n + kSymTile - 1) / kSymTile;
+  const dim3 grid((unsigned)(tb * tb < 152 * 16 ? tb * tb : 152 * 16), 1 + k_out);
   if (L.precision == DMPT_FP64)
-    finalize_kernel<double><<<grid, 256, 0, s>>>(st, (const double*)(base + L.off_master), P,
-                                                 P1, L.n, L.Np, ld, L.k, slot0);
-  else
-    finalize_kernel<float><<<grid, 256, 0, s>>>(st, (const float*)(base + L.off_master), P, P1,
-                                                L.n, L.Np, ld, L.k, slot0);
-  return cudaGetLastError();
+    return launch_pdl(finalize_kernel<double>, grid, dim3(256), 0, s, st,
+                      (const double*)(base + L.off_master), P, P1, L.n, L.Np, ld, L.k, slot0);
+  return launch_pdl(finalize_kernel<float>, grid, dim3(256), 0, s, st,
+                    (const float*)(base + L.off_master), P, P1, L.n, L.Np, ld, L.k, slot0);
 }
 
 // n_occ = 0 (full = 0) or n_occ = n (full = 1): P = 0 or I, P1 = 0.
@@ -1914,7 +1991,7 @@ __global__ void __launch_bounds__(kDecideThreads)
     batch_decide_init_kernel(const BatchInst* __restrict__ bi) {
   __shared__ DecideShared sh;
   const BatchInst& b = bi[blockIdx.x];
-  decide_body(b.st, b.partials, b.ptiles, kInitBlocks, 1 + b.k, kDecideInit, sh);
+  decide_body<false>(b.st, b.partials, b.ptiles, kInitBlocks, 1 + b.k, kDecideInit, sh);
 }
 
 // 16-bit split of matrices 0 .. layout k (as split_kernel), kBatchChunk
