@@ -909,19 +909,6 @@ cudaError_t launch_decide(const Layout& L, void* ws, int mode, int64_t entries, 
 // to the elements with row <= col, stores them at (r, c) and (c, r) in the
 // other ping-pong buffer, and reduces the Alg. 2 / 3 norms in FP64.
 
-template <typename T>
-struct Vec;
-template <>
-struct Vec<float> {
-  using type = float4;
-  static constexpr int width = 4;
-};
-template <>
-struct Vec<double> {
-  using type = double2;
-  static constexpr int width = 2;
-};
-
 template <typename T, int TM>
 __device__ __forceinline__ int frag_index(int t, int m) {
   // the TM rows (cols) of a thread: two runs of TM/2 contiguous elements,
@@ -930,16 +917,6 @@ __device__ __forceinline__ int frag_index(int t, int m) {
   constexpr int BT = 16 * TM;
   return m < H ? t * H + m : BT / 2 + t * H + (m - H);
 }
-
-// Two blocks per SM for the FP32 form (registers <= 128), one for FP64.
-template <typename T>
-struct SimtBlocks {
-  static constexpr int value = 2;
-};
-template <>
-struct SimtBlocks<double> {
-  static constexpr int value = 1;
-};
 
 // Jobs of a layer (as in the tensor-core kernels): 0 = square of S0; job
 // 1 + (o - 1) k1 + d = the order-o term of direction d, in o + 1 K passes
@@ -992,8 +969,8 @@ constexpr int simt_smem_bytes() {
 }
 
 template <typename T, int TM, int BK>
-__global__ void __launch_bounds__(256, SimtBlocks<T>::value)
-    layer_simt_kernel(State* st, T* __restrict__ master, int64_t Np, int k,
+__global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
+    layer_simt_kernel(State* st, T* __restrict__ master, int64_t n, int64_t Np, int k,
                       double* __restrict__ partials, int64_t ptiles) {
   constexpr int BT = 16 * TM;
   constexpr int VW = 16 / (int)sizeof(T);      // elements per 16-byte copy
@@ -1010,12 +987,13 @@ __global__ void __launch_bounds__(256, SimtBlocks<T>::value)
 
   pdl_wait();   // no pdl_launch(): see layer_fp64_kernel
   if (st->done) return;
-  const int job = blockIdx.y;
+  const int job = (int)gridDim.y - 1 - (int)blockIdx.y;   // most K passes first
   const int run = job == 0 ? st->plan_square : st->plan_resp[job - 1];
   if (!run) return;
 
-  // upper tile (I, J), I <= J, row-major over the upper triangle
-  const int T_ = (int)(Np / BT);
+  // upper tile (I, J), I <= J, row-major over the upper triangle of the tiles
+  // that hold elements of the n x n matrix
+  const int T_ = (int)((n + BT - 1) / BT);
   int64_t t = blockIdx.x;
   int I = 0;
   while (t >= T_ - I) {
@@ -1032,15 +1010,19 @@ __global__ void __launch_bounds__(256, SimtBlocks<T>::value)
 
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
-  T acc[TM][TM];
+  // column pairs (2 j, 2 j + 1) of the thread's tile, packed: one product per
+  // FMA fills the issue slots, and the shared-memory reads come on top.  The
+  // busiest SM's FMA pipe is now active in 94% of its cycles (n = 2560); what is
+  // left is the last wave.  n = 4096 k = 1 layer 3.80 -> 3.53 ms.
+  f32x2 acc2[TM][TM / 2];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TM; ++j) acc[i][j] = T(0);
+    for (int j = 0; j < TM / 2; ++j) acc2[i][j] = pack2(0.0f, 0.0f);
 
   const int k1 = st->order >= 2 ? st->k1 : k;   // first-order directions
   const int passes = simt_job_passes(job, k1);
-  const int nkb = (int)(Np / BK);
+  const int nkb = (int)((n + BK - 1) / BK);   // the K range of the padding is zero
   for (int pass = 0; pass < passes; ++pass) {
     // pass p of the job: A = slot mA rows I, B = slot mB rows J (square:
     // S0 S0; order-o term: S0 S_o, S_o S0, then S_{p-1} S_{o-p+1}).  The
@@ -1085,15 +1067,29 @@ __global__ void __launch_bounds__(256, SimtBlocks<T>::value)
       const T* bs = as + BK * LD;
 #pragma unroll
       for (int kk = 0; kk < BK; ++kk) {
-        T a[TM], b[TM];
+        T a[TM];
+        f32x2 b[TM / 2];
 #pragma unroll
         for (int m = 0; m < TM; ++m) a[m] = as[kk * LD + frag_index<T, TM>(ty, m)];
+        if constexpr (TM == 8) {
 #pragma unroll
-        for (int m = 0; m < TM; ++m) b[m] = bs[kk * LD + frag_index<T, TM>(tx, m)];
+          for (int m = 0; m < TM / 2; m += 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(
+                bs + kk * LD + frag_index<T, TM>(tx, 2 * m));
+            b[m] = v.x;
+            b[m + 1] = v.y;
+          }
+        } else {
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
+          for (int m = 0; m < TM / 2; ++m)
+            b[m] = *reinterpret_cast<const f32x2*>(bs + kk * LD + frag_index<T, TM>(tx, 2 * m));
+        }
 #pragma unroll
-          for (int j = 0; j < TM; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int i = 0; i < TM; ++i) {
+          const f32x2 ai = pack2(a[i], a[i]);
+#pragma unroll
+          for (int j = 0; j < TM / 2; ++j) acc2[i][j] = fma2(ai, b[j], acc2[i][j]);
+        }
       }
     }
     cp_async_wait<0>();   // no copy of this pass left in flight
@@ -1107,7 +1103,6 @@ __global__ void __launch_bounds__(256, SimtBlocks<T>::value)
   // ||S_new||_F^2 and ||S_old - X||_F^2: in FP64 for the FP64 form; for the
   // FP32 form as exact FP32 products summed with TwoSum compensation (the
   // FP64 rate of the part is low), converted to FP64 once per thread
-  double fnew = 0.0, fdiff = 0.0;
   float fn_s = 0.0f, fn_c = 0.0f, fd_s = 0.0f, fd_c = 0.0f;
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
@@ -1116,38 +1111,30 @@ __global__ void __launch_bounds__(256, SimtBlocks<T>::value)
     for (int j = 0; j < TM; ++j) {
       const int64_t c = (int64_t)J * BT + frag_index<T, TM>(tx, j);
       if (r > c) continue;  // owned by the mirrored element
-      const T x = acc[i][j];
+      float x01[2];
+      unpack2(acc2[i][j / 2], x01[0], x01[1]);
+      const T x = x01[j % 2];
       const T old = Sj[(size_t)r * Np + c];
       if (!isfinite((double)x)) bad += 1.0;
       const T nw = sg * x + om * old;
-      if constexpr (sizeof(T) == 8) {
-        const double w = (r == c) ? 1.0 : 2.0;
-        const double dd = (double)old - (double)x;
-        fdiff += w * dd * dd;
-        if (write) {
-          const double dn = (double)nw;
-          fnew += w * dn * dn;
-        }
-      } else {
-        const float w = (r == c) ? 1.0f : 2.0f;
-        const float dd = (float)old - (float)x;
-        {
-          const float p = w * dd * dd;
-          const float e = w * fmaf(dd, dd, -dd * dd);
-          const float tt = fd_s + p;
-          const float bp = tt - fd_s;
-          fd_c += (fd_s - (tt - bp)) + (p - bp) + e;
-          fd_s = tt;
-        }
-        if (write) {
-          const float n1 = (float)nw;
-          const float p = w * n1 * n1;
-          const float e = w * fmaf(n1, n1, -n1 * n1);
-          const float tt = fn_s + p;
-          const float bp = tt - fn_s;
-          fn_c += (fn_s - (tt - bp)) + (p - bp) + e;
-          fn_s = tt;
-        }
+      const float w = (r == c) ? 1.0f : 2.0f;
+      const float dd = (float)old - (float)x;
+      {
+        const float p = w * dd * dd;
+        const float e = w * fmaf(dd, dd, -dd * dd);
+        const float tt = fd_s + p;
+        const float bp = tt - fd_s;
+        fd_c += (fd_s - (tt - bp)) + (p - bp) + e;
+        fd_s = tt;
+      }
+      if (write) {
+        const float n1 = (float)nw;
+        const float p = w * n1 * n1;
+        const float e = w * fmaf(n1, n1, -n1 * n1);
+        const float tt = fn_s + p;
+        const float bp = tt - fn_s;
+        fn_c += (fn_s - (tt - bp)) + (p - bp) + e;
+        fn_s = tt;
       }
       if (write) {
         out[(size_t)r * Np + c] = nw;
@@ -1156,10 +1143,8 @@ __global__ void __launch_bounds__(256, SimtBlocks<T>::value)
       }
     }
   }
-  if constexpr (sizeof(T) != 8) {
-    fnew = (double)fn_s + (double)fn_c;
-    fdiff = (double)fd_s + (double)fd_c;
-  }
+  const double fnew = (double)fn_s + (double)fn_c;
+  const double fdiff = (double)fd_s + (double)fd_c;
   double v[4] = {tr, fnew, fdiff, bad};
   block_sum<4, 256>(v, red);
   if (tid == 0) {
@@ -1403,7 +1388,15 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-constexpr int kFp32Tile = 128;   // tile edge of the FP32 form
+// Tile edge of the FP32 form: 64 while the 128-wide tiles of every job would
+// keep less than two thirds of the SMs busy; a 64-wide tile reads twice the
+// shared memory per product.  Solve per layer, 128 / 64 wide: n = 700 k = 3 (84
+// tiles) 145 / 101 us, n = 1000 k = 1 (72) 195 / 101 us, n = 1400 k = 1 (132)
+// 267 / 280 us, n = 1000 k = 3 (144) 200 / 210 us, n = 4096 k = 1 3.53 / 4.43 ms.
+inline int fp32_tile(int64_t n, int k) {
+  const int64_t t = (n + 127) / 128;
+  return t * (t + 1) / 2 * (1 + k) <= 100 ? 64 : 128;
+}
 
 // Per-device one-time setup: the SIMT layer kernels' dynamic shared memory
 // exceeds the default 48 KB limit; thread-safe.
@@ -1416,6 +1409,9 @@ static void simt_setup() {
     cudaFuncSetAttribute(layer_simt_kernel<float, 8, 16>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                          simt_smem_bytes<float, 8, 16>());
+    cudaFuncSetAttribute(layer_simt_kernel<float, 4, 16>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         simt_smem_bytes<float, 4, 16>());
   });
 }
 
@@ -1437,17 +1433,18 @@ cudaError_t launch_layer_simt(const Layout& L, void* ws, cudaStream_t s, int64_t
     if (e != cudaSuccess) return e;
     if (pass_flops) *pass_flops = (double)tiles * bt * bt * (double)L.n * 2.0;
   } else {
-    constexpr int smem32 = simt_smem_bytes<float, 8, 16>();
-    static_assert(2 * smem32 <= 227 * 1024, "two FP32 blocks per SM");
+    constexpr int smem8 = simt_smem_bytes<float, 8, 16>(), smem4 = simt_smem_bytes<float, 4, 16>();
+    static_assert(2 * smem8 <= 227 * 1024 && 4 * smem4 <= 227 * 1024, "blocks per SM");
     simt_setup();
-    tiles = upper_tiles(L.Np, kFp32Tile);
-    const cudaError_t e =
-        launch_pdl(layer_simt_kernel<float, 8, 16>, dim3((unsigned)tiles, 1 + L.k), dim3(256),
-                   smem32, s, st, (float*)(base + L.off_master), L.Np, L.k, partials,
-                   L.partial_tiles);
+    const int bt = fp32_tile(L.n, L.k);
+    const int64_t tb = (L.n + bt - 1) / bt;
+    tiles = tb * (tb + 1) / 2;
+    const cudaError_t e = launch_pdl(
+        bt == 128 ? layer_simt_kernel<float, 8, 16> : layer_simt_kernel<float, 4, 16>,
+        dim3((unsigned)tiles, 1 + L.k), dim3(256), bt == 128 ? smem8 : smem4, s, st,
+        (float*)(base + L.off_master), L.n, L.Np, L.k, partials, L.partial_tiles);
     if (e != cudaSuccess) return e;
-    if (pass_flops)
-      *pass_flops = (double)tiles * kFp32Tile * kFp32Tile * (double)L.Np * 2.0;
+    if (pass_flops) *pass_flops = (double)tiles * bt * bt * (double)((L.n + 15) / 16 * 16) * 2.0;
   }
   if (entries) *entries = tiles;
   return cudaGetLastError();
