@@ -387,6 +387,17 @@ __device__ __forceinline__ float cross_unscale(const State* st, int job, int pas
 // chunks keep the boundaries they have over all Np / 32 blocks, so results do
 // not change: a backwards sweep starts `kchunk0` stages into its first chunk.
 __host__ __device__ __forceinline__ int k_blocks(int64_t n) { return (int)((n + BK - 1) / BK); }
+
+// Columns of a tile (width nt, from column c) left of cend = 32 k_blocks(n).
+// Columns and rows from cend on are neither computed nor stored: as K range
+// they are left out, and as rows of a tile they only reach elements that are
+// left out as well, so they may hold anything.  The tiles of the last column
+// block shrink their MMAs' N to what is left: n = 5904 (32 of 256 columns in 24
+// of 300 tiles) 53.3 -> 52.5 ms, 32 uneven instances 18.3 -> 17.2 ms.
+__host__ __device__ __forceinline__ int tile_cols(int c, int nt, int cend) {
+  const int w = cend - c;
+  return w < 0 ? 0 : (w < nt ? w : nt);
+}
 __device__ __forceinline__ int kchunk0(int64_t Np, int kblocks, int chunk, bool rev) {
   return rev ? ((int)(Np / BK) - kblocks) % chunk : 0;
 }
@@ -471,6 +482,12 @@ __device__ __forceinline__ void store32(void* p, const uint32_t (&v)[8]) {
 __device__ __forceinline__ int epi_first_group(int r0, int c0) {
   return r0 > c0 ? (r0 - c0) >> 4 : 0;
 }
+// Groups of a warp's columns from c0 that lie left of column cend.
+template <int NG>
+__device__ __forceinline__ int epi_groups(int c0, int cend) {
+  const int g = (cend - c0) >> 4;
+  return g < NG ? g : NG;
+}
 __device__ __forceinline__ void epi_load_old(float (&olds)[16], const float* Sc, int np, int g16) {
 #pragma unroll
   for (int q = 0; q < 16; ++q) olds[q] = __ldcg(Sc + (16 * g16 + q) * np);
@@ -489,13 +506,14 @@ template <class CV, int NG, bool PRE, class Rel>
 __device__ __forceinline__ void rolled_tile_epilogue(
     const uint32_t ta_sum, const float* __restrict__ Sold, float* Snew, typename CV::T* hi_new,
     typename CV::T* lo_new, const int lane, const int64_t Np, const int r, const int c0,
-    const float sg, const float om, const float scale_new, const bool write, float (&olds)[16],
-    uint16_t* dbuf, TileSums& ts, Rel release) {
+    const int cend, const float sg, const float om, const float scale_new, const bool write,
+    float (&olds)[16], uint16_t* dbuf, TileSums& ts, Rel release) {
   const int r0 = r - lane;   // row of lane 0
   const int np = (int)Np;
   // groups below the warp's rows come first, groups above them last
   int g16 = epi_first_group(r0, c0);
-  if (g16 >= NG) {
+  const int ng = epi_groups<NG>(c0, cend);
+  if (g16 >= ng) {
     release();
     return;
   }
@@ -519,10 +537,10 @@ __device__ __forceinline__ void rolled_tile_epilogue(
   f32x2 fs = zero2, fc = zero2, fd = zero2, z = zero2;
   if constexpr (!PRE) epi_load_old(olds, Sc, np, g16);
 #pragma unroll 1
-  for (; g16 < NG; ++g16) {
+  for (; g16 < ng; ++g16) {
     uint32_t xs[16];
     tmem_ld16(ta_sum + 16 * g16, xs);
-    if (g16 == NG - 1) release();
+    if (g16 == ng - 1) release();
     const int d = c0 + 16 * g16 - r0;   // < 32: a group on the diagonal
     if (d < 32) {
       // elements below the diagonal belong to their mirror elements; the one on
@@ -633,7 +651,7 @@ __device__ __forceinline__ void rolled_tile_epilogue(
         }
       }
     }
-    if (g16 < NG - 1) epi_load_old(olds, Sc, np, g16 + 1);
+    if (g16 < ng - 1) epi_load_old(olds, Sc, np, g16 + 1);
   }
   float a0, a1, b0, b1;
   unpack2(fs, a0, a1);
@@ -980,8 +998,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tempty + 8 * ab);
       };
-      rolled_tile_epilogue<CV, 8, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
-                                   scale_new, write, olds, epi_block(red), ts, release);
+      rolled_tile_epilogue<CV, 8, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0,
+                                         kblocks * BK, sg, om, scale_new, write, olds, epi_block(red), ts, release);
       if (++ab == 2) {
         ab = 0;
         abphase ^= 1;
@@ -1208,8 +1226,8 @@ __device__ __forceinline__ void producer_drain(RingPos rg, int stages, uint32_t 
 // block of 32 the three products hi*hi, hi*lo, lo*hi for two K16 steps into
 // the current accumulation chunk; a chunk ends every `chunk` blocks and at the
 // end of each K pass (so chunks never straddle a pass), the first of a pass
-// after chunk - cp0 blocks, and is then published to both CTAs.  False when a
-// bounded wait expired.
+// after chunk - cp0 blocks, and is then published to both CTAs.  cols: the
+// tile's columns (a multiple of 32).  False when a bounded wait expired.
 //
 // The whole warp runs the loop and one elected lane issues: what bounds a
 // narrow tile is the issue of its MMAs, and with the loop under `lane == 0`
@@ -1218,13 +1236,13 @@ __device__ __forceinline__ void producer_drain(RingPos rg, int stages, uint32_t 
 // each.
 template <bool BF16, int NT>
 __device__ __forceinline__ bool mma_item(RingPos& rg, RingPos& tb, int passes, int kblocks,
-                                         int chunk, int cp0, bool rev, uint32_t tmem_base,
-                                         uint32_t ring, uint32_t bar_full, uint32_t bar_empty,
+                                         int chunk, int cp0, bool rev, int cols,
+                                         uint32_t tmem_base, uint32_t ring, uint32_t bar_full, uint32_t bar_empty,
                                          uint32_t bar_tfull, uint32_t bar_tempty,
                                          uint64_t limit_ns, volatile int* abort_flag,
                                          int* timeout_global) {
   using PT = PairTile<NT>;
-  constexpr uint32_t idesc = make_idesc_m256(BF16 ? 1 : 0, NT);
+  const uint32_t idesc = make_idesc_m256(BF16 ? 1 : 0, cols);
   constexpr int H = PT::SK / BK;   // blocks per stage
   const int nst = (kblocks + H - 1) / H;
   for (int pass = 0; pass < passes; ++pass) {
@@ -1406,6 +1424,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const unsigned tiles = (unsigned)num_pair_tiles(Np);
   const unsigned items = SP * tiles * (unsigned)njobs;
   const int kblocks = k_blocks(st->n);
+  const int cend = kblocks * BK;
 
   int* timeout_global = &gst->timeout_flag;
 
@@ -1437,9 +1456,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         const int job = job_at(jmask, (int)(it / tiles));
         int I2, J;
         pair_tile_banded(it % tiles, (int)(Np / BN), band, &I2, &J);
+        const int cb = J * BN + (int)(v % SP) * NT, cols = tile_cols(cb, NT, cend);
+        if (SP > 1 && cols == 0) continue;
         ok = produce_item<NT>(rg, &mapA, &mapB, st, job, job_passes(job, k1), k, k1, cur0, z0c,
-                              I2 * 2 * BM + (int)rank * BM,
-                              J * BN + (int)(v % SP) * NT + (int)rank * PT::B_ROWS, kblocks,
+                              I2 * 2 * BM + (int)rank * BM, cb + (int)rank * (cols / 2), kblocks,
                               item_rev(v), leader, ring, bar_full, bar_empty, lead_full, limit_ns,
                               abort_flag, timeout_global);
       }
@@ -1456,8 +1476,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         if (v < vbase) continue;
         const unsigned it = (v - vbase) / SP;
         const int job = job_at(jmask, (int)(it / tiles));
+        int I2, J;
+        pair_tile_banded(it % tiles, (int)(Np / BN), band, &I2, &J);
+        const int cols = tile_cols(J * BN + (int)(v % SP) * NT, NT, cend);
+        if (SP > 1 && cols == 0) continue;
         ok = mma_item<BF16, NT>(rg, tb, job_passes(job, k1), kblocks, chunk,
-                                kchunk0(Np, kblocks, chunk, item_rev(v)), item_rev(v), tmem_base, ring,
+                                kchunk0(Np, kblocks, chunk, item_rev(v)), item_rev(v), cols,
+                                tmem_base, ring,
                                 bar_full, bar_empty, bar_tfull, bar_tempty, limit_ns, abort_flag,
                                 timeout_global);
       }
@@ -1496,17 +1521,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       // S_old of this thread's first columns: narrow tiles have the registers to
       // read them while the products run
       float olds[16];
-      auto first_old = [&]() {
+      if constexpr (NT < BN) {
         int I2, J;
         pair_tile_banded(it % tiles, (int)(Np / BN), band, &I2, &J);
+        if (tile_cols(J * BN + (int)(v % SP) * NT, NT, cend) == 0) {   // nothing in the matrix
+          tile_sums_out(TileSums(), red, seq++, warp - EPI_WARP0, lane,
+                        partials +
+                            ((size_t)job * ptiles + 2 * (SP * (size_t)(it % tiles) + v % SP) + rank) * kNQ);
+          continue;
+        }
         const int r = I2 * 2 * BM + (int)rank * BM + rloc;
         const int c0 = J * BN + (int)(v % SP) * NT + half * (NT / 2);
         const int g0 = epi_first_group(r - lane, c0);
         const int curj = job == 0 ? cur0 : st->cur1[job - 1];
         const float* Sc = master + (size_t)(curj * (1 + k) + job) * mat + (size_t)c0 * Np + r;
-        if (g0 < NT / 32) epi_load_old(olds, Sc, (int)Np, g0);
-      };
-      if constexpr (NT < BN) first_old();
+        if (g0 < epi_groups<NT / 32>(c0, cend)) epi_load_old(olds, Sc, (int)Np, g0);
+      }
       float sum[NT / 2];
 #pragma unroll
       for (int i = 0; i < NT / 2; ++i) sum[i] = 0.0f;
@@ -1563,8 +1593,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab.idx);
       };
-      rolled_tile_epilogue<CV, NT / 32, NT < BN>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
-                                   scale_new, write, olds, epi_block(red), ts, release);
+      rolled_tile_epilogue<CV, NT / 32, NT < BN>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r,
+                                                 c0, cend, sg, om, scale_new, write, olds, epi_block(red), ts, release);
       ab.next(PT::ACC);
       tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane,
                     partials + ((size_t)job * ptiles + 2 * (SP * (size_t)t + v % SP) + rank) * kNQ);
@@ -1805,8 +1835,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         const State* sti = gi.st;
         int I2, J;
         pair_tile_banded((unsigned)itm.t, (int)(gi.Np / BN), band, &I2, &J);
+        const int cols = tile_cols(J * BN, BN, itm.kblocks * BK);
         ok = produce_item<BN>(rg, &gi.map, &gi.map, sti, itm.job, itm.passes, gi.k, gi.k, sti->cur0,
-                          sti->z0_cur, I2 * 2 * BM + (int)rank * BM, J * BN + (int)rank * BM,
+                          sti->z0_cur, I2 * 2 * BM + (int)rank * BM,
+                          J * BN + (int)rank * (cols / 2),
                           itm.kblocks, itm.rev, leader, ring, bar_full, bar_empty, lead_full,
                           limit_ns, abort_flag, timeout_global);
       }
@@ -1825,7 +1857,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g == kNoItem) break;
         const GroupItem itm = group_item(inst, first, jmask, count, g, k_snake, chunk);
+        int I2, J;
+        pair_tile_banded((unsigned)itm.t, (int)(inst[itm.inst].Np / BN), band, &I2, &J);
         ok = mma_item<BF16, BN>(rg, tb, itm.passes, itm.kblocks, chunk, itm.cp0, itm.rev,
+                                tile_cols(J * BN, BN, itm.kblocks * BK),
                             tmem_base, ring, bar_full, bar_empty, bar_tfull, bar_tempty, limit_ns,
                             abort_flag, timeout_global);
       }
@@ -1935,8 +1970,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab);
       };
-      rolled_tile_epilogue<CV, 8, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
-                                   scale_new, write, olds, epi_block(red), ts, release);
+      rolled_tile_epilogue<CV, 8, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0,
+                                         itm.kblocks * BK, sg, om, scale_new, write, olds, epi_block(red), ts, release);
       if (++ab == 2) {
         ab = 0;
         abphase ^= 1;
@@ -2123,9 +2158,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         const State* sti = gi.st;
         int I2, J;
         tile128_coords(itm.t, gi.Np, &I2, &J);
+        const int cols = tile_cols(J * G_BN, G_BN, itm.kblocks * BK);
         ok = produce_item<G_BN>(rg, &gi.map, &gi.map64, sti, itm.job, itm.passes, gi.k, gi.k,
                                 sti->cur0, sti->z0_cur, I2 * 2 * BM + (int)rank * BM,
-                                J * G_BN + (int)rank * GT::B_ROWS, itm.kblocks, false, leader,
+                                J * G_BN + (int)rank * (cols / 2), itm.kblocks, false, leader,
                                 ring, bar_full, bar_empty, lead_full, limit_ns, abort_flag,
                                 timeout_global);
       }
@@ -2144,7 +2180,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g == kNoItem) break;
         const GroupItem128 itm = group_item128(inst, first, jmask, count, g);
+        int I2, J;
+        tile128_coords(itm.t, inst[itm.inst].Np, &I2, &J);
         ok = mma_item<BF16, G_BN>(rg, tb, itm.passes, itm.kblocks, chunk, 0, false,
+                                  tile_cols(J * G_BN, G_BN, itm.kblocks * BK),
                                   tmem_base, ring, bar_full, bar_empty, bar_tfull, bar_tempty,
                                   limit_ns, abort_flag, timeout_global);
       }
@@ -2252,8 +2291,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       // rows past Np (a 256-row block over a matrix padded to 128): nothing to
       // store; the products there are zeros
       if ((int64_t)row0 < Np)
-        rolled_tile_epilogue<CV, 4, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0, sg, om,
-                                     scale_new, write, olds, epi_block(red), ts, release);
+        rolled_tile_epilogue<CV, 4, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0,
+                                           itm.kblocks * BK, sg, om, scale_new, write, olds, epi_block(red), ts, release);
       else
         release();
       ab.next(GT::ACC);
@@ -2388,7 +2427,11 @@ int tc_tile() { return tc::BN; }
 
 void pair_tile_info(const Layout& L, int64_t* entries, double* pass_flops, bool n128) {
   const int64_t tiles = n128 ? tc::num_tiles128(L.Np) : tc::num_pair_tiles(L.Np);
-  const double cols = n128 ? tc::G_BN : tc::BN;
+  // the last column block's tiles are as wide as what is left of the matrix
+  const int nt = n128 ? tc::G_BN : tc::BN;
+  const int64_t edge = n128 ? (L.Np + 255) / 256 : L.Np / tc::BN;
+  const int cend = tc::k_blocks(L.n) * tc::BK;
+  const double cols = nt - (double)edge / tiles * (L.Np - cend);
   if (entries) *entries = 2 * tiles;
   if (pass_flops) *pass_flops = (double)tiles * 2 * tc::BM * cols * tc::k_blocks(L.n) * tc::BK * 2.0;
 }
@@ -2485,7 +2528,7 @@ cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double ti
         band, inject_stall, round_align);
     if (e != cudaSuccess) return e;
     if (entries) *entries = 2 * split * ptiles;
-    if (pass_flops) *pass_flops = (double)ptiles * 2 * BM * BN * k_blocks(L.n) * BK * 2.0;
+    pair_tile_info(L, nullptr, pass_flops);
     return cudaGetLastError();
   }
   const int64_t tiles = num_tiles(L.Np);

@@ -56,3 +56,23 @@ def test_higher_orders_equal_the_single_cta_kernel(n, order, k):
     assert torch.equal(P, Pc)
     for a, b in zip(terms, termsc):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n,k,opts", [
+    (65, 2, {}), (257, 1, {}), (1000, 2, {}), (1281, 3, {}), (2081, 2, {}),
+    (300, 1, dict(cta_pair=0)), (1281, 1, dict(cta_pair=0)), (700, 1, dict(precision="dual_bf16")),
+])
+def test_padding_of_the_workspace_may_hold_anything(n, k, opts):
+    """Elements past the last K block are neither computed nor read as data."""
+    ctx = dmpt.context(0)
+    H, H1, n_occ = instance(n, k)
+    prec = dict(precision=opts["precision"]) if "precision" in opts else {}
+    nbytes = ctx.workspace_size(n, k, dmpt.options(**opts))
+    P, P1, info = ctx.sp2_response(H, H1, n_occ, **opts)
+    for fill in (0xFF, 0x7C):   # NaN in every type; large values
+        ws = torch.full((nbytes + 256,), fill, dtype=torch.uint8, device=DEV)
+        Pw, P1w, infow = ctx.sp2_response(H, H1, n_occ, workspace=ws, **opts)
+        assert infow.converged and infow.layers == info.layers
+        assert torch.equal(P, Pw) and torch.equal(P1, P1w)
+    Pb, P1b, _ = ctx.sp2_response_batch([H, H], [H1, H1], [n_occ, n_occ], **prec)
+    assert torch.equal(Pb[1], P) and torch.equal(P1b[1], P1)
