@@ -76,6 +76,35 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* smem /* NT*NV
 }
 
 // ---------------------------------------------------------------------------
+// Conversions between FP32 and FP64 on the integer pipe.  The part converts two
+// values per clock and SM on its FP64 pipe, which bounded the initial layer (68%
+// of that pipe's peak at n = 4096, 41% of DRAM's) and the outputs; these take
+// about ten integer instructions (outputs n = 5904 k = 1: 503 -> 146 us, initial
+// layer n = 2048 k = 3: 62 -> 46 us).  Subnormal, infinite and NaN values, and
+// results outside the normal FP32 range, take the conversion instruction.
+
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), a = u & 0x7FFFFFFFu;
+  if (a - 0x00800000u < 0x7F000000u)   // normal: rebias the exponent by 1023 - 127
+    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(u << 29));
+  return a == 0u ? __hiloint2double((int)u, 0) : (double)x;
+}
+
+// (float)(x 2^-HALF), rounded to nearest even
+template <int HALF = 0>
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned a = hi & 0x7FFFFFFFu;
+  constexpr unsigned kOne = 0x00100000u;   // one in the exponent
+  if (a - (0x38100000u + HALF * kOne) < 0x0FE00000u) {
+    unsigned m = __funnelshift_l(lo, a - (0x38000000u + HALF * kOne), 3);
+    m += (lo & 0x1FFFFFFFu) + (m & 1u) > 0x10000000u ? 1u : 0u;   // may carry into infinity
+    return __uint_as_float((hi & 0x80000000u) | m);
+  }
+  return (a | lo) == 0u ? __uint_as_float(hi) : (float)(HALF ? 0.5 * x : x);
+}
+
+// ---------------------------------------------------------------------------
 // Gershgorin bounds (Sec. II B; Alg. 1 inputs).  Min / max are taken with
 // 64-bit integer atomics on an order-preserving encoding of the doubles, so
 // the result is independent of the order in which rows finish and the call
@@ -260,7 +289,7 @@ __device__ __forceinline__ void init_body(State* st, T* master, const double* __
         // outside the matrix (h = 0 there)
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
-          const float hw = (float)hv[i] * wf;
+          const float hw = narrow(hv[i]) * wf;
           tile[ty + RS * i][tx] = hole ? hw : -hw;
         }
         // the diagonal element of column tx, formed in FP64 and rounded once
@@ -1702,8 +1731,13 @@ cudaError_t launch_recompute_done(const Layout& L, void* ws, cudaStream_t s) {
 __global__ void __launch_bounds__(256) adj_init_kernel(const double* __restrict__ G, float* master,
                                                        int64_t n, int64_t Np, int64_t ld, int lk,
                                                        double* partials, int64_t ptiles) {
-  __shared__ double up[32][33];
+  // 32 x 32 tile pairs (bi <= bj): the upper tile in registers, the lower one
+  // through shared memory; the mirror tile is the upper one's result transposed.
+  // Two FP64 operations per element of the upper tile (the FP64 rate of the part
+  // is low): the sum and the squared norm, which keeps FP64's range (G may be
+  // tiny or huge).  n = 4096: 245 -> 79 us.
   __shared__ double dn[32][33];
+  __shared__ float sv[32][33];
   __shared__ double red[2 * 256];
   const size_t mat = (size_t)Np * Np;
   float* dst = master + (size_t)1 * mat;   // buffer 0, slot 1
@@ -1711,37 +1745,46 @@ __global__ void __launch_bounds__(256) adj_init_kernel(const double* __restrict_
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t TB = Np / 32;
   const int64_t pairs = TB * (TB + 1) / 2;
-  double f = 0.0, bad = 0.0;
+  double f = 0.0;
+  int nbad = 0;
   for (int64_t tp = blockIdx.x; tp < pairs; tp += gridDim.x) {
-    int64_t bj = (int64_t)((sqrt(8.0 * (double)tp + 1.0) - 1.0) * 0.5);
+    int64_t bj = (int64_t)((sqrtf(8.0f * (float)tp + 1.0f) - 1.0f) * 0.5f);
     while ((bj + 1) * (bj + 2) / 2 <= tp) ++bj;
     while (bj * (bj + 1) / 2 > tp) --bj;
     const int64_t bi = tp - bj * (bj + 1) / 2;
+    double up[4];
+#pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int rl = ty + 8 * i;
       const int64_t r = bi * 32 + rl, c = bj * 32 + tx;
       const int64_t r2 = bj * 32 + rl, c2 = bi * 32 + tx;
-      up[rl][tx] = (r < n && c < n) ? G[r * ld + c] : 0.0;
+      up[i] = (r < n && c < n) ? G[r * ld + c] : 0.0;
       dn[rl][tx] = (r2 < n && c2 < n) ? G[r2 * ld + c2] : 0.0;
     }
     __syncthreads();
+    double ft = 0.0;
+#pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int rl = ty + 8 * i;
-      const int64_t r = bi * 32 + rl, c = bj * 32 + tx;
-      // (G + G^T)/2 at (r, c): up[rl][tx] and the transposed element dn[tx][rl]
-      const float v = (float)(0.5 * (up[rl][tx] + dn[tx][rl]));
-      dst[(size_t)r * Np + c] = v;
-      const double wgt = bi < bj ? 2.0 : 1.0;
-      f += wgt * (double)v * (double)v;
-      if (!isfinite(v)) bad += 1.0;
-      if (bi < bj) {
-        const float vt = (float)(0.5 * (up[tx][rl] + dn[rl][tx]));
-        dst[(size_t)(bj * 32 + rl) * Np + bi * 32 + tx] = vt;
+      // (G + G^T)/2 at (r, c): up and the transposed element dn[tx][rl]
+      const float v = narrow<1>(up[i] + dn[tx][rl]);
+      dst[(size_t)(bi * 32 + rl) * Np + bj * 32 + tx] = v;
+      sv[rl][tx] = v;
+      const double w = widen(v);
+      ft = fma(w, w, ft);
+      nbad += isfinite(v) ? 0 : 1;
+    }
+    f += bi < bj ? 2.0 * ft : ft;
+    __syncthreads();
+    if (bi < bj) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int rl = ty + 8 * i;
+        dst[(size_t)(bj * 32 + rl) * Np + bi * 32 + tx] = sv[tx][rl];
       }
     }
-    __syncthreads();
   }
-  double v[2] = {f, bad};
+  double v[2] = {f, (double)nbad};
   block_sum<2, 256>(v, red);
   if (threadIdx.x == 0) {
     double* p = partials + ((size_t)1 * ptiles + blockIdx.x) * kNQ;
@@ -1771,7 +1814,7 @@ __global__ void __launch_bounds__(256) adj_finalize_kernel(const State* st,
   const int64_t tb = (n + kSymTile - 1) / kSymTile;
   for (int64_t tile = blockIdx.x; tile < tb * tb; tile += gridDim.x)
     sym_tile<float>(src, Np, n, tile / tb, tile % tb, t, [&](int64_t r, int64_t c, float v) {
-      dLdH[r * ld + c] = scale * (double)v;
+      dLdH[r * ld + c] = scale * widen(v);
     });
 }
 
@@ -1792,6 +1835,11 @@ cudaError_t launch_adj_finalize(const Layout& L, void* ws, double* dLdH, int64_t
 // P_o = -S_o.
 __device__ __forceinline__ double out_value(double v, int64_t r, int64_t c, int y, bool hole) {
   return !hole ? v : (y == 0 ? (r == c ? 1.0 : 0.0) - v : -v);
+}
+__device__ __forceinline__ double out_value(float v, int64_t r, int64_t c, int y, bool hole) {
+  if (!hole) return widen(v);
+  if (y == 0) return r == c ? 1.0 - (double)v : widen(0.0f - v);   // 0 - 0 = +0, as in FP64
+  return widen(-v);
 }
 
 template <typename T>
@@ -1815,7 +1863,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(const State* st,
   const int64_t tb = (n + kSymTile - 1) / kSymTile;
   for (int64_t tile = blockIdx.x; tile < tb * tb; tile += gridDim.x)
     sym_tile<T>(src, Np, n, tile / tb, tile % tb, t, [&](int64_t r, int64_t c, T v) {
-      dst[r * ld + c] = out_value((double)v, r, c, y, hole);
+      dst[r * ld + c] = out_value(v, r, c, y, hole);
     });
 }
 
@@ -2046,7 +2094,7 @@ __global__ void __launch_bounds__(256) batch_finalize_kernel(const BatchInst* __
   const bool hole = st->hole != 0;
   const int64_t ld = b.ld;
   sym_tile<T>(src, b.Np, n, tile / tb, tile % tb, t, [&](int64_t r, int64_t cc, T v) {
-    dst[r * ld + cc] = out_value((double)v, r, cc, y, hole);
+    dst[r * ld + cc] = out_value(v, r, cc, y, hole);
   });
 }
 
