@@ -958,18 +958,21 @@ dmpt_status dmpt_sp2_backward(dmpt_handle h, const double* G, int64_t n, int64_t
         return cuda_fail(h, e, "segment load");
       if ((e = launch_split(L, workspace, 0, s, 1)) != cudaSuccess)
         return cuda_fail(h, e, "segment split");
+      // in the forward's D0 layers all k_fwd response jobs ran, and their
+      // items came before the square's in each launch
+      if (a + 1 < b &&
+          (e = launch_recompute_step(L, workspace, false, a + 1, a, rec_item_base, s)) !=
+              cudaSuccess)
+        return cuda_fail(h, e, "recompute plan");
       for (int m = a + 1; m < b; ++m) {
-        // in the forward's D0 layers all k_fwd response jobs ran, and their
-        // items came before the square's in each launch
-        if ((e = launch_recompute_plan(L, workspace, m, a, rec_item_base, s)) != cudaSuccess)
-          return cuda_fail(h, e, "recompute plan");
         // no round alignment: the skipped leading items are never counted in
         if ((e = launch_layer_tc(L, workspace, s, o->timeout_s, fs.fwd_chunk, fs.fwd_cta_pair,
                                  fs.fwd_k_snake, fs.fwd_band, &entries, &pass_flops, 0,
                                  0)) != cudaSuccess)
           return cuda_fail(h, e, "recompute layer");
-        if ((e = launch_recompute_done(L, workspace, s)) != cudaSuccess)
-          return cuda_fail(h, e, "recompute done");
+        if ((e = launch_recompute_step(L, workspace, true, m + 1 < b ? m + 1 : 0, a,
+                                       rec_item_base, s)) != cudaSuccess)
+          return cuda_fail(h, e, "recompute step");
       }
       if ((e = launch_decide(L, workspace, kDecideAdjResume, 0, s)) != cudaSuccess)
         return cuda_fail(h, e, "adjoint decide");

@@ -273,15 +273,15 @@ cudaError_t launch_split(const Layout& L, void* ws, int first_job, cudaStream_t 
 // checkpoint slot when the last decide step asked for it (State::ckpt_pending).
 cudaError_t launch_ckpt_store(const Layout& L, void* ws, cudaStream_t s);
 // Backward with checkpoints: load checkpoint `c` (state a = c * ckpt_k) as the
-// current S0 master (buffer 0) and the first tape state, and plan / finish
-// the recompute of state m from state m - 1 (its 16-bit copies into tape slot
-// m - a) with the forward's sigma_m.
+// current S0 master (buffer 0) and the first tape state.
 cudaError_t launch_seg_load(const Layout& L, void* ws, int c, int a, cudaStream_t s);
-// item_base: the forward launch's response items that preceded the square's
-// (pair kernel), so that the square's tiles keep their rounds.
-cudaError_t launch_recompute_plan(const Layout& L, void* ws, int m, int a, int64_t item_base,
-                                  cudaStream_t s);
-cudaError_t launch_recompute_done(const Layout& L, void* ws, cudaStream_t s);
+// One step between the recompute layers of a segment starting at state a: after
+// a layer (after) its state becomes the current S0; then the recompute of state
+// m from state m - 1 (16-bit copies into tape slot m - a, the forward's sigma_m)
+// is planned (0: none).  item_base: the forward launch's response items that preceded the
+// square's (pair kernel), so that the square's tiles keep their rounds.
+cudaError_t launch_recompute_step(const Layout& L, void* ws, bool after, int m, int a,
+                                  int64_t item_base, cudaStream_t s);
 // adjoint: Gbar = sym(G) into response slot 1 (upper triangle mirrored)
 cudaError_t launch_adj_init(const Layout& L, void* ws, const double* G, int64_t ld, int blocks,
                             cudaStream_t s);

@@ -1588,8 +1588,10 @@ __device__ __forceinline__ void sym_tile(const T* __restrict__ src, int64_t Np, 
 // Checkpoints of the S0 recursion (ckpt_every = k >= 2) and the recompute of a
 // segment of states from its checkpoint in the backward pass.
 
-__global__ void ckpt_store_kernel(const State* st, const float4* __restrict__ master,
+__global__ void ckpt_store_kernel(const State* st, const float4* master,
                                   float4* ckpt, int64_t Np, int lk) {
+  pdl_wait();
+  pdl_launch();
   if (!st->ckpt_pending) return;
   const int slot = st->d0_updates / st->ckpt_k;
   if (slot >= st->ckpt_slots) return;   // cannot happen: slots cover max_layers / k + 1
@@ -1598,15 +1600,14 @@ __global__ void ckpt_store_kernel(const State* st, const float4* __restrict__ ma
   float4* dst = ckpt + (size_t)slot * n4;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
        i += (size_t)gridDim.x * blockDim.x)
-    dst[i] = src[i];
+    dst[i] = __ldcg(&src[i]);
 }
 
 cudaError_t launch_ckpt_store(const Layout& L, void* ws, cudaStream_t s) {
   char* base = (char*)ws;
-  ckpt_store_kernel<<<152 * 4, 256, 0, s>>>((const State*)(base + L.off_state),
-                                            (const float4*)(base + L.off_master),
-                                            (float4*)(base + L.off_ckpt), L.Np, L.k);
-  return cudaGetLastError();
+  return launch_pdl(ckpt_store_kernel, dim3(152 * 4), dim3(256), 0, s,
+                    (const State*)(base + L.off_state), (const float4*)(base + L.off_master),
+                    (float4*)(base + L.off_ckpt), L.Np, L.k);
 }
 
 // Checkpoint c (state a) into S0 master buffer 0; it becomes the current S0
@@ -1687,39 +1688,32 @@ cudaError_t launch_seg_load(const Layout& L, void* ws, int c, int a, cudaStream_
 
 // Plan the recompute of S_m = sigma_m S_{m-1}^2 + (1 - sigma_m) S_{m-1}: the
 // square job only, S0 update stored, 16-bit copies into tape slot m - a.
-__global__ void recompute_plan_kernel(State* st, int m, int a, int64_t item_base) {
+__global__ void recompute_step_kernel(State* st, int after, int m, int a, int64_t item_base) {
+  pdl_wait();
+  if (m > 0) pdl_launch();   // the next kernel is a layer product, which reads after its wait
   st->round_ctr = 0u;
-  st->item_base = item_base;
-  st->plan_square = 1;
-  st->plan_write0 = 1;
-  st->sigma_cur = st->sigma[m];
-  for (int j = 0; j < kMaxK; ++j) st->plan_resp[j] = 0;
-  st->z0_next = st->tape_base + 2 * (m - a);
-}
-
-// After a recompute layer: the new state is the current S0.
-__global__ void recompute_done_kernel(State* st) {
-  st->round_ctr = 0u;
-  st->item_base = 0;
-  st->cur0 ^= 1;
-  st->z0_cur = st->z0_next;
-  st->plan_square = 0;
-  st->plan_write0 = 0;
-  if (st->timeout_flag) {
-    st->status = DMPT_ETIMEOUT;
-    st->done = 1;
+  if (after) {   // the layer's new state is the current S0
+    st->cur0 ^= 1;
+    st->z0_cur = st->z0_next;
+    if (st->timeout_flag) {
+      st->status = DMPT_ETIMEOUT;
+      st->done = 1;
+    }
+  }
+  st->item_base = m > 0 ? item_base : 0;
+  st->plan_square = m > 0;
+  st->plan_write0 = m > 0;
+  if (m > 0) {
+    st->sigma_cur = st->sigma[m];
+    for (int j = 0; j < kMaxK; ++j) st->plan_resp[j] = 0;
+    st->z0_next = st->tape_base + 2 * (m - a);
   }
 }
 
-cudaError_t launch_recompute_plan(const Layout& L, void* ws, int m, int a, int64_t item_base,
-                                  cudaStream_t s) {
-  recompute_plan_kernel<<<1, 1, 0, s>>>((State*)((char*)ws + L.off_state), m, a, item_base);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_recompute_done(const Layout& L, void* ws, cudaStream_t s) {
-  recompute_done_kernel<<<1, 1, 0, s>>>((State*)((char*)ws + L.off_state));
-  return cudaGetLastError();
+cudaError_t launch_recompute_step(const Layout& L, void* ws, bool after, int m, int a,
+                                  int64_t item_base, cudaStream_t s) {
+  return launch_pdl(recompute_step_kernel, dim3(1), dim3(1), 0, s,
+                    (State*)((char*)ws + L.off_state), (int)after, m, a, item_base);
 }
 
 // ---------------------------------------------------------------------------
