@@ -1231,51 +1231,63 @@ static dmpt_status batch_impl(dmpt_handle h, int count, const double* const* H,
         return cuda_fail(h, e, "join");
     }
   }
-  // one CUDA graph = one layer of every active instance, each on its own stream
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  if ((e = cudaStreamBeginCapture(h->origin, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
-    return cuda_fail(h, e, "batch capture");
-  cudaError_t ce = cudaEventRecord(h->fork, h->origin);
+  int steps = grouped ? 0 : 1;
   if (grouped) {
-    ce = launch_layer_tc_group(d_ginst, n_group, o->precision == DMPT_DUAL_BF16, d_gtimeout,
-                               d_gqueue, o->timeout_s, o->accum_chunk, o->k_snake, o->tile_band,
-                               h->sm_count, h->origin, n128);
-    if (ce == cudaSuccess)
-      ce = launch_decide_group(d_gdec, n_group, d_gtimeout, d_gqueue, h->origin);
-  }
-  for (int i = 0; i < count && ce == cudaSuccess && !grouped; ++i) {
-    if (!active[i]) continue;
-    ce = cudaStreamWaitEvent(h->streams[i], h->fork, 0);
-    if (ce == cudaSuccess) ce = issue_step(i);
-    if (ce == cudaSuccess) ce = cudaEventRecord(h->joins[i], h->streams[i]);
-    if (ce == cudaSuccess) ce = cudaStreamWaitEvent(h->origin, h->joins[i], 0);
-  }
-  e = cudaStreamEndCapture(h->origin, &graph);
-  if (ce != cudaSuccess || e != cudaSuccess) {
-    if (graph) cudaGraphDestroy(graph);
-    return cuda_fail(h, ce != cudaSuccess ? ce : e, "batch capture");
-  }
-  e = cudaGraphInstantiate(&exec, graph, 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) return cuda_fail(h, e, "batch instantiate");
-  int steps = grouped ? 0 : 1, all_done = n_active == 0 ? 1 : 0;
-  while (steps < o->max_layers && !all_done) {
-    for (int j = 0; j < o->sync_every && steps < o->max_layers; ++j, ++steps) {
-      if ((e = cudaGraphLaunch(exec, h->origin)) != cudaSuccess) {
+    // a grouped launch and its decide step per layer, followed through the
+    // mapped word (LayerFeed)
+    const LayerFeed feed(h, h->origin, layers_ahead(o));
+    bool done = false;
+    while (steps < o->max_layers && !done) {
+      if ((e = launch_layer_tc_group(d_ginst, n_group, o->precision == DMPT_DUAL_BF16, d_gtimeout,
+                                     d_gqueue, o->timeout_s, o->accum_chunk, o->k_snake,
+                                     o->tile_band, h->sm_count, h->origin, n128)) != cudaSuccess)
+        return cuda_fail(h, e, "batch layer");
+      ++steps;
+      if ((e = launch_decide_group(d_gdec, n_group, d_gtimeout, d_gqueue, h->progress_dev,
+                                   feed.code(steps), h->origin)) != cudaSuccess)
+        return cuda_fail(h, e, "batch decide");
+      if ((e = feed.wait(steps, &done)) != cudaSuccess) return cuda_fail(h, e, "batch loop");
+    }
+  } else {
+    // one CUDA graph = one layer of every active instance, each on its own stream
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    if ((e = cudaStreamBeginCapture(h->origin, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
+      return cuda_fail(h, e, "batch capture");
+    cudaError_t ce = cudaEventRecord(h->fork, h->origin);
+    for (int i = 0; i < count && ce == cudaSuccess; ++i) {
+      if (!active[i]) continue;
+      ce = cudaStreamWaitEvent(h->streams[i], h->fork, 0);
+      if (ce == cudaSuccess) ce = issue_step(i);
+      if (ce == cudaSuccess) ce = cudaEventRecord(h->joins[i], h->streams[i]);
+      if (ce == cudaSuccess) ce = cudaStreamWaitEvent(h->origin, h->joins[i], 0);
+    }
+    e = cudaStreamEndCapture(h->origin, &graph);
+    if (ce != cudaSuccess || e != cudaSuccess) {
+      if (graph) cudaGraphDestroy(graph);
+      return cuda_fail(h, ce != cudaSuccess ? ce : e, "batch capture");
+    }
+    e = cudaGraphInstantiate(&exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) return cuda_fail(h, e, "batch instantiate");
+    int all_done = n_active == 0 ? 1 : 0;
+    while (steps < o->max_layers && !all_done) {
+      for (int j = 0; j < o->sync_every && steps < o->max_layers; ++j, ++steps) {
+        if ((e = cudaGraphLaunch(exec, h->origin)) != cudaSuccess) {
+          cudaGraphExecDestroy(exec);
+          return cuda_fail(h, e, "batch graph launch");
+        }
+      }
+      if ((e = launch_batch_all_done(base, d_offs, n_active, d_flag, h->origin)) == cudaSuccess)
+        e = cudaMemcpyAsync(&all_done, d_flag, sizeof(int), cudaMemcpyDeviceToHost, h->origin);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(h->origin);
+      if (e != cudaSuccess) {
         cudaGraphExecDestroy(exec);
-        return cuda_fail(h, e, "batch graph launch");
+        return cuda_fail(h, e, "batch poll");
       }
     }
-    if ((e = launch_batch_all_done(base, d_offs, n_active, d_flag, h->origin)) == cudaSuccess)
-      e = cudaMemcpyAsync(&all_done, d_flag, sizeof(int), cudaMemcpyDeviceToHost, h->origin);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->origin);
-    if (e != cudaSuccess) {
-      cudaGraphExecDestroy(exec);
-      return cuda_fail(h, e, "batch poll");
-    }
+    cudaGraphExecDestroy(exec);
   }
-  cudaGraphExecDestroy(exec);
   // every instance's outputs, then every control block in one copy and one
   // synchronisation
   if ((e = launch_batch_finalize(d_binst, d_bfirst, n_active, units[kBsOut],

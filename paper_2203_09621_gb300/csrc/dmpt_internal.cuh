@@ -346,7 +346,8 @@ constexpr int kQueuePairs = 128;   // CTA pairs per grouped launch (<= 256 SMs)
 struct GroupQueue {
   unsigned counter;
   unsigned epoch;
-  unsigned pad[62];
+  unsigned decided;   // blocks of the running decide step that are through
+  unsigned pad[61];
   unsigned long long slot[kQueuePairs][kQueueRing];
 };
 // Fills `gi` for the instance whose workspace is `ws` (false: no tensor map);
@@ -366,7 +367,8 @@ cudaError_t launch_layer_tc_group(const GroupInst* inst, int count, bool bf16, i
 // Decide step of every instance (device array of `count`), one block each; a
 // set *group_timeout marks every instance timed out.
 cudaError_t launch_decide_group(const GroupDecide* args, int count, const int* group_timeout,
-                                GroupQueue* queue, cudaStream_t s);
+                                GroupQueue* queue, unsigned* progress, unsigned code,
+                                cudaStream_t s);
 
 enum DecideMode {
   kDecideInit = 0,

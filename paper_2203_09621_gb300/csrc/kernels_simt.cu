@@ -789,7 +789,8 @@ __device__ void decide_layer(State* S, State* G, const DecideShared& sh, int lan
 // the block is read before pdl_wait().
 template <bool Pdl>
 __device__ void decide_body(State* st, const double* partials, int64_t ptiles,
-                            int64_t entries, int jobs, int mode, DecideShared& sh) {
+                            int64_t entries, int jobs, int mode, DecideShared& sh,
+                            const int* group_timeout = nullptr) {
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid < kHeadWords) sh.head[tid] = __ldcg(reinterpret_cast<const unsigned*>(st) + tid);
   if (tid >= kDecideThreads - 32) {
@@ -813,7 +814,10 @@ __device__ void decide_body(State* st, const double* partials, int64_t ptiles,
   if constexpr (Pdl) {
     pdl_wait();
     constexpr int kTimeoutWord = (int)(offsetof(State, timeout_flag) / sizeof(unsigned));
-    if (tid == kTimeoutWord) sh.head[tid] = __ldcg(reinterpret_cast<const unsigned*>(st) + tid);
+    if (tid == kTimeoutWord)
+      sh.head[tid] = group_timeout && __ldcg(group_timeout)
+                         ? 1u
+                         : __ldcg(reinterpret_cast<const unsigned*>(st) + tid);
   }
   // Sums of the partials, four jobs at once, in a fixed order: lane 4 u + q of
   // warp w of a job adds quantity q of the entries 8 w + u (mod 64), three
@@ -878,28 +882,37 @@ __global__ void __launch_bounds__(kDecideThreads)
     *progress = code | (reinterpret_cast<const State*>(sh.head)->done ? 1u : 0u);
 }
 
-// Layer decide of every instance of a grouped launch, one block each.
+// Layer decide of every instance of a grouped launch, one block each; the last
+// block to finish reports to the host (progress, as in decide_kernel; bit 0:
+// every instance has ended).
 __global__ void __launch_bounds__(kDecideThreads)
-    decide_group_kernel(const GroupDecide* __restrict__ args, const int* __restrict__ group_timeout,
-                        GroupQueue* queue) {
+    decide_group_kernel(const GroupDecide* __restrict__ args, const int* group_timeout,
+                        GroupQueue* queue, volatile unsigned* progress, unsigned code) {
   __shared__ DecideShared sh;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {   // the next grouped launch starts a new queue
+  pdl_launch();
+  const GroupDecide a = args[blockIdx.x];
+  decide_body<true>(a.st, a.partials, a.ptiles, a.entries, a.jobs, kDecideLayer, sh,
+                    group_timeout);
+  if (threadIdx.x != 0) return;
+  if (blockIdx.x == 0) {   // the next grouped launch starts a new queue
     queue->counter = 0u;
     queue->epoch += 1u;
   }
-  const GroupDecide a = args[blockIdx.x];
-  if (*group_timeout) {   // uniform across the grid
-    if (threadIdx.x == 0 && !a.st->done) a.st->timeout_flag = 1;
-    __syncthreads();
+  // blocks that are through (low half) and instances that have ended (high half)
+  const unsigned one = 1u | (reinterpret_cast<const State*>(sh.head)->done ? 0x10000u : 0u);
+  const unsigned all = atomicAdd(&queue->decided, one) + one;
+  if ((all & 0xFFFFu) == gridDim.x) {
+    queue->decided = 0u;
+    *progress = code | ((all >> 16) == gridDim.x ? 1u : 0u);
   }
-  decide_body<false>(a.st, a.partials, a.ptiles, a.entries, a.jobs, kDecideLayer, sh);
 }
 
 cudaError_t launch_decide_group(const GroupDecide* args, int count, const int* group_timeout,
-                                GroupQueue* queue, cudaStream_t s) {
+                                GroupQueue* queue, unsigned* progress, unsigned code,
+                                cudaStream_t s) {
   if (count < 1) return cudaSuccess;
-  decide_group_kernel<<<count, kDecideThreads, 0, s>>>(args, group_timeout, queue);
-  return cudaGetLastError();
+  return launch_pdl(decide_group_kernel, dim3(count), dim3(kDecideThreads), 0, s, args,
+                    group_timeout, queue, progress, code);
 }
 
 // Per-device one-time setup; thread-safe.  The decide kernel runs between

@@ -1743,29 +1743,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   int64_t* first = reinterpret_cast<int64_t*>(misc + 1024 + EPI_SCRATCH);
   uint32_t* jmask = reinterpret_cast<uint32_t*>(first + count + 1);
 
-  // ---- this layer's items of every instance (same values in every CTA:
-  //      the control blocks do not change during the launch)
-  for (int i = threadIdx.x; i < count; i += blockDim.x) {
-    const State* sti = inst[i].st;
-    uint32_t jm = 0;
-    if (!sti->done) {
-      jm = sti->plan_square ? 1u : 0u;
-      for (int j = 0; j < inst[i].k; ++j)
-        if (sti->plan_resp[j]) jm |= 1u << (1 + j);
-    }
-    jmask[i] = jm;
-    first[i + 1] = num_pair_tiles(inst[i].Np) * __popc(jm);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    first[0] = 0;
-    for (int i = 0; i < count; ++i) first[i + 1] += first[i];
-  }
-  __syncthreads();
-  const int64_t items = first[count];
-  if (items == 0) return;   // every CTA takes this exit together
-  const unsigned epoch = *(volatile unsigned*)&gq->epoch;   // fixed during the launch
-
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
   const int64_t pair = blockIdx.x >> 1;
@@ -1810,7 +1787,37 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
   int* timeout_global = group_timeout;
 
-  if (warp == 0) {
+  // ---- everything above ran while the decide step before finished
+  pdl_wait();
+  pdl_launch();
+  __threadfence();   // the control blocks are read through L1
+
+  // ---- this layer's items of every instance (same values in every CTA:
+  //      the control blocks do not change during the launch)
+  for (int i = threadIdx.x; i < count; i += blockDim.x) {
+    const State* sti = inst[i].st;
+    uint32_t jm = 0;
+    if (!sti->done) {
+      jm = sti->plan_square ? 1u : 0u;
+      for (int j = 0; j < inst[i].k; ++j)
+        if (sti->plan_resp[j]) jm |= 1u << (1 + j);
+    }
+    jmask[i] = jm;
+    first[i + 1] = num_pair_tiles(inst[i].Np) * __popc(jm);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    first[0] = 0;
+    for (int i = 0; i < count; ++i) first[i + 1] += first[i];
+  }
+  __syncthreads();
+  const int64_t items = first[count];
+  const unsigned epoch = *(volatile unsigned*)&gq->epoch;   // fixed during the launch
+
+
+  if (items == 0) {
+    // every instance has ended
+  } else if (warp == 0) {
     // ================= TMA producer (both CTAs load their own halves) ======
     {
       RingPos rg;
@@ -2066,28 +2073,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   int64_t* first = reinterpret_cast<int64_t*>(misc + 1024 + EPI_SCRATCH);
   uint32_t* jmask = reinterpret_cast<uint32_t*>(first + count + 1);
 
-  // ---- this layer's items of every instance (as in the 256 x 256 kernel)
-  for (int i = threadIdx.x; i < count; i += blockDim.x) {
-    const State* sti = inst[i].st;
-    uint32_t jm = 0;
-    if (!sti->done) {
-      jm = sti->plan_square ? 1u : 0u;
-      for (int j = 0; j < inst[i].k; ++j)
-        if (sti->plan_resp[j]) jm |= 1u << (1 + j);
-    }
-    jmask[i] = jm;
-    first[i + 1] = num_tiles128(inst[i].Np) * __popc(jm);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    first[0] = 0;
-    for (int i = 0; i < count; ++i) first[i + 1] += first[i];
-  }
-  __syncthreads();
-  const int64_t items = first[count];
-  if (items == 0) return;   // every CTA takes this exit together
-  const unsigned epoch = *(volatile unsigned*)&gq->epoch;   // fixed during the launch
-
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
   const int64_t pair = blockIdx.x >> 1;
@@ -2132,7 +2117,36 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
   int* timeout_global = group_timeout;
 
-  if (warp == 0) {
+  // ---- everything above ran while the decide step before finished
+  pdl_wait();
+  pdl_launch();
+  __threadfence();   // the control blocks are read through L1
+
+  // ---- this layer's items of every instance (as in the 256 x 256 kernel)
+  for (int i = threadIdx.x; i < count; i += blockDim.x) {
+    const State* sti = inst[i].st;
+    uint32_t jm = 0;
+    if (!sti->done) {
+      jm = sti->plan_square ? 1u : 0u;
+      for (int j = 0; j < inst[i].k; ++j)
+        if (sti->plan_resp[j]) jm |= 1u << (1 + j);
+    }
+    jmask[i] = jm;
+    first[i + 1] = num_tiles128(inst[i].Np) * __popc(jm);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    first[0] = 0;
+    for (int i = 0; i < count; ++i) first[i + 1] += first[i];
+  }
+  __syncthreads();
+  const int64_t items = first[count];
+  const unsigned epoch = *(volatile unsigned*)&gq->epoch;   // fixed during the launch
+
+
+  if (items == 0) {
+    // every instance has ended
+  } else if (warp == 0) {
     // ================= TMA producer (both CTAs load their own rows) ======
     {
       RingPos rg;
@@ -2473,22 +2487,13 @@ cudaError_t launch_layer_tc_group(const GroupInst* inst, int count, bool bf16, i
   const int ck = accum_chunk_k > 0 ? accum_chunk_k : DEFAULT_CHUNK_K;
   const int chunk = ck / BK < 1 ? 1 : ck / BK;
   const int grid = 2 * (sm_count / 2);
-  if (n128) {
-    if (bf16)
-      layer_tc2_group128_kernel<true><<<grid, NUM_THREADS, smem, s>>>(inst, count, group_timeout,
-                                                                      queue, limit_ns, chunk);
-    else
-      layer_tc2_group128_kernel<false><<<grid, NUM_THREADS, smem, s>>>(
-          inst, count, group_timeout, queue, limit_ns, chunk);
-    return cudaGetLastError();
-  }
-  if (bf16)
-    layer_tc2_group_kernel<true><<<grid, NUM_THREADS, smem, s>>>(
-        inst, count, group_timeout, queue, limit_ns, chunk, k_snake, band);
-  else
-    layer_tc2_group_kernel<false><<<grid, NUM_THREADS, smem, s>>>(
-        inst, count, group_timeout, queue, limit_ns, chunk, k_snake, band);
-  return cudaGetLastError();
+  if (n128)
+    return launch_pdl(bf16 ? layer_tc2_group128_kernel<true> : layer_tc2_group128_kernel<false>,
+                      dim3(grid), dim3(NUM_THREADS), smem, s, inst, count, group_timeout, queue,
+                      limit_ns, chunk);
+  return launch_pdl(bf16 ? layer_tc2_group_kernel<true> : layer_tc2_group_kernel<false>,
+                    dim3(grid), dim3(NUM_THREADS), smem, s, inst, count, group_timeout, queue,
+                    limit_ns, chunk, k_snake, band);
 }
 
 cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double timeout_s,
