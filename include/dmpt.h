@@ -143,9 +143,11 @@ typedef struct {
                            recursion on P as printed                         */
   int group_tile_n;     /* batches on the grouped kernel: tile width 256
                            (default: 256 x 256 pair tiles, instances padded to
-                           a multiple of 256) or 128 (256 x 128 tiles, four
-                           tensor-memory accumulators, instances padded to a
-                           multiple of 128)                                   */
+                           a multiple of 256; batches of small instances run
+                           on 256 x 128 tiles where that gives the same bits)
+                           or 128 (256 x 128 tiles, four tensor-memory
+                           accumulators, instances padded to a multiple of
+                           128)                                               */
 } dmpt_options;
 
 /* Filled on the host by dmpt_sp2_response (when info != NULL). */

@@ -939,13 +939,14 @@ cudaError_t launch_decide(const Layout& L, void* ws, int mode, int64_t entries, 
 }
 
 // ---------------------------------------------------------------------------
-// SIMT layer product with fused epilogue (FP64 and FP32 forms).
+// FP32 layer product with fused epilogue.
 //
 // Grid: (upper tiles, 1 + slots).  Job 0 computes X = S0 S0 (Sec. II B,
 // Eq. (DNN-SP2_act)) for tile (I, J), I <= J; job 1+k computes
 // X1 = S0 S1_k + S1_k S0 (activation f^(1), Eq. (eq:activation-function))
 // as one accumulation over two K-passes; a higher-order term (Sec. III A,
-// Eq. (S_n detailed)) adds its cross products S_a S_{o-a} as further passes.  Both operands are read as row
+// Eq. (S_n detailed)) adds its cross products S_a S_{o-a} as further passes.
+// Both operands are read as row
 // panels: for symmetric B, B[k][j] = B[j][k].  The epilogue applies
 // S_n = sigma X + (1 - sigma) S_{n-1} (Eq. (eq:Sn); Alg. 2 / Alg. 3 updates)
 // to the elements with row <= col, stores them at (r, c) and (c, r) in the
@@ -1142,9 +1143,9 @@ __global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
   const T om = (T)1 - sg;
   const bool write = job == 0 ? st->plan_write0 != 0 : true;
   double tr = 0.0, bad = 0.0;
-  // ||S_new||_F^2 and ||S_old - X||_F^2: in FP64 for the FP64 form; for the
-  // FP32 form as exact FP32 products summed with TwoSum compensation (the
-  // FP64 rate of the part is low), converted to FP64 once per thread
+  // ||S_new||_F^2 and ||S_old - X||_F^2 as exact FP32 products summed with
+  // TwoSum compensation (the FP64 rate of the part is low), converted to FP64
+  // once per thread
   float fn_s = 0.0f, fn_c = 0.0f, fd_s = 0.0f, fd_c = 0.0f;
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
