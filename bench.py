@@ -804,7 +804,7 @@ def main():
     traffic = recorded_traffic({"n": n, "k": k, "precision": args.precision, "cta_pair": args.cta_pair,
                                 "k_snake": args.k_snake, "tile_band": args.tile_band,
                                 "accum_chunk": args.accum_chunk})
-    launches_per_step = 7 + (1 if args.precision.startswith("dual") else 0) + 2 * infos[0].product_launches
+    launches_per_step = 5 + (1 if args.precision.startswith("dual") else 0) + 2 * infos[0].product_launches
     if rank == 0:
         line = {
             "metric": METRIC, "value": value, "unit": "TFLOP/s", "n_gpus": world,
