@@ -227,15 +227,16 @@ cudaError_t launch_forward_setup(const Layout& L, void* ws, const double* H, int
 // matrices are exactly symmetric.  Partial sums per block: Tr S0, ||S0||_F^2,
 // ||S1_k||_F^2 and a count of non-finite values.
 
-// Block vb of a grid of vgrid blocks (256 threads): tile pairs vb, vb + vgrid,
-// ... of each matrix in turn (S0, then S1_1 .. S1_k).
+// Block vb of vgrid blocks (256 threads): tile pairs vb, vb + vgrid, ... of
+// matrices m_lo .. m_hi in turn (0 = S0, m = S1_m; those above k are the
+// higher-order slots, which start at zero: a linear perturbation has H^(o) = 0
+// for o >= 2).  The count of non-finite values goes with job m_lo.
 template <typename T>
 __device__ __forceinline__ void init_body(State* st, T* master, const double* __restrict__ H,
                                           const double* __restrict__ H1, int64_t n, int64_t Np,
-                                          int64_t ld, int k, int first_m,
-                                          const double* __restrict__ shift, int k_zero,
-                                          double* partials, int64_t ptiles, int64_t vb,
-                                          int64_t vgrid) {
+                                          int64_t ld, int k, int m_lo, int m_hi,
+                                          const double* __restrict__ shift, double* partials,
+                                          int64_t ptiles, int64_t vb, int64_t vgrid) {
   // 64 x 64 tile pairs (bi <= bj): the upper tile is read row-wise (coalesced,
   // every load of the tile in flight at once), written in place and, through
   // shared memory, transposed into the mirror tile, so both triangles of S
@@ -262,7 +263,7 @@ __device__ __forceinline__ void init_body(State* st, T* master, const double* __
   const int64_t TB = Np / TS;
   const int64_t pairs = TB * (TB + 1) / 2;
   int nbad = 0;
-  for (int m = first_m; m <= k; ++m) {
+  for (int m = m_lo; m <= m_hi && m <= k; ++m) {
     const double* src = m == 0 ? H : H1 + (size_t)(m - 1) * n * ld;
     T* dst = master + (size_t)m * mat;   // buffer 0 (slots 0 .. layout k)
     double tr = 0.0, fd = 0.0;
@@ -359,8 +360,7 @@ __device__ __forceinline__ void init_body(State* st, T* master, const double* __
       p[kQBad] = 0.0;
     }
   }
-  // higher-order slots start at zero (a linear perturbation: H^(o) = 0, o >= 2)
-  for (int m = k + 1; m <= k + k_zero; ++m) {
+  for (int m = m_lo > k ? m_lo : k + 1; m <= m_hi; ++m) {
     T* dst = master + (size_t)m * mat;
     for (int64_t idx = vb * blockDim.x + threadIdx.x; idx < (int64_t)mat;
          idx += vgrid * blockDim.x)
@@ -373,24 +373,25 @@ __device__ __forceinline__ void init_body(State* st, T* master, const double* __
       p[kQBad] = 0.0;
     }
   }
-  // the count of non-finite values goes with job 0 (job 1 in a replay, which
-  // starts at S1_1)
   double vb_bad[1] = {(double)nbad};
   block_sum<1, 256>(vb_bad, red);
-  if (threadIdx.x == 0 && (first_m == 0 || k > 0))
-    partials[((size_t)first_m * ptiles + vb) * kNQ + kQBad] = vb_bad[0];
+  if (threadIdx.x == 0) partials[((size_t)m_lo * ptiles + vb) * kNQ + kQBad] = vb_bad[0];
 }
 
+// One matrix per grid row: the matrices one after the other in each block was a
+// chain of loads and block sums (n = 1000 k = 2 34 -> 21 us, order 3 at n = 512
+// k = 2 19 -> 8 us; at n = 2048 k = 3 both take 46 us).
 template <typename T>
 __global__ void __launch_bounds__(256) init_kernel(State* st, T* master, const double* __restrict__ H,
                                                    const double* __restrict__ H1, int64_t n,
                                                    int64_t Np, int64_t ld, int k, int first_m,
-                                                   const double* __restrict__ shift, int k_zero,
+                                                   const double* __restrict__ shift,
                                                    double* partials, int64_t ptiles) {
   pdl_wait();
   pdl_launch();
-  init_body<T>(st, master, H, H1, n, Np, ld, k, first_m, shift, k_zero, partials, ptiles,
-               blockIdx.x, gridDim.x);
+  const int m = first_m + (int)blockIdx.y;
+  init_body<T>(st, master, H, H1, n, Np, ld, k, m, m, shift, partials, ptiles, blockIdx.x,
+               gridDim.x);
 }
 
 int init_blocks(int64_t Np) {
@@ -404,13 +405,13 @@ cudaError_t launch_init(const Layout& L, void* ws, const double* H, const double
   char* base = (char*)ws;
   State* st = (State*)(base + L.off_state);
   double* partials = (double*)(base + L.off_partials);
+  const dim3 grid(blocks, k + k_zero + 1 - first_m);
   if (L.precision == DMPT_FP64)
-    return launch_pdl(init_kernel<double>, dim3(blocks), dim3(256), 0, s, st,
+    return launch_pdl(init_kernel<double>, grid, dim3(256), 0, s, st,
                       (double*)(base + L.off_master), H, H1, L.n, L.Np, ld, k, first_m, shift,
-                      k_zero, partials, L.partial_tiles);
-  return launch_pdl(init_kernel<float>, dim3(blocks), dim3(256), 0, s, st,
-                    (float*)(base + L.off_master), H, H1, L.n, L.Np, ld, k, first_m, shift, k_zero,
-                    partials, L.partial_tiles);
+                      partials, L.partial_tiles);
+  return launch_pdl(init_kernel<float>, grid, dim3(256), 0, s, st, (float*)(base + L.off_master),
+                    H, H1, L.n, L.Np, ld, k, first_m, shift, partials, L.partial_tiles);
 }
 
 // ---------------------------------------------------------------------------
@@ -693,8 +694,9 @@ __device__ void decide_adjoint(State* S, const DecideShared& sh, int mode) {
 
 // The initial layer has run: start of a forward run (one warp).
 __device__ void decide_init(State* S, State* G, const DecideShared& sh, int lane) {
-  if (!(S->epsN > S->eps1) || !isfinite(S->epsN) || !isfinite(S->eps1) ||
-      sh.sums[0][kQBad] > 0.0)
+  const bool bad =
+      __any_sync(0xffffffffu, lane <= S->k && sh.sums[lane <= S->k ? lane : 0][kQBad] > 0.0);
+  if (!(S->epsN > S->eps1) || !isfinite(S->epsN) || !isfinite(S->eps1) || bad)
     return decide_end(S, lane, DMPT_ENUMERIC);
   if (lane == 0) {
     S->NS = sh.sums[0][kQTrace];
@@ -2036,8 +2038,8 @@ __global__ void __launch_bounds__(256) batch_init_kernel(const BatchInst* __rest
   const int64_t u = blockIdx.x;
   const int i = batch_find(first, count, u);
   const BatchInst& b = bi[i];
-  init_body<T>(b.st, static_cast<T*>(b.master), b.H, b.H1, b.n, b.Np, b.ld, b.k, 0, nullptr, 0,
-               b.partials, b.ptiles, u - first[i], kInitBlocks);
+  init_body<T>(b.st, static_cast<T*>(b.master), b.H, b.H1, b.n, b.Np, b.ld, b.k, 0, b.k,
+               nullptr, b.partials, b.ptiles, u - first[i], kInitBlocks);
 }
 
 __global__ void __launch_bounds__(kDecideThreads)
