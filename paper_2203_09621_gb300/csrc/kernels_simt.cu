@@ -785,15 +785,22 @@ __device__ void decide_layer(State* S, State* G, const DecideShared& sh, int lan
 
 // The decide step of one instance, run by one block of kDecideThreads
 // threads.  jobs: 1 + the response slots of the partials array.
-// Pdl: launched while the layer product may still run.  That product writes
-// nothing of the control block but timeout_flag (and round_ctr, reset here),
-// and it started after the previous decide step had finished, so the rest of
-// the block is read before pdl_wait().
+// Pdl: launched while the kernel before it may still run.  That kernel is a
+// layer product or an initial kernel, which write nothing of the control block
+// but timeout_flag (and round_ctr, reset here), and it started after the last
+// kernel that did write the block had finished, so the rest is read before
+// pdl_wait().  The exception is kDecideAdjResume, which follows the step kernel
+// between recompute layers or the load of a segment: a grid's writes are only
+// visible after the wait (its end alone, without pdl_launch(), orders nothing),
+// and the whole head is stored back below, so it waits first.
 template <bool Pdl>
 __device__ void decide_body(State* st, const double* partials, int64_t ptiles,
                             int64_t entries, int jobs, int mode, DecideShared& sh,
                             const int* group_timeout = nullptr) {
   const int tid = threadIdx.x, lane = tid & 31;
+  if constexpr (Pdl) {
+    if (mode == kDecideAdjResume) pdl_wait();
+  }
   if (tid < kHeadWords) sh.head[tid] = __ldcg(reinterpret_cast<const unsigned*>(st) + tid);
   if (tid >= kDecideThreads - 32) {
     // the history entries the tests read, fetched while the sums are formed
