@@ -141,13 +141,12 @@ typedef struct {
                            the rounding of the products small next to the
                            response when few levels are empty; 0: always the
                            recursion on P as printed                         */
-  int group_tile_n;     /* batches on the grouped kernel: tile width 256
-                           (default: 256 x 256 pair tiles, instances padded to
-                           a multiple of 256; batches of small instances run
-                           on 256 x 128 tiles where that gives the same bits)
-                           or 128 (256 x 128 tiles, four tensor-memory
-                           accumulators, instances padded to a multiple of
-                           128)                                               */
+  int group_tile_n;     /* batches on the grouped kernel: tile width 256 (256 x
+                           256 pair tiles, instances padded to a multiple of
+                           256), 128 (256 x 128 tiles, four tensor-memory
+                           accumulators, instances padded to a multiple of 128)
+                           or 0 (default): 128 for batches of small instances,
+                           where it gives the same bits, else 256             */
 } dmpt_options;
 
 /* Filled on the host by dmpt_sp2_response (when info != NULL). */
@@ -325,7 +324,8 @@ dmpt_status dmpt_sp2_backward(dmpt_handle h, const double* G, int64_t n, int64_t
  * internal stream of its own.  One CUDA graph holds a layer step and is
  * replayed until all instances have converged (finished instances add no
  * work).  Each instance's results equal those of its own dmpt_sp2_response
- * call bit for bit, except on 256 x 128 tiles (o->group_tile_n = 128).
+ * call bit for bit; with o->group_tile_n = 128 that holds for instances whose
+ * 256 x 256 tiles take one round of the CTA pairs, the others agree to rounding.
  *   count       instances; H, H1, P, P1: host arrays of `count` device
  *               pointers (H1/P1 entries: k blocks of n_i x n_i (ld_i)).
  *   n, ld, n_occ: host arrays of `count` values.

@@ -158,7 +158,7 @@ bool valid_options(const dmpt_options* o) {
   if (o->autotune < 0 || o->autotune > 1) return false;
   if (o->round_align < 0 || o->round_align > 1) return false;
   if (o->hole_form < 0 || o->hole_form > 1) return false;
-  if (o->group_tile_n != 128 && o->group_tile_n != 256) return false;
+  if (o->group_tile_n != 0 && o->group_tile_n != 128 && o->group_tile_n != 256) return false;
   return true;
 }
 
@@ -356,7 +356,7 @@ void dmpt_default_options(dmpt_options* o) {
   o->tile_band = 8;
   o->round_align = 1;
   o->hole_form = 1;
-  o->group_tile_n = 256;
+  o->group_tile_n = 0;
 }
 
 const char* dmpt_status_string(dmpt_status s) {
@@ -1096,21 +1096,21 @@ static dmpt_status batch_impl(dmpt_handle h, int count, const double* const* H,
   // instances (GroupInst table, batched decide); otherwise one launch per
   // instance on its own stream
   const bool can_group = dual && o->cta_pair && o->order == 1 && n_act > 0 && n_act <= kGroupMax;
-  // 256 x 128 tiles, padding to 128: where asked for, and in the default for
-  // batches of small instances.  Their four accumulators keep the MMAs going
-  // during the tile epilogues, which pays until operand traffic counts more
-  // (us, 256 / 128 wide: 64 instances of n = 64 to 512 3931 / 3609, 8 of 256 to
-  // 1024 with k = 3 2567 / 2238, 32 of 1024 to 1100 15595 / 15022, 12 of 900 to
-  // 1400 with k = 2 10581 / 10513, 16 of 1800 to 2048 30950 / 32809).  An instance
-  // whose 256 x 256 tiles take one round of the CTA pairs has the same bits at
-  // both widths (no backwards K sweeps).
+  // 256 x 128 tiles, padding to 128: where asked for, and by default
+  // (group_tile_n = 0) for batches of small instances.  Their four accumulators
+  // keep the MMAs going during the tile epilogues, which pays until operand
+  // traffic counts more (us, 256 / 128 wide: 64 instances of n = 64 to 512
+  // 3931 / 3609, 8 of 256 to 1024 with k = 3 2567 / 2238, 32 of 1024 to 1100
+  // 15595 / 15022, 12 of 900 to 1400 with k = 2 10581 / 10513, 16 of 1800 to 2048
+  // 30950 / 32809).  An instance whose 256 x 256 tiles take one round of the CTA
+  // pairs has the same bits at both widths (no backwards K sweeps).
   bool narrow = true;
   for (int i = 0; i < count; ++i) {
     const int64_t tb = (n[i] + kPad - 1) / kPad;
     if (active[i] && (tb > 5 || tb * (tb + 1) / 2 * (1 + k) > h->sm_count / 2)) narrow = false;
   }
-  const bool n128 =
-      (path == 3 || (path == -1 && (o->group_tile_n == 128 || narrow))) && can_group;
+  const int gtn = o->group_tile_n != 0 ? o->group_tile_n : (narrow ? 128 : 256);
+  const bool n128 = (path == 3 || (path == -1 && gtn == 128)) && can_group;
   size_t off = batch_scratch_bytes(count);
   for (int i = 0; i < count; ++i) {
     L[i] = layout_for(n[i], k, o, n128 ? 128 : kPad);

@@ -205,7 +205,7 @@ def options(precision="dual_fp16", max_layers=100, c_pt=9.0, c_d0=4.5, operand_s
             sync_every=4, timing=False, timeout_s=2.0, accum_chunk=0,
             cta_pair=1, k_snake=1, ckpt_every=0, order=1, tile_band=8,
             inject_stall=0, autotune=0, round_align=1, hole_form=1,
-            group_tile_n=256) -> DmptOptions:
+            group_tile_n=0) -> DmptOptions:
     lib = load_library()
     o = DmptOptions()
     lib.dmpt_default_options(ctypes.byref(o))
