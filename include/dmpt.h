@@ -28,9 +28,14 @@
  *  - The library only runs on an sm_103 device (GB300); other devices give
  *    DMPT_EUNSUPPORTED from dmpt_create().
  *  - Threads: a handle (its error text, events and internal streams) is
- *    used by one host thread at a time; separate handles, also on separate
- *    devices of one process, may be used from separate threads.  One-time
- *    per-device setup inside the library is thread-safe.
+ *    used by one host thread at a time, with one exception: single solves
+ *    (dmpt_sp2_response, _response2, _response_m, dmpt_sp2_backward,
+ *    dmpt_response_replay and dmpt_scc_response, without timing or autotune)
+ *    may run side by side on one handle from several threads, each with its
+ *    own stream and workspace; the error text is then that of whichever call
+ *    failed last.  Separate handles, also on separate devices of one process,
+ *    may be used from separate threads.  One-time per-device setup inside the
+ *    library is thread-safe.
  */
 #ifndef DMPT_H
 #define DMPT_H
@@ -226,9 +231,9 @@ dmpt_status dmpt_bounds(dmpt_handle h, const double* H, int64_t n, int64_t ld,
  *   info   host pointer, may be NULL.
  *   workspace / ws_bytes: caller scratch of dmpt_workspace_size() bytes.
  * The call issues all work on `stream`, at most two layers ahead of the
- * device (it follows the run through a word of mapped host memory that the
- * handle owns), and synchronises that stream; it returns when the outputs are
- * written.  Returns DMPT_ENOTCONV (outputs = last iterate) when
+ * device (it follows the run through a word of mapped host memory, one of the
+ * handle's for each running solve), and synchronises that stream; it returns
+ * when the outputs are written.  Returns DMPT_ENOTCONV (outputs = last iterate) when
  * max_layers is reached, DMPT_ENUMERIC on non-finite values or
  * eps_N <= eps_1 for 0 < n_occ < n.  With o->ckpt_every = 1 the workspace
  * (sized by dmpt_workspace_size with the same options) also keeps every S0

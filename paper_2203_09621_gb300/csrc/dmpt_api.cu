@@ -11,6 +11,9 @@
 #include <string.h>
 
 #include <algorithm>
+#include <condition_variable>
+#include <mutex>
+#include <optional>
 #include <vector>
 
 #include "dmpt_internal.cuh"
@@ -24,11 +27,14 @@ struct dmpt_ctx {
   std::vector<cudaEvent_t> joins;    // per-instance join events
   cudaStream_t origin = nullptr;     // capture / issue stream of batched solves
   cudaEvent_t fork = nullptr;
-  // mapped host word in which the decide steps of a running solve report
-  // (LayerFeed), its device address, and the number of the solve
-  volatile unsigned* progress = nullptr;
-  unsigned* progress_dev = nullptr;
-  unsigned solve = 0;
+  // mapped host words in which the decide steps of running solves report, one
+  // per solve (LayerFeed), their device address and the words in use (bits)
+  static constexpr int kWords = 64, kWordStride = 16;   // a 64-byte line each
+  volatile unsigned* words = nullptr;
+  unsigned* words_dev = nullptr;
+  std::mutex words_mu;
+  std::condition_variable words_free;
+  unsigned long long words_used = 0;
   // host-buffer pipeline: copy-in / copy-out streams and their events
   cudaStream_t copy_in = nullptr, copy_out = nullptr;
   cudaEvent_t ev_start = nullptr, ev_in[2] = {nullptr, nullptr}, ev_solved[2] = {nullptr, nullptr},
@@ -83,33 +89,49 @@ struct DeviceGuard {
 // launches.  (Polling by a device-to-host copy and a stream synchronisation
 // after every fourth layer left the GPU idle for 22-28 us each time: 0.2 of
 // 1.2 ms at n = 128.)  Launches that follow the end of a run exit at once.
+// Each running solve has a word of its own, so that threads which share a
+// handle can solve side by side; a solve that finds all of them taken waits.
+// The word goes back once the last step that may write it has.
 struct LayerFeed {
   dmpt_handle h;
   cudaStream_t s;
-  unsigned tag;
-  int ahead;
+  unsigned last = 0;   // code of the last step issued
+  int ahead, slot = 0;
   LayerFeed(dmpt_handle h_, cudaStream_t s_, int ahead_) : h(h_), s(s_), ahead(ahead_) {
-    tag = ++h->solve & 0x3FFFFFu;
+    std::unique_lock<std::mutex> lock(h->words_mu);
+    h->words_free.wait(lock, [&] { return ~h->words_used != 0; });
+    while (h->words_used >> slot & 1) ++slot;
+    h->words_used |= 1ull << slot;
+    *word() = 0;
   }
-  // code of the decide step of layer `layer` (1 .. DMPT_MAX_LAYERS)
-  unsigned code(int layer) const { return (tag << 10) | ((unsigned)layer << 1); }
+  ~LayerFeed() {
+    if ((*word() | 1u) != (last | 1u)) cudaStreamSynchronize(s);   // left early
+    std::lock_guard<std::mutex> lock(h->words_mu);
+    h->words_used &= ~(1ull << slot);
+    h->words_free.notify_one();
+  }
+  LayerFeed(const LayerFeed&) = delete;
+  LayerFeed& operator=(const LayerFeed&) = delete;
+  volatile unsigned* word() const { return h->words + slot * dmpt_ctx::kWordStride; }
+  unsigned* word_dev() const { return h->words_dev + slot * dmpt_ctx::kWordStride; }
+  // code of the decide step of layer `layer` (1 .. DMPT_MAX_LAYERS), to be issued now
+  unsigned code(int layer) { return last = (unsigned)layer << 1; }
   // Returns when the next layer may be issued or the run has ended (*done).
   cudaError_t wait(int launched, bool* done) const {
     for (unsigned it = 1;; ++it) {
-      const unsigned w = *h->progress;
-      const bool mine = (w >> 10) == tag;
-      if (mine && (w & 1u)) {
+      const unsigned w = *word();
+      if (w & 1u) {
         *done = true;
         return cudaSuccess;
       }
-      if (launched - (mine ? (int)((w >> 1) & 511u) : 0) < ahead) return cudaSuccess;
+      if (launched - (int)(w >> 1) < ahead) return cudaSuccess;
       if ((it & 4095u) == 0) {
         // the word lags only while work is pending; a failed stream ends the wait
         const cudaError_t e = cudaStreamQuery(s);
         if (e == cudaErrorNotReady) {
           (void)cudaGetLastError();   // not an error
         } else {
-          const unsigned w2 = *h->progress;
+          const unsigned w2 = *word();
           if (e != cudaSuccess) return e;
           if (w2 == w) return cudaErrorUnknown;
         }
@@ -241,14 +263,14 @@ dmpt_status replay_run(dmpt_handle h, const Layout& L, const double* H1, const d
   bool done = false;
   int64_t entries = 0;
   double pass_flops = 0.0;
-  const LayerFeed feed(h, s, layers_ahead(o));
+  LayerFeed feed(h, s, layers_ahead(o));
   while (launched < o->max_layers && !done) {
     if ((e = launch_layer_tc(L, workspace, s, o->timeout_s, o->accum_chunk, o->cta_pair,
                              o->k_snake, o->tile_band, &entries, &pass_flops, 0,
                              o->round_align)) != cudaSuccess)
       return cuda_fail(h, e, "replay layer");
     ++launched;
-    if ((e = launch_decide(L, workspace, kDecideReplayLayer, entries, s, h->progress_dev,
+    if ((e = launch_decide(L, workspace, kDecideReplayLayer, entries, s, feed.word_dev(),
                            feed.code(launched))) != cudaSuccess)
       return cuda_fail(h, e, "replay decide");
     if ((e = feed.wait(launched, &done)) != cudaSuccess) return cuda_fail(h, e, "replay loop");
@@ -388,18 +410,17 @@ dmpt_status dmpt_create(dmpt_handle* h, int device) {
   c->device = device;
   c->sm_count = prop.multiProcessorCount;
   DeviceGuard g(device);
-  void* word = nullptr;
-  void* word_dev = nullptr;
-  if (cudaHostAlloc(&word, sizeof(unsigned), cudaHostAllocMapped | cudaHostAllocPortable) !=
-          cudaSuccess ||
-      cudaHostGetDevicePointer(&word_dev, word, 0) != cudaSuccess) {
-    if (word) cudaFreeHost(word);
+  void* words = nullptr;
+  void* words_dev = nullptr;
+  constexpr size_t bytes = dmpt_ctx::kWords * dmpt_ctx::kWordStride * sizeof(unsigned);
+  if (cudaHostAlloc(&words, bytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess ||
+      cudaHostGetDevicePointer(&words_dev, words, 0) != cudaSuccess) {
+    if (words) cudaFreeHost(words);
     delete c;
     return DMPT_ECUDA;
   }
-  c->progress = (volatile unsigned*)word;
-  *c->progress = 0;
-  c->progress_dev = (unsigned*)word_dev;
+  c->words = (volatile unsigned*)words;
+  c->words_dev = (unsigned*)words_dev;
   *h = c;
   return DMPT_OK;
 }
@@ -413,7 +434,7 @@ dmpt_status dmpt_destroy(dmpt_handle h) {
     for (cudaStream_t st : h->streams) cudaStreamDestroy(st);
     if (h->origin) cudaStreamDestroy(h->origin);
     if (h->fork) cudaEventDestroy(h->fork);
-    if (h->progress) cudaFreeHost((void*)h->progress);
+    if (h->words) cudaFreeHost((void*)h->words);
     if (h->copy_in) cudaStreamDestroy(h->copy_in);
     if (h->copy_out) cudaStreamDestroy(h->copy_out);
     for (cudaEvent_t e : {h->ev_start, h->ev_in[0], h->ev_in[1], h->ev_solved[0], h->ev_solved[1],
@@ -527,7 +548,7 @@ static dmpt_status forward_impl(dmpt_handle h, const double* H, const double* H1
   int64_t entries = 0;
   double pass_flops = 0.0;
   bool done = false;
-  const LayerFeed feed(h, s, layers_ahead(o));
+  LayerFeed feed(h, s, layers_ahead(o));
   while (launched < max_layers && !done) {
     if (o->timing) cudaEventRecord(h->events[2 * launched], s);
     e = dual ? launch_layer_tc(L, workspace, s, o->timeout_s, o->accum_chunk, o->cta_pair,
@@ -537,7 +558,7 @@ static dmpt_status forward_impl(dmpt_handle h, const double* H, const double* H1
     if (e != cudaSuccess) return cuda_fail(h, e, "layer product");
     if (o->timing) cudaEventRecord(h->events[2 * launched + 1], s);
     ++launched;
-    if ((e = launch_decide(L, workspace, kDecideLayer, entries, s, h->progress_dev,
+    if ((e = launch_decide(L, workspace, kDecideLayer, entries, s, feed.word_dev(),
                            feed.code(launched))) != cudaSuccess)
       return cuda_fail(h, e, "decide(layer)");
     if (ckpt && (e = launch_ckpt_store(L, workspace, s)) != cudaSuccess)
@@ -1246,10 +1267,11 @@ static dmpt_status batch_impl(dmpt_handle h, int count, const double* const* H,
     }
   }
   int steps = grouped ? 0 : 1;
+  std::optional<LayerFeed> feed;
   if (grouped) {
     // a grouped launch and its decide step per layer, followed through the
     // mapped word (LayerFeed)
-    const LayerFeed feed(h, h->origin, layers_ahead(o));
+    feed.emplace(h, h->origin, layers_ahead(o));
     bool done = false;
     while (steps < o->max_layers && !done) {
       if ((e = launch_layer_tc_group(d_ginst, n_group, o->precision == DMPT_DUAL_BF16, d_gtimeout,
@@ -1257,10 +1279,10 @@ static dmpt_status batch_impl(dmpt_handle h, int count, const double* const* H,
                                      o->tile_band, h->sm_count, h->origin, n128)) != cudaSuccess)
         return cuda_fail(h, e, "batch layer");
       ++steps;
-      if ((e = launch_decide_group(d_gdec, n_group, d_gtimeout, d_gqueue, h->progress_dev,
-                                   feed.code(steps), h->origin)) != cudaSuccess)
+      if ((e = launch_decide_group(d_gdec, n_group, d_gtimeout, d_gqueue, feed->word_dev(),
+                                   feed->code(steps), h->origin)) != cudaSuccess)
         return cuda_fail(h, e, "batch decide");
-      if ((e = feed.wait(steps, &done)) != cudaSuccess) return cuda_fail(h, e, "batch loop");
+      if ((e = feed->wait(steps, &done)) != cudaSuccess) return cuda_fail(h, e, "batch loop");
     }
   } else {
     // one CUDA graph = one layer of every active instance, each on its own stream

@@ -602,6 +602,12 @@ _default_ctx: Optional[Context] = None
 
 
 def context(device: int = 0) -> Context:
+    """The process's shared Context of `device` (the last device asked for).
+
+    Single solves may run on it from several threads at once when each passes
+    its own `workspace` on its own stream (density() keeps one per call); the
+    Context's cached workspace, batches, host solves, timing and autotune are
+    for one thread at a time."""
     global _default_ctx
     if _default_ctx is None or _default_ctx.device != device:
         _default_ctx = Context(device)
