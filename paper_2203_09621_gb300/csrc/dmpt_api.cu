@@ -83,6 +83,14 @@ struct DeviceGuard {
   }
 };
 
+// Host memory is mapped and freed while the caller may be capturing a graph on
+// another stream: neither call is part of it.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The host side of a layer loop.  The host runs ahead of the device by at most
 // `ahead` layers: each decide step writes its layer number, and whether the
 // run has ended, to a word of mapped host memory, which the host reads between
@@ -410,6 +418,7 @@ dmpt_status dmpt_create(dmpt_handle* h, int device) {
   c->device = device;
   c->sm_count = prop.multiProcessorCount;
   DeviceGuard g(device);
+  RelaxedCapture rc;
   void* words = nullptr;
   void* words_dev = nullptr;
   constexpr size_t bytes = dmpt_ctx::kWords * dmpt_ctx::kWordStride * sizeof(unsigned);
@@ -429,6 +438,7 @@ dmpt_status dmpt_destroy(dmpt_handle h) {
   if (!h) return DMPT_EINVAL;
   {
     DeviceGuard g(h->device);
+    RelaxedCapture rc;
     for (cudaEvent_t e : h->events) cudaEventDestroy(e);
     for (cudaEvent_t e : h->joins) cudaEventDestroy(e);
     for (cudaStream_t st : h->streams) cudaStreamDestroy(st);
