@@ -274,8 +274,8 @@ dmpt_status replay_run(dmpt_handle h, const Layout& L, const double* H1, const d
   LayerFeed feed(h, s, layers_ahead(o));
   while (launched < o->max_layers && !done) {
     if ((e = launch_layer_tc(L, workspace, s, o->timeout_s, o->accum_chunk, o->cta_pair,
-                             o->k_snake, o->tile_band, &entries, &pass_flops, 0,
-                             o->round_align)) != cudaSuccess)
+                             o->k_snake, o->tile_band, LayerJobs{k, false}, &entries,
+                             &pass_flops, 0, o->round_align)) != cudaSuccess)
       return cuda_fail(h, e, "replay layer");
     ++launched;
     if ((e = launch_decide(L, workspace, kDecideReplayLayer, entries, s, feed.word_dev(),
@@ -558,12 +558,13 @@ static dmpt_status forward_impl(dmpt_handle h, const double* H, const double* H1
   int64_t entries = 0;
   double pass_flops = 0.0;
   bool done = false;
+  const LayerJobs jobs{order >= 2 ? order * k : k, true};
   LayerFeed feed(h, s, layers_ahead(o));
   while (launched < max_layers && !done) {
     if (o->timing) cudaEventRecord(h->events[2 * launched], s);
     e = dual ? launch_layer_tc(L, workspace, s, o->timeout_s, o->accum_chunk, o->cta_pair,
-                               o->k_snake, o->tile_band, &entries, &pass_flops, o->inject_stall,
-                               o->round_align)
+                               o->k_snake, o->tile_band, jobs, &entries, &pass_flops,
+                               o->inject_stall, o->round_align)
              : launch_layer_simt(L, workspace, s, &entries, &pass_flops);
     if (e != cudaSuccess) return cuda_fail(h, e, "layer product");
     if (o->timing) cudaEventRecord(h->events[2 * launched + 1], s);
@@ -998,8 +999,8 @@ dmpt_status dmpt_sp2_backward(dmpt_handle h, const double* G, int64_t n, int64_t
       for (int m = a + 1; m < b; ++m) {
         // no round alignment: the skipped leading items are never counted in
         if ((e = launch_layer_tc(L, workspace, s, o->timeout_s, fs.fwd_chunk, fs.fwd_cta_pair,
-                                 fs.fwd_k_snake, fs.fwd_band, &entries, &pass_flops, 0,
-                                 0)) != cudaSuccess)
+                                 fs.fwd_k_snake, fs.fwd_band, LayerJobs{0, true}, &entries,
+                                 &pass_flops, 0, 0)) != cudaSuccess)
           return cuda_fail(h, e, "recompute layer");
         if ((e = launch_recompute_step(L, workspace, true, m + 1 < b ? m + 1 : 0, a,
                                        rec_item_base, s)) != cudaSuccess)
@@ -1010,8 +1011,8 @@ dmpt_status dmpt_sp2_backward(dmpt_handle h, const double* G, int64_t n, int64_t
     }
     for (int m = b; m >= a + 1; --m) {
       if ((e = launch_layer_tc(L, workspace, s, o->timeout_s, o->accum_chunk, o->cta_pair,
-                               o->k_snake, o->tile_band, &entries, &pass_flops, 0,
-                               o->round_align)) != cudaSuccess)
+                               o->k_snake, o->tile_band, LayerJobs{1, false}, &entries,
+                               &pass_flops, 0, o->round_align)) != cudaSuccess)
         return cuda_fail(h, e, "adjoint layer");
       if ((e = launch_decide(L, workspace, kDecideAdjLayer, entries, s)) != cudaSuccess)
         return cuda_fail(h, e, "adjoint decide");
@@ -1212,8 +1213,9 @@ static dmpt_status batch_impl(dmpt_handle h, int count, const double* const* H,
     void* ws = base + offs[i];
     // the instances' layer kernels run side by side: no round alignment
     cudaError_t r = dual ? launch_layer_tc(L[i], ws, si, o->timeout_s, o->accum_chunk,
-                                           o->cta_pair, o->k_snake, o->tile_band, &entries[i],
-                                           &pass_flops[i], 0, /*round_align=*/0)
+                                           o->cta_pair, o->k_snake, o->tile_band,
+                                           LayerJobs{k, true}, &entries[i], &pass_flops[i], 0,
+                                           /*round_align=*/0)
                          : launch_layer_simt(L[i], ws, si, &entries[i], &pass_flops[i]);
     if (r != cudaSuccess) return r;
     return launch_decide(L[i], ws, kDecideLayer, entries[i], si);

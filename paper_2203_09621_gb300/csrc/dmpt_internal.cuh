@@ -298,14 +298,21 @@ cudaError_t launch_trivial(int64_t n, int k, int64_t ld, int full, double* P,
                            double* P1, cudaStream_t s);
 
 // ---- tensor-core path (kernels_tc.cu) ----
+// Jobs of a layer launch that run until the first of them converges: response
+// terms (of the layout's slots) and the square.  Only the tile width depends on
+// them; every width gives the same bits.
+struct LayerJobs {
+  int responses;
+  bool square;
+};
 // round_align: the pair kernel's producers keep their rounds in step (a
 // bounded wait, never an error); off where several instances' layer kernels
 // run at the same time, whose CTAs need not all be resident (dmpt_options::
 // round_align; always off on the per-instance batch path).
 cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double timeout_s,
                             int accum_chunk_k, int cta_pair, int k_snake, int band,
-                            int64_t* entries, double* pass_flops, int inject_stall = 0,
-                            int round_align = 1);
+                            const LayerJobs& jobs, int64_t* entries, double* pass_flops,
+                            int inject_stall = 0, int round_align = 1);
 int tc_tile();
 
 // ---- grouped layer products of a batch (kernels_tc.cu) ----

@@ -2340,7 +2340,7 @@ int pair_smem(int nt) {
   return nt == 64 ? PairTile<64>::SMEM : (nt == 128 ? PairTile<128>::SMEM : PairTile<BN>::SMEM);
 }
 
-// Tile width of the pair kernel for `tiles` 256 x 256 tiles of 1 + k jobs.
+// Tile width of the pair kernel for `tiles` 256 x 256 tiles of each job.
 // Measured time per layer in us of a whole solve, 256 / 128 / 64 wide:
 //   n = 128 k = 1   29 /  22 /  20       n = 2048 k = 1   84 /  74 / 106
 //   n = 768 k = 1   45 /  31 /  29       n = 2048 k = 3  155 / 150 / 224
@@ -2352,14 +2352,22 @@ int pair_smem(int nt) {
 // (it loads 24 KB per 32-wide block for half the products, and its MMAs issue
 // no faster than 0.24 us per block against 0.4), and its last epilogue is
 // about 14 blocks shorter.  The pairs take the items round-robin, responses
-// (two K passes) first, so pair 0 has the largest load.
-int pair_tile_width(int64_t tiles, int k, int64_t kblocks, int pairs) {
-  const int64_t items = tiles * (1 + k);
+// (two K passes; those of higher orders, which have more, are counted alike)
+// first, so pair 0 has the largest load.
+// The jobs are those that run, not the layout's slots: a density forward runs
+// the square alone, its backward one response, a replay the responses alone
+// (whole calls in ms, by the width for the slots and a square / by the jobs:
+// forward with a checkpoint every eight states n = 1280 1.09 / 1.02, 2560 2.52 /
+// 2.43, 3584 5.30 / 4.79; its backward 1.99 / 1.87, 5.51 / 5.28, 12.5 / 11.0;
+// replay n = 1536 k = 3 2.71 / 2.59, 2304 k = 1 3.58 / 3.38).
+int pair_tile_width(int64_t tiles, const LayerJobs& jobs, int64_t kblocks, int pairs) {
+  const int64_t items = tiles * (jobs.responses + (jobs.square ? 1 : 0));
   if (BN / 64 * items <= pairs) return 64;
   if (items > 8 * pairs) return BN;
   auto load = [&](int split) {
     int64_t passes = 0;
-    for (int64_t i = 0; i < split * items; i += pairs) passes += i < split * tiles * k ? 2 : 1;
+    for (int64_t i = 0; i < split * items; i += pairs)
+      passes += i < split * tiles * jobs.responses ? 2 : 1;
     return passes * kblocks;
   };
   return 3 * load(2) < 5 * (load(1) + 14) ? 128 : BN;
@@ -2498,8 +2506,8 @@ cudaError_t launch_layer_tc_group(const GroupInst* inst, int count, bool bf16, i
 
 cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double timeout_s,
                             int accum_chunk_k, int cta_pair, int k_snake, int band,
-                            int64_t* entries, double* pass_flops, int inject_stall,
-                            int round_align) {
+                            const LayerJobs& jobs, int64_t* entries, double* pass_flops,
+                            int inject_stall, int round_align) {
   using namespace tc;
   char* base = (char*)ws;
   const bool bf16 = L.precision == DMPT_DUAL_BF16;
@@ -2507,9 +2515,10 @@ cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double ti
   CUtensorMap mA, mB;
   const int sms = device_setup();
   if (sms == 0) return cudaErrorInvalidDevice;
-  // 256 x 256 tiles of every job (the jobs that run are only known on the device)
+  // 256 x 256 tiles of every slot; `jobs` of them run at first (which ones still
+  // do is only known on the device)
   const int64_t ptiles = num_pair_tiles(L.Np), pitems = ptiles * (1 + L.k);
-  const int nt = pair_tile_width(ptiles, L.k, k_blocks(L.n), sms / 2);
+  const int nt = pair_tile_width(ptiles, jobs, k_blocks(L.n), sms / 2);
   const int sk = cta_pair ? PairTile<BN>::SK : BK;
   if (!make_map(&mA, base + L.off_ops16, L.Np, slices, BM, bf16, sk) ||
       !make_map(&mB, base + L.off_ops16, L.Np, slices, cta_pair ? nt / 2 : BN, bf16, sk))
