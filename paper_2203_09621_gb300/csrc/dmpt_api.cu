@@ -11,9 +11,11 @@
 #include <string.h>
 
 #include <algorithm>
+#include <chrono>
 #include <condition_variable>
 #include <mutex>
 #include <optional>
+#include <thread>
 #include <vector>
 
 #include "dmpt_internal.cuh"
@@ -100,12 +102,23 @@ struct RelaxedCapture {
 // Each running solve has a word of its own, so that threads which share a
 // handle can solve side by side; a solve that finds all of them taken waits.
 // The word goes back once the last step that may write it has.
+// How the host waits follows the device's schedule flags, as a stream
+// synchronisation does: it reads the word in a loop, with yields where they say
+// so, and where they ask for blocking it synchronises the stream after every
+// `burst` layers instead.  By default it naps once a layer has taken kNapAfter
+// (an FP64 layer of n = 8192 takes seconds): a nap of 50 us ends within about
+// 0.1 ms, 2% of that, and the device has the next layer meanwhile.
 struct LayerFeed {
+  static constexpr std::chrono::microseconds kNapAfter{5000}, kNap{50}, kQuery{1000};
   dmpt_handle h;
   cudaStream_t s;
   unsigned last = 0;   // code of the last step issued
-  int ahead, slot = 0;
-  LayerFeed(dmpt_handle h_, cudaStream_t s_, int ahead_) : h(h_), s(s_), ahead(ahead_) {
+  unsigned flags = 0;  // the device's cudaDeviceSchedule* flag
+  int ahead, burst, slot = 0;
+  LayerFeed(dmpt_handle h_, cudaStream_t s_, int ahead_, int burst_)
+      : h(h_), s(s_), ahead(ahead_), burst(burst_) {
+    if (cudaGetDeviceFlags(&flags) != cudaSuccess) flags = 0;
+    flags &= cudaDeviceScheduleMask;
     std::unique_lock<std::mutex> lock(h->words_mu);
     h->words_free.wait(lock, [&] { return ~h->words_used != 0; });
     while (h->words_used >> slot & 1) ++slot;
@@ -126,24 +139,42 @@ struct LayerFeed {
   unsigned code(int layer) { return last = (unsigned)layer << 1; }
   // Returns when the next layer may be issued or the run has ended (*done).
   cudaError_t wait(int launched, bool* done) const {
-    for (unsigned it = 1;; ++it) {
+    using clock = std::chrono::steady_clock;
+    if (flags == cudaDeviceScheduleBlockingSync) {
+      if (launched % burst != 0) return cudaSuccess;
+      const cudaError_t e = cudaStreamSynchronize(s);
+      *done = e == cudaSuccess && (*word() & 1u);
+      return e;
+    }
+    clock::time_point start, query;   // of the wait, of the next look at the stream
+    for (unsigned it = 0;; ++it) {
       const unsigned w = *word();
       if (w & 1u) {
         *done = true;
         return cudaSuccess;
       }
       if (launched - (int)(w >> 1) < ahead) return cudaSuccess;
-      if ((it & 4095u) == 0) {
+      if ((it & 255u) != 0) continue;
+      const clock::time_point now = clock::now();
+      if (it == 0) {
+        start = now;
+        query = now + kQuery;
+      }
+      if (now >= query) {
         // the word lags only while work is pending; a failed stream ends the wait
         const cudaError_t e = cudaStreamQuery(s);
         if (e == cudaErrorNotReady) {
           (void)cudaGetLastError();   // not an error
         } else {
-          const unsigned w2 = *word();
           if (e != cudaSuccess) return e;
-          if (w2 == w) return cudaErrorUnknown;
+          if (*word() == w) return cudaErrorUnknown;
         }
+        query = now + kQuery;
       }
+      if (flags == cudaDeviceScheduleYield)
+        std::this_thread::yield();
+      else if (flags == cudaDeviceScheduleAuto && now - start >= kNapAfter)
+        std::this_thread::sleep_for(kNap);
     }
   }
 };
@@ -271,7 +302,7 @@ dmpt_status replay_run(dmpt_handle h, const Layout& L, const double* H1, const d
   bool done = false;
   int64_t entries = 0;
   double pass_flops = 0.0;
-  LayerFeed feed(h, s, layers_ahead(o));
+  LayerFeed feed(h, s, layers_ahead(o), o->sync_every);
   while (launched < o->max_layers && !done) {
     if ((e = launch_layer_tc(L, workspace, s, o->timeout_s, o->accum_chunk, o->cta_pair,
                              o->k_snake, o->tile_band, LayerJobs{k, false}, &entries,
@@ -559,7 +590,7 @@ static dmpt_status forward_impl(dmpt_handle h, const double* H, const double* H1
   double pass_flops = 0.0;
   bool done = false;
   const LayerJobs jobs{order >= 2 ? order * k : k, true};
-  LayerFeed feed(h, s, layers_ahead(o));
+  LayerFeed feed(h, s, layers_ahead(o), o->sync_every);
   while (launched < max_layers && !done) {
     if (o->timing) cudaEventRecord(h->events[2 * launched], s);
     e = dual ? launch_layer_tc(L, workspace, s, o->timeout_s, o->accum_chunk, o->cta_pair,
@@ -1283,7 +1314,7 @@ static dmpt_status batch_impl(dmpt_handle h, int count, const double* const* H,
   if (grouped) {
     // a grouped launch and its decide step per layer, followed through the
     // mapped word (LayerFeed)
-    feed.emplace(h, h->origin, layers_ahead(o));
+    feed.emplace(h, h->origin, layers_ahead(o), o->sync_every);
     bool done = false;
     while (steps < o->max_layers && !done) {
       if ((e = launch_layer_tc_group(d_ginst, n_group, o->precision == DMPT_DUAL_BF16, d_gtimeout,
