@@ -86,9 +86,10 @@ typedef struct {
   double c_d0;          /* factor of the Alg. 2 test (default 4.5)            */
   int operand_scaling;  /* 1: exact power-of-two scaling of the 16-bit halves
                            (FP16 range); 0: none (default 1)                  */
-  int sync_every;       /* batches: layers issued between host polls of the
-                           device state; single solves: most layers issued
-                           ahead of the device (at most 2) (default 4)        */
+  int sync_every;       /* layers issued between host polls of the device
+                           state where a batch runs one launch per instance
+                           (default 4); elsewhere the most layers issued ahead
+                           of the device: itself when above 4, else at most 2 */
   int timing;           /* 1: time every layer-product launch with CUDA events
                            on `stream` and report it in dmpt_info             */
   double timeout_s;     /* limit of any device-side spin wait, in seconds,
@@ -230,11 +231,11 @@ dmpt_status dmpt_bounds(dmpt_handle h, const double* H, int64_t n, int64_t ld,
  *   P1     device, k blocks n x n (ld) outputs.
  *   info   host pointer, may be NULL.
  *   workspace / ws_bytes: caller scratch of dmpt_workspace_size() bytes.
- * The call issues all work on `stream`, at most two layers ahead of the
- * device (it follows the run through a word of mapped host memory, one of the
- * handle's for each running solve), and synchronises that stream; it returns
- * when the outputs are written.  Returns DMPT_ENOTCONV (outputs = last iterate) when
- * max_layers is reached, DMPT_ENUMERIC on non-finite values or
+ * The call issues all work on `stream`, a few layers (o->sync_every) ahead of
+ * the device, and synchronises that stream; it follows the run through a word
+ * of mapped host memory, one of the handle's for each running solve, and
+ * returns when the outputs are written.  Returns DMPT_ENOTCONV (outputs = last
+ * iterate) when max_layers is reached, DMPT_ENUMERIC on non-finite values or
  * eps_N <= eps_1 for 0 < n_occ < n.  With o->ckpt_every = 1 the workspace
  * (sized by dmpt_workspace_size with the same options) also keeps every S0
  * layer state for dmpt_sp2_backward. */
@@ -326,8 +327,8 @@ dmpt_status dmpt_sp2_backward(dmpt_handle h, const double* G, int64_t n, int64_t
  * grouped tensor-core launch per layer step serves every instance from one
  * pool of tiles, claimed through a device-side queue, followed by one
  * batched decide launch; otherwise every instance's layer kernels run on an
- * internal stream of its own.  One CUDA graph holds a layer step and is
- * replayed until all instances have converged (finished instances add no
+ * internal stream of its own, and one CUDA graph holds such a step.  Steps
+ * are issued until all instances have converged (finished instances add no
  * work).  Each instance's results equal those of its own dmpt_sp2_response
  * call bit for bit; with o->group_tile_n = 128 that holds for instances whose
  * 256 x 256 tiles take one round of the CTA pairs, the others agree to rounding.
@@ -337,10 +338,11 @@ dmpt_status dmpt_sp2_backward(dmpt_handle h, const double* G, int64_t n, int64_t
  *   k           directions per instance (same for all), 0..DMPT_MAX_K.
  *   info        host array of `count` entries (may be NULL).
  *   workspace   dmpt_workspace_size_batch() bytes, 256-byte aligned.
- * Options: no tape (ckpt_every = 0) and no per-launch timing.  Synchronises
- * the issuing stream every o->sync_every layers; the caller's `stream` is
- * ordered before and after the batch.  Returns the first failing instance's
- * status (all instances are still written). */
+ * Options: no tape (ckpt_every = 0) and no per-launch timing.  Grouped launches
+ * are followed as those of a single solve; with one launch per instance the
+ * issuing stream is synchronised every o->sync_every layers.  The caller's
+ * `stream` is ordered before and after the batch.  Returns the first failing
+ * instance's status (all instances are still written). */
 size_t dmpt_workspace_size_batch(int count, const int64_t* n, int k, const dmpt_options* o);
 dmpt_status dmpt_sp2_response_batch(dmpt_handle h, int count, const double* const* H,
                                     const double* const* H1, int k, const int64_t* n,

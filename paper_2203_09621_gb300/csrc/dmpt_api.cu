@@ -226,10 +226,11 @@ bool valid_options(const dmpt_options* o) {
 // Layers the host may issue ahead of the device (LayerFeed).  Two keep the
 // device busy (issuing a layer takes about 4 us of host time); each further one
 // is a launch more that finds the run ended (three: 1.6 us per layer more at
-// n = 128 to 1000).
-constexpr int kLayersAhead = 2;
+// n = 128 to 1000).  A sync_every above its default of 4 asks for a longer
+// queue, for instance where the host thread may lose its core.
+constexpr int kLayersAhead = 2, kSyncDefault = 4;
 int layers_ahead(const dmpt_options* o) {
-  return o->sync_every < kLayersAhead ? o->sync_every : kLayersAhead;
+  return o->sync_every > kSyncDefault ? o->sync_every : std::min(o->sync_every, kLayersAhead);
 }
 
 // Workspace geometry for (n, k) under options o: response slots (at least
@@ -406,7 +407,7 @@ void dmpt_default_options(dmpt_options* o) {
   o->c_pt = 9.0;
   o->c_d0 = 4.5;
   o->operand_scaling = 1;
-  o->sync_every = 4;
+  o->sync_every = kSyncDefault;
   o->timing = 0;
   o->timeout_s = 2.0;
   o->ckpt_every = 0;

@@ -67,3 +67,21 @@ def test_schedule_flags_give_the_same_results(tmp_path):
                        env=env, timeout=300)
         results.append(torch.load(out))
     assert all(torch.equal(r, results[0]) for r in results)
+
+
+def test_sync_every_sets_how_far_the_host_runs_ahead():
+    """Layers of about 1 ms: the number issued beyond the last one that ran says
+    how long the queue was.  Results do not depend on it."""
+    n = 700
+    x = make_instance("ha", n, n // 2, (-2.0, -0.1), (0.1, 2.0), seed=9492)
+    ctx = dmpt.context(0)
+    H, H1 = (torch.from_numpy(a).to("cuda:0") for a in (x.H, x.H1))
+    P, P1, ref = ctx.sp2_response(H, H1, x.n_occ, precision="fp64")
+    for sync_every in (1, 2, 3, 5, 16, 100):
+        Ps, P1s, info = ctx.sp2_response(H, H1, x.n_occ, precision="fp64", sync_every=sync_every)
+        assert info.layers == ref.layers and torch.equal(Ps, P) and torch.equal(P1s, P1)
+        beyond = info.product_launches - info.layers
+        if sync_every <= 4:
+            assert 0 <= beyond <= min(sync_every, 2)
+        else:
+            assert 2 < beyond <= sync_every or info.product_launches == 100
