@@ -1102,6 +1102,25 @@ size_t dmpt_workspace_size_batch(int count, const int64_t* n, int k, const dmpt_
   return total;
 }
 
+// Tile width of a grouped batch: the one asked for, or by size (group_tile_n =
+// 0) 256 x 128 tiles, padding to 128, for batches of small instances.  Their four
+// accumulators keep the MMAs going during the tile epilogues, which pays until
+// operand traffic counts more (us, 256 / 128 wide: 64 instances of n = 64 to 512
+// 3931 / 3609, 8 of 256 to 1024 with k = 3 2567 / 2238, 32 of 1024 to 1100
+// 15595 / 15022, 12 of 900 to 1400 with k = 2 10581 / 10513, 16 of 1800 to 2048
+// 30950 / 32809).  An instance whose 256 x 256 tiles take one round of the CTA
+// pairs has the same bits at both widths (no backwards K sweeps).
+static int batch_tile_n(dmpt_handle h, int count, const int64_t* n, const int64_t* n_occ, int k,
+                        const dmpt_options* o) {
+  if (o->group_tile_n != 0) return o->group_tile_n;
+  for (int i = 0; i < count; ++i) {
+    const int64_t tb = (n[i] + kPad - 1) / kPad;
+    const bool active = n_occ[i] > 0 && n_occ[i] < n[i];
+    if (active && (tb > 5 || tb * (tb + 1) / 2 * (1 + k) > h->sm_count / 2)) return 256;
+  }
+  return 128;
+}
+
 // path: -1 = the default rule (grouped launch for dual forms on CTA pairs, tile
 // width by size),
 // 0 = grouped, 1 = one launch per instance on its own stream, 3 = grouped on
@@ -1160,21 +1179,8 @@ static dmpt_status batch_impl(dmpt_handle h, int count, const double* const* H,
   // instances (GroupInst table, batched decide); otherwise one launch per
   // instance on its own stream
   const bool can_group = dual && o->cta_pair && o->order == 1 && n_act > 0 && n_act <= kGroupMax;
-  // 256 x 128 tiles, padding to 128: where asked for, and by default
-  // (group_tile_n = 0) for batches of small instances.  Their four accumulators
-  // keep the MMAs going during the tile epilogues, which pays until operand
-  // traffic counts more (us, 256 / 128 wide: 64 instances of n = 64 to 512
-  // 3931 / 3609, 8 of 256 to 1024 with k = 3 2567 / 2238, 32 of 1024 to 1100
-  // 15595 / 15022, 12 of 900 to 1400 with k = 2 10581 / 10513, 16 of 1800 to 2048
-  // 30950 / 32809).  An instance whose 256 x 256 tiles take one round of the CTA
-  // pairs has the same bits at both widths (no backwards K sweeps).
-  bool narrow = true;
-  for (int i = 0; i < count; ++i) {
-    const int64_t tb = (n[i] + kPad - 1) / kPad;
-    if (active[i] && (tb > 5 || tb * (tb + 1) / 2 * (1 + k) > h->sm_count / 2)) narrow = false;
-  }
-  const int gtn = o->group_tile_n != 0 ? o->group_tile_n : (narrow ? 128 : 256);
-  const bool n128 = (path == 3 || (path == -1 && gtn == 128)) && can_group;
+  const bool n128 =
+      (path == 3 || (path == -1 && batch_tile_n(h, count, n, n_occ, k, o) == 128)) && can_group;
   size_t off = batch_scratch_bytes(count);
   for (int i = 0; i < count; ++i) {
     L[i] = layout_for(n[i], k, o, n128 ? 128 : kPad);
@@ -1447,10 +1453,10 @@ dmpt_status dmpt_sp2_response_batch(dmpt_handle h, int count, const double* cons
         count >= 1 && n != nullptr))
     return batch_impl(h, count, H, H1, k, n, ld, n_occ, o, P, P1, info, workspace, ws_bytes,
                       stream, -1);
-  // autotuned batch: the grouped launch on CTA pairs with 256 x 256 or
-  // 256 x 128 tiles, or one launch per instance with 256 x 256 (CTA-pair) or
-  // 128 x 256 (single-CTA) tiles; chosen once per batch signature by timing a
-  // short probe of each
+  // autotuned batch: the grouped launch on CTA pairs with 256 x 256 (0) or
+  // 256 x 128 tiles (3), or one launch per instance with 256 x 256 (CTA-pair, 1)
+  // or 128 x 256 (single-CTA, 2) tiles; chosen once per batch signature by timing
+  // short probes of each.
   std::vector<int64_t> sig(count);
   for (int i = 0; i < count; ++i) sig[i] = n[i] >= 1 ? make_layout(n[i], k, o->precision).Np : 0;
   std::sort(sig.begin(), sig.end());
@@ -1466,9 +1472,17 @@ dmpt_status dmpt_sp2_response_batch(dmpt_handle h, int count, const double* cons
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
       return cuda_fail(h, cudaGetLastError(), "batch autotune events");
     dmpt_options p = t;
-    p.max_layers = 3;
-    double best_ms = 1e300;
-    for (int rep = 0; rep < 2; ++rep) {   // the first round warms every path up
+    // The time per layer is the difference of two probes, 1 and 3 layers long:
+    // the set-up and the outputs, which differ with the padding, are half of a
+    // 3-layer probe and a tenth of a solve.  The first layers tell a few per cent
+    // at best (8 instances of n = 1500 to 2500, 256 / 128 wide: 0.41 / 0.40 ms per
+    // layer over the first two, 16.4 / 17.3 ms for the solve), so the default
+    // stays unless another path is 5% faster per layer.
+    constexpr int kProbe[3] = {1, 1, 3};   // the first round warms every path up
+    constexpr float kGain = 0.95f;
+    float ms[3][4] = {};
+    for (int rep = 0; rep < 3; ++rep) {
+      p.max_layers = kProbe[rep];
       for (int cand = 0; cand < 4; ++cand) {
         p.cta_pair = cand == 2 ? 0 : 1;
         cudaEventRecord(e0, s);
@@ -1481,17 +1495,22 @@ dmpt_status dmpt_sp2_response_batch(dmpt_handle h, int count, const double* cons
           cudaEventDestroy(e1);
           return st;
         }
-        float ms = 0.f;
-        if (cudaEventSynchronize(e1) == cudaSuccess &&
-            cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && rep == 1 && ms < best_ms) {
-          best_ms = ms;
-          path = cand;
-        }
+        if (cudaEventSynchronize(e1) != cudaSuccess ||
+            cudaEventElapsedTime(&ms[rep][cand], e0, e1) != cudaSuccess)
+          ms[rep][cand] = rep == 2 ? INFINITY : 0.0f;
       }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (path < 0) path = 0;
+    const int base = o->cta_pair == 0 ? 2
+                                      : (batch_tile_n(h, count, n, n_occ, k, o) == 128 ? 3 : 0);
+    path = base;
+    float best = kGain * (ms[2][base] - ms[1][base]);
+    for (int cand = 0; cand < 4; ++cand)
+      if (cand != base && ms[2][cand] - ms[1][cand] < best) {
+        best = ms[2][cand] - ms[1][cand];
+        path = cand;
+      }
     h->batch_tune.push_back({sig, k, o->precision, path});
     h->err[0] = 0;
   }
