@@ -3,9 +3,10 @@
 //
 // The host only issues launches.  Each layer is one product kernel (SIMT for
 // FP64 / FP32, tcgen05 for the dual forms) followed by the one-block decide
-// kernel that applies Algorithms 2 and 3 on the device.  Every
-// `sync_every` layers the host reads the device "done" flag; launches that
-// follow a finished run exit at once.
+// kernel that applies Algorithms 2 and 3 on the device and reports to a word of
+// mapped host memory (LayerFeed); launches that follow a finished run exit at
+// once.  Batches on one launch per instance poll the device's flags every
+// `sync_every` layers.
 #include <cuda_runtime.h>
 #include <stdio.h>
 #include <string.h>

@@ -313,7 +313,6 @@ cudaError_t launch_layer_tc(const Layout& L, void* ws, cudaStream_t s, double ti
                             int accum_chunk_k, int cta_pair, int k_snake, int band,
                             const LayerJobs& jobs, int64_t* entries, double* pass_flops,
                             int inject_stall = 0, int round_align = 1);
-int tc_tile();
 
 // ---- grouped layer products of a batch (kernels_tc.cu) ----
 // One instance of a grouped launch: everything the pair kernel takes as

@@ -1,10 +1,12 @@
 // Element-wise kernels, device-side control of Algorithms 1-3, and the SIMT
 // (FP64 / FP32) layer product with its fused epilogue.
 //
-// Matrices inside the workspace are n x n zero-padded to Np x Np (Np a
-// multiple of 256).  Zero padding is invariant under the SP2 layers
-// (0^2 = 0, 2*0 - 0^2 = 0) and adds nothing to traces or norms, so the
-// product kernels need no bounds checks.
+// Matrices inside the workspace are n x n in a stride of Np, the multiple of 256
+// (128 on the 256 x 128 tiles of a batch) at or above n.  The initial kernels
+// write all Np x Np elements, zeros outside the matrix; zeros are invariant
+// under the SP2 layers (0^2 = 0, 2*0 - 0^2 = 0) and add nothing to traces or
+// norms.  The layer products work on the blocks that hold rows and columns < n
+// (the FP64 form on those elements alone), so what lies beyond is not kept up.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math.h>
@@ -961,7 +963,7 @@ cudaError_t launch_decide(const Layout& L, void* ws, int mode, int64_t entries, 
 // to the elements with row <= col, stores them at (r, c) and (c, r) in the
 // other ping-pong buffer, and reduces the Alg. 2 / 3 norms in FP64.
 
-template <typename T, int TM>
+template <int TM>
 __device__ __forceinline__ int frag_index(int t, int m) {
   // the TM rows (cols) of a thread: two runs of TM/2 contiguous elements,
   // the second BT/2 after the first
@@ -1015,17 +1017,17 @@ __device__ __forceinline__ void cp_async_wait() {
 // operand slabs (BK x BT, rows padded by one 16-byte chunk), then the
 // block's reduction array.
 constexpr int SIMT_STAGES = 3;
-template <typename T, int TM, int BK>
+template <int TM, int BK>
 constexpr int simt_smem_bytes() {
-  return SIMT_STAGES * 2 * BK * (16 * TM + 16 / (int)sizeof(T)) * (int)sizeof(T) + 4 * 256 * 8;
+  return SIMT_STAGES * 2 * BK * (16 * TM + 4) * (int)sizeof(float) + 4 * 256 * 8;
 }
 
-template <typename T, int TM, int BK>
+template <int TM, int BK>
 __global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
-    layer_simt_kernel(State* st, T* __restrict__ master, int64_t n, int64_t Np, int k,
+    layer_simt_kernel(State* st, float* __restrict__ master, int64_t n, int64_t Np, int k,
                       double* __restrict__ partials, int64_t ptiles) {
   constexpr int BT = 16 * TM;
-  constexpr int VW = 16 / (int)sizeof(T);      // elements per 16-byte copy
+  constexpr int VW = 4;                        // elements per 16-byte copy
   constexpr int LD = BT + VW;                  // padded row of a slab
   constexpr int CPR = BT / VW;                 // copies per slab row
   constexpr int NCP = BK * CPR / 256;          // copies per thread per slab
@@ -1034,8 +1036,8 @@ __global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
   // stage s: As = slab of the A operand, Bs = slab of the B operand, each
   // BK rows (K index) x BT columns (output rows / columns of the tile)
   extern __shared__ __align__(16) uint8_t simt_smem[];
-  T* slabs = reinterpret_cast<T*>(simt_smem);
-  double* red = reinterpret_cast<double*>(simt_smem + SIMT_STAGES * 2 * BK * LD * sizeof(T));
+  float* slabs = reinterpret_cast<float*>(simt_smem);
+  double* red = reinterpret_cast<double*>(simt_smem + SIMT_STAGES * 2 * BK * LD * sizeof(float));
 
   pdl_wait();   // no pdl_launch(): see layer_fp64_kernel
   if (st->done) return;
@@ -1057,15 +1059,17 @@ __global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
   const size_t mat = (size_t)Np * Np;
   const int cur0 = st->cur0;
   const int cur = job == 0 ? cur0 : st->cur1[job - 1];
-  const T* Sj = master + (size_t)(cur * (1 + k) + job) * mat;   // the job's own slot
-  T* out = master + (size_t)((cur ^ 1) * (1 + k) + job) * mat;
+  const float* Sj = master + (size_t)(cur * (1 + k) + job) * mat;   // the job's own slot
+  float* out = master + (size_t)((cur ^ 1) * (1 + k) + job) * mat;
 
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
   // column pairs (2 j, 2 j + 1) of the thread's tile, packed: one product per
-  // FMA fills the issue slots, and the shared-memory reads come on top.  The
-  // busiest SM's FMA pipe is now active in 94% of its cycles (n = 2560); what is
-  // left is the last wave.  n = 4096 k = 1 layer 3.80 -> 3.53 ms.
+  // FMA fills the issue slots, and the shared-memory reads come on top.  n = 4096
+  // k = 1 layer 3.80 -> 3.53 ms.  While an SM has blocks its FMA pipe is active in
+  // 80% of the cycles (four warps per scheduler, which at times all wait for
+  // operand reads or the barrier of a K step), and at n = 4096 the SMs have
+  // blocks for 95% of the layer (n = 2560: 78% and 83%).
   f32x2 acc2[TM][TM / 2];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
@@ -1084,13 +1088,13 @@ __global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
     // copies that land in shared memory already K-major.
     int mA, mB;
     simt_job_operands(job, pass, k1, &mA, &mB);
-    const T* A = master + (size_t)((mA == 0 ? cur0 : st->cur1[mA - 1]) * (1 + k) + mA) * mat +
+    const float* A = master + (size_t)((mA == 0 ? cur0 : st->cur1[mA - 1]) * (1 + k) + mA) * mat +
                  (size_t)I * BT;
-    const T* B = master + (size_t)((mB == 0 ? cur0 : st->cur1[mB - 1]) * (1 + k) + mB) * mat +
+    const float* B = master + (size_t)((mB == 0 ? cur0 : st->cur1[mB - 1]) * (1 + k) + mB) * mat +
                  (size_t)J * BT;
     auto load = [&](int stage, int kb) {
-      T* as = slabs + (size_t)stage * 2 * BK * LD;
-      T* bs = as + BK * LD;
+      float* as = slabs + (size_t)stage * 2 * BK * LD;
+      float* bs = as + BK * LD;
 #pragma unroll
       for (int v = 0; v < NCP; ++v) {
         const int idx = tid + 256 * v;
@@ -1115,26 +1119,26 @@ __global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
         if (nx < nkb) load(nx % SIMT_STAGES, nx * BK);
         cp_async_commit();
       }
-      const T* as = slabs + (size_t)(it % SIMT_STAGES) * 2 * BK * LD;
-      const T* bs = as + BK * LD;
+      const float* as = slabs + (size_t)(it % SIMT_STAGES) * 2 * BK * LD;
+      const float* bs = as + BK * LD;
 #pragma unroll
       for (int kk = 0; kk < BK; ++kk) {
-        T a[TM];
+        float a[TM];
         f32x2 b[TM / 2];
 #pragma unroll
-        for (int m = 0; m < TM; ++m) a[m] = as[kk * LD + frag_index<T, TM>(ty, m)];
+        for (int m = 0; m < TM; ++m) a[m] = as[kk * LD + frag_index<TM>(ty, m)];
         if constexpr (TM == 8) {
 #pragma unroll
           for (int m = 0; m < TM / 2; m += 2) {
             const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(
-                bs + kk * LD + frag_index<T, TM>(tx, 2 * m));
+                bs + kk * LD + frag_index<TM>(tx, 2 * m));
             b[m] = v.x;
             b[m + 1] = v.y;
           }
         } else {
 #pragma unroll
           for (int m = 0; m < TM / 2; ++m)
-            b[m] = *reinterpret_cast<const f32x2*>(bs + kk * LD + frag_index<T, TM>(tx, 2 * m));
+            b[m] = *reinterpret_cast<const f32x2*>(bs + kk * LD + frag_index<TM>(tx, 2 * m));
         }
 #pragma unroll
         for (int i = 0; i < TM; ++i) {
@@ -1148,8 +1152,8 @@ __global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
   }
 
   // ---- fused epilogue
-  const T sg = (T)st->sigma_cur;
-  const T om = (T)1 - sg;
+  const float sg = (float)st->sigma_cur;
+  const float om = 1.0f - sg;
   const bool write = job == 0 ? st->plan_write0 != 0 : true;
   double tr = 0.0, bad = 0.0;
   // ||S_new||_F^2 and ||S_old - X||_F^2 as exact FP32 products summed with
@@ -1158,19 +1162,19 @@ __global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
   float fn_s = 0.0f, fn_c = 0.0f, fd_s = 0.0f, fd_c = 0.0f;
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
-    const int64_t r = (int64_t)I * BT + frag_index<T, TM>(ty, i);
+    const int64_t r = (int64_t)I * BT + frag_index<TM>(ty, i);
 #pragma unroll
     for (int j = 0; j < TM; ++j) {
-      const int64_t c = (int64_t)J * BT + frag_index<T, TM>(tx, j);
+      const int64_t c = (int64_t)J * BT + frag_index<TM>(tx, j);
       if (r > c) continue;  // owned by the mirrored element
       float x01[2];
       unpack2(acc2[i][j / 2], x01[0], x01[1]);
-      const T x = x01[j % 2];
-      const T old = Sj[(size_t)r * Np + c];
-      if (!isfinite((double)x)) bad += 1.0;
-      const T nw = sg * x + om * old;
+      const float x = x01[j % 2];
+      const float old = Sj[(size_t)r * Np + c];
+      if (!isfinite(x)) bad += 1.0;
+      const float nw = sg * x + om * old;
       const float w = (r == c) ? 1.0f : 2.0f;
-      const float dd = (float)old - (float)x;
+      const float dd = old - x;
       {
         const float p = w * dd * dd;
         const float e = w * fmaf(dd, dd, -dd * dd);
@@ -1180,9 +1184,8 @@ __global__ void __launch_bounds__(256, TM == 8 ? 2 : 4)
         fd_s = tt;
       }
       if (write) {
-        const float n1 = (float)nw;
-        const float p = w * n1 * n1;
-        const float e = w * fmaf(n1, n1, -n1 * n1);
+        const float p = w * nw * nw;
+        const float e = w * fmaf(nw, nw, -nw * nw);
         const float tt = fn_s + p;
         const float bp = tt - fn_s;
         fn_c += (fn_s - (tt - bp)) + (p - bp) + e;
@@ -1458,12 +1461,12 @@ static void simt_setup() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return;
   std::call_once(once[dev], [] {
-    cudaFuncSetAttribute(layer_simt_kernel<float, 8, 16>,
+    cudaFuncSetAttribute(layer_simt_kernel<8, 16>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         simt_smem_bytes<float, 8, 16>());
-    cudaFuncSetAttribute(layer_simt_kernel<float, 4, 16>,
+                         simt_smem_bytes<8, 16>());
+    cudaFuncSetAttribute(layer_simt_kernel<4, 16>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         simt_smem_bytes<float, 4, 16>());
+                         simt_smem_bytes<4, 16>());
   });
 }
 
@@ -1485,14 +1488,14 @@ cudaError_t launch_layer_simt(const Layout& L, void* ws, cudaStream_t s, int64_t
     if (e != cudaSuccess) return e;
     if (pass_flops) *pass_flops = (double)tiles * bt * bt * (double)L.n * 2.0;
   } else {
-    constexpr int smem8 = simt_smem_bytes<float, 8, 16>(), smem4 = simt_smem_bytes<float, 4, 16>();
+    constexpr int smem8 = simt_smem_bytes<8, 16>(), smem4 = simt_smem_bytes<4, 16>();
     static_assert(2 * smem8 <= 227 * 1024 && 4 * smem4 <= 227 * 1024, "blocks per SM");
     simt_setup();
     const int bt = fp32_tile(L.n, L.k);
     const int64_t tb = (L.n + bt - 1) / bt;
     tiles = tb * (tb + 1) / 2;
     const cudaError_t e = launch_pdl(
-        bt == 128 ? layer_simt_kernel<float, 8, 16> : layer_simt_kernel<float, 4, 16>,
+        bt == 128 ? layer_simt_kernel<8, 16> : layer_simt_kernel<4, 16>,
         dim3((unsigned)tiles, 1 + L.k), dim3(256), bt == 128 ? smem8 : smem4, s, st,
         (float*)(base + L.off_master), L.n, L.Np, L.k, partials, L.partial_tiles);
     if (e != cudaSuccess) return e;

@@ -247,32 +247,12 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
       : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-        "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // FP16 / BF16 rounding (round to nearest even) used by the dual split.
 template <bool BF>
 struct Cvt;
 template <>
 struct Cvt<false> {
   using T = __half;
-  static __device__ __forceinline__ T to(float x) { return __float2half_rn(x); }
-  static __device__ __forceinline__ float from(T h) { return __half2float(h); }
   static __device__ __forceinline__ uint32_t pack(float a, float b) {   // a in the low half
     const __half2 v = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&v);
@@ -286,8 +266,6 @@ struct Cvt<false> {
 template <>
 struct Cvt<true> {
   using T = __nv_bfloat16;
-  static __device__ __forceinline__ T to(float x) { return __float2bfloat16_rn(x); }
-  static __device__ __forceinline__ float from(T h) { return __bfloat162float(h); }
   static __device__ __forceinline__ uint32_t pack(float a, float b) {   // a in the low half
     const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&v);
@@ -414,12 +392,6 @@ __device__ __forceinline__ int chunk_pass(int c, int cpp, int passes, bool rev) 
 // adjoint); S1_j from its ping-pong slot.
 __device__ __forceinline__ int zop(int m, int buf, int part, int k, int z0) {
   return m == 0 ? z0 + part : zslice(buf, m, part, k);
-}
-
-// Bit pattern of a 16-bit float (FP16 or BF16).
-template <class H16>
-__device__ __forceinline__ uint32_t h16_bits(H16 x) {
-  return (uint32_t)(*reinterpret_cast<const uint16_t*>(&x));
 }
 
 // (s, c) += (s2, c2): sums held as s + c, the rounding of s kept in c (TwoSum)
@@ -713,10 +685,11 @@ static_assert(kQTrace == 0 && kQFroNew == 1 && kQFroDiff == 2 && kQBad == 3 && E
 
 template <bool BF16>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
-    layer_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-                    State* st, float* __restrict__ master, uint16_t* __restrict__ ops,
-                    int64_t Np, int k, double* __restrict__ partials, int64_t ptiles,
-                    uint64_t limit_ns, int chunk, int inject_stall) {
+    layer_tc_kernel(const __grid_constant__ CUtensorMap mapA,
+                    const __grid_constant__ CUtensorMap mapB, State* st,
+                    float* __restrict__ master, uint16_t* __restrict__ ops, int64_t Np, int k,
+                    double* __restrict__ partials, int64_t ptiles, uint64_t limit_ns, int chunk,
+                    int inject_stall) {
   using CV = Cvt<BF16>;
   using H16 = typename CV::T;
   extern __shared__ uint8_t smem_raw[];
@@ -913,7 +886,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
     }
   } else if (warp >= EPI_WARP0) {
-    // ================= epilogue (warps 4..11) =================
+    // ================= epilogue (warps 2..9) =================
     // Thread = one row of the tile (TMEM lane) and one half of its columns.
     const int q = warp & 3;                 // TMEM lane quadrant of this warp
     const int half = (warp - EPI_WARP0) >> 2;  // column half: 0 -> 0..127, 1 -> 128..255
@@ -956,7 +929,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           uint32_t x[16];
           tmem_ld16(ta + 16 * cc, x);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) sum[16 * cc + i] = fmaf(__uint_as_float(x[i]), u, sum[16 * cc + i]);
+          for (int i = 0; i < 16; ++i)
+            sum[16 * cc + i] = fmaf(__uint_as_float(x[i]), u, sum[16 * cc + i]);
         }
         if (ch + 1 == nchunks) break;   // keep the last chunk's buffer
         fence_before();
@@ -999,12 +973,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if (lane == 0) mbar_arrive(bar_tempty + 8 * ab);
       };
       rolled_tile_epilogue<CV, 8, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0,
-                                         kblocks * BK, sg, om, scale_new, write, olds, epi_block(red), ts, release);
+                                         kblocks * BK, sg, om, scale_new, write, olds,
+                                         epi_block(red), ts, release);
       if (++ab == 2) {
         ab = 0;
         abphase ^= 1;
       }
-      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, partials + ((size_t)job * ptiles + t) * kNQ);
+      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane,
+                    partials + ((size_t)job * ptiles + t) * kNQ);
     }
   }
 
@@ -1024,10 +1000,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 // (output columns) 128 r .. 128 r + 127; the leader (rank 0) issues
 // M = 256, N = 256 MMAs that read A from each CTA's own shared memory and B
 // from both, and each CTA's tensor memory receives its 128 rows of the
-// accumulator.  Per SM this halves the operand bytes loaded per MMA
-// (32 KB per 6 MMAs instead of 48 KB).
-//   full[s]   leader only: leader producer's expect_tx(64 KB); both CTAs'
-//             TMA loads complete their bytes on it
+// accumulator.  Per SM this cuts the operand bytes loaded for 32 columns of K
+// and 256 columns of the tile from 48 to 32 KB.
+//   full[s]   leader only: leader producer's expect_tx of both CTAs' stages;
+//             both CTAs' TMA loads complete their bytes on it
 //   empty[s]  each CTA: the leader's MMA commit arrives on both (multicast)
 //   tfull[b]  each CTA: leader's commit, multicast
 //   tempty[b] leader only: 16 arrivals (8 epilogue warps per CTA)
@@ -1133,8 +1109,8 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(leader_bar)
       : "memory");
 }
-__device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                             uint32_t accumulate) {
+__device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a, uint64_t b,
+                                             uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
@@ -1172,13 +1148,11 @@ struct RingPos {
 // pair leader's full barrier.  False when a bounded wait expired or the CTA
 // aborted.
 template <int NT>
-__device__ __forceinline__ bool produce_item(RingPos& rg, const CUtensorMap* map,
-                                             const CUtensorMap* mapB, const State* st, int job, int passes, int k,
-                                             int k1, int cur0, int z0c, int rowA, int rowB,
-                                             int kblocks, bool rev, bool leader, uint32_t ring,
-                                             uint32_t bar_full, uint32_t bar_empty,
-                                             uint32_t lead_full, uint64_t limit_ns,
-                                             volatile int* abort_flag, int* timeout_global) {
+__device__ __forceinline__ bool produce_item(
+    RingPos& rg, const CUtensorMap* map, const CUtensorMap* mapB, const State* st, int job,
+    int passes, int k, int k1, int cur0, int z0c, int rowA, int rowB, int kblocks, bool rev,
+    bool leader, uint32_t ring, uint32_t bar_full, uint32_t bar_empty, uint32_t lead_full,
+    uint64_t limit_ns, volatile int* abort_flag, int* timeout_global) {
   using PT = PairTile<NT>;
   for (int pp = 0; pp < passes; ++pp) {
     const int pass = rev ? passes - 1 - pp : pp;
@@ -1237,10 +1211,10 @@ __device__ __forceinline__ void producer_drain(RingPos rg, int stages, uint32_t 
 template <bool BF16, int NT>
 __device__ __forceinline__ bool mma_item(RingPos& rg, RingPos& tb, int passes, int kblocks,
                                          int chunk, int cp0, bool rev, int cols,
-                                         uint32_t tmem_base, uint32_t ring, uint32_t bar_full, uint32_t bar_empty,
-                                         uint32_t bar_tfull, uint32_t bar_tempty,
-                                         uint64_t limit_ns, volatile int* abort_flag,
-                                         int* timeout_global) {
+                                         uint32_t tmem_base, uint32_t ring, uint32_t bar_full,
+                                         uint32_t bar_empty, uint32_t bar_tfull,
+                                         uint32_t bar_tempty, uint64_t limit_ns,
+                                         volatile int* abort_flag, int* timeout_global) {
   using PT = PairTile<NT>;
   const uint32_t idesc = make_idesc_m256(BF16 ? 1 : 0, cols);
   constexpr int H = PT::SK / BK;   // blocks per stage
@@ -1326,7 +1300,8 @@ __device__ __forceinline__ void round_start(unsigned* ctr, int64_t round, int64_
 
 // Tile epilogue of the pair kernel: after a tile's last chunk the sums are
 // written back into that chunk's tensor-memory buffer and read 16 columns at
-// a time by rolled_tile_epilogue (no register spills, little code per tile);
+// a time by rolled_tile_epilogue (little code per tile; one register spilled at
+// 256 columns, none below);
 // the buffer returns to the MMA after that loop, so the MMA runs one chunk
 // ahead of the epilogue during it.
 template <bool BF16, int NT>
@@ -1525,9 +1500,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         int I2, J;
         pair_tile_banded(it % tiles, (int)(Np / BN), band, &I2, &J);
         if (tile_cols(J * BN + (int)(v % SP) * NT, NT, cend) == 0) {   // nothing in the matrix
+          const size_t e = 2 * (SP * (size_t)(it % tiles) + v % SP) + rank;
           tile_sums_out(TileSums(), red, seq++, warp - EPI_WARP0, lane,
-                        partials +
-                            ((size_t)job * ptiles + 2 * (SP * (size_t)(it % tiles) + v % SP) + rank) * kNQ);
+                        partials + ((size_t)job * ptiles + e) * kNQ);
           continue;
         }
         const int r = I2 * 2 * BM + (int)rank * BM + rloc;
@@ -1556,7 +1531,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
           uint32_t x[16];
           tmem_ld16(ta + 16 * cc, x);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) sum[16 * cc + i] = fmaf(__uint_as_float(x[i]), u, sum[16 * cc + i]);
+          for (int i = 0; i < 16; ++i)
+            sum[16 * cc + i] = fmaf(__uint_as_float(x[i]), u, sum[16 * cc + i]);
         }
         if (ch + 1 == nchunks) break;   // keep the last chunk's buffer
         fence_before();
@@ -1594,7 +1570,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab.idx);
       };
       rolled_tile_epilogue<CV, NT / 32, NT < BN>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r,
-                                                 c0, cend, sg, om, scale_new, write, olds, epi_block(red), ts, release);
+                                                 c0, cend, sg, om, scale_new, write, olds,
+                                                 epi_block(red), ts, release);
       ab.next(PT::ACC);
       tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane,
                     partials + ((size_t)job * ptiles + 2 * (SP * (size_t)t + v % SP) + rank) * kNQ);
@@ -1814,7 +1791,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const int64_t items = first[count];
   const unsigned epoch = *(volatile unsigned*)&gq->epoch;   // fixed during the launch
 
-
   if (items == 0) {
     // every instance has ended
   } else if (warp == 0) {
@@ -1868,8 +1844,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         pair_tile_banded((unsigned)itm.t, (int)(inst[itm.inst].Np / BN), band, &I2, &J);
         ok = mma_item<BF16, BN>(rg, tb, itm.passes, itm.kblocks, chunk, itm.cp0, itm.rev,
                                 tile_cols(J * BN, BN, itm.kblocks * BK),
-                            tmem_base, ring, bar_full, bar_empty, bar_tfull, bar_tempty, limit_ns,
-                            abort_flag, timeout_global);
+                                tmem_base, ring, bar_full, bar_empty, bar_tfull, bar_tempty,
+                                limit_ns, abort_flag, timeout_global);
       }
       if (elect_one())
         asm volatile(
@@ -1932,7 +1908,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
           uint32_t x[16];
           tmem_ld16(ta + 16 * cc, x);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) sum[16 * cc + i] = fmaf(__uint_as_float(x[i]), u, sum[16 * cc + i]);
+          for (int i = 0; i < 16; ++i)
+            sum[16 * cc + i] = fmaf(__uint_as_float(x[i]), u, sum[16 * cc + i]);
         }
         if (ch + 1 == nchunks) break;   // keep the last chunk's buffer
         fence_before();
@@ -1978,12 +1955,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         if (lane == 0) mbar_arrive_cluster(lead_tempty + 8 * ab);
       };
       rolled_tile_epilogue<CV, 8, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0,
-                                         itm.kblocks * BK, sg, om, scale_new, write, olds, epi_block(red), ts, release);
+                                         itm.kblocks * BK, sg, om, scale_new, write, olds,
+                                         epi_block(red), ts, release);
       if (++ab == 2) {
         ab = 0;
         abphase ^= 1;
       }
-      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, gi.partials + ((size_t)job * gi.ptiles + 2 * itm.t + rank) * kNQ);
+      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane,
+                    gi.partials + ((size_t)job * gi.ptiles + 2 * itm.t + rank) * kNQ);
     }
   }
 
@@ -2004,7 +1983,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 // The same pool of items, dynamic queue and per-item work as the 256 x 256
 // grouped kernel, with three changes that suit small instances:
 //  - N = 128: each CTA of a pair loads 64 B rows per stage (a 64-row tensor
-//    map), so a stage is 24 KB and the ring holds 8 of them;
+//    map), so a stage is 48 KB and the ring holds 4 of them (PairTile);
 //  - tensor memory holds four 128-column accumulators, so a tile epilogue,
 //    which keeps its tile's sums in the last chunk's accumulator while it
 //    stores, leaves the MMA issuer three accumulators to run ahead with;
@@ -2013,9 +1992,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 //    multiplies zeros (the tensor map fills rows past Np with zeros) and skips
 //    its epilogue.
 // Items run their K passes forwards (no K-snake): the queue keeps the items
-// in flight within a few instances, whose operand panels stay in L2.  The
-// tile order differs from the 256 x 256 kernels, so results agree with them
-// to rounding, not bit for bit.
+// in flight within a few instances, whose operand panels stay in L2.  An
+// instance whose 256 x 256 tiles take one round of the CTA pairs has no
+// backwards sweep in the other kernels either and gets the same bits from all
+// of them; larger ones agree to rounding.
 constexpr int G_BN = 128;                                   // tile columns
 using GT = PairTile<G_BN>;
 static_assert(GT::COLS == TMEM_COLS, "accumulators fill the allocation");
@@ -2143,7 +2123,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const int64_t items = first[count];
   const unsigned epoch = *(volatile unsigned*)&gq->epoch;   // fixed during the launch
 
-
   if (items == 0) {
     // every instance has ended
   } else if (warp == 0) {
@@ -2259,7 +2238,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
           uint32_t x[16];
           tmem_ld16(ta + 16 * cc, x);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) sum[16 * cc + i] = fmaf(__uint_as_float(x[i]), u, sum[16 * cc + i]);
+          for (int i = 0; i < 16; ++i)
+            sum[16 * cc + i] = fmaf(__uint_as_float(x[i]), u, sum[16 * cc + i]);
         }
         if (ch + 1 == nchunks) break;   // keep the last chunk's accumulator
         fence_before();
@@ -2306,11 +2286,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       // store; the products there are zeros
       if ((int64_t)row0 < Np)
         rolled_tile_epilogue<CV, 4, false>(ta_sum, Sold, Snew, hi_new, lo_new, lane, Np, r, c0,
-                                           itm.kblocks * BK, sg, om, scale_new, write, olds, epi_block(red), ts, release);
+                                           itm.kblocks * BK, sg, om, scale_new, write, olds,
+                                           epi_block(red), ts, release);
       else
         release();
       ab.next(GT::ACC);
-      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane, gi.partials + ((size_t)job * gi.ptiles + 2 * itm.t + rank) * kNQ);
+      tile_sums_out(ts, red, seq++, warp - EPI_WARP0, lane,
+                    gi.partials + ((size_t)job * gi.ptiles + 2 * itm.t + rank) * kNQ);
     }
   }
 
@@ -2324,7 +2306,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
                  "r"(TMEM_COLS));
   }
 }
-
 
 // ---------------------------------------------------------------------------
 // Host side
@@ -2438,14 +2419,12 @@ bool make_map(CUtensorMap* map, void* base, int64_t Np, int slices, int box_rows
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
                    3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   sk == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                   sk == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
 
 }  // namespace tc
-
-int tc_tile() { return tc::BN; }
 
 void pair_tile_info(const Layout& L, int64_t* entries, double* pass_flops, bool n128) {
   const int64_t tiles = n128 ? tc::num_tiles128(L.Np) : tc::num_pair_tiles(L.Np);
@@ -2455,7 +2434,8 @@ void pair_tile_info(const Layout& L, int64_t* entries, double* pass_flops, bool 
   const int cend = tc::k_blocks(L.n) * tc::BK;
   const double cols = nt - (double)edge / tiles * (L.Np - cend);
   if (entries) *entries = 2 * tiles;
-  if (pass_flops) *pass_flops = (double)tiles * 2 * tc::BM * cols * tc::k_blocks(L.n) * tc::BK * 2.0;
+  if (pass_flops)
+    *pass_flops = (double)tiles * 2 * tc::BM * cols * tc::k_blocks(L.n) * tc::BK * 2.0;
 }
 
 bool make_group_inst(const Layout& L, void* ws, int sm_count, GroupInst* gi, bool n128) {
@@ -2488,8 +2468,8 @@ cudaError_t launch_layer_tc_group(const GroupInst* inst, int count, bool bf16, i
   using namespace tc;
   if (count < 1 || count > kGroupMax || !queue || sm_count / 2 > kQueuePairs)
     return cudaErrorInvalidValue;
-  const int smem =
-      (n128 ? GT::SMEM : PairTile<BN>::SMEM) + (count + 1) * (int)sizeof(int64_t) + count * (int)sizeof(uint32_t);
+  const int smem = (n128 ? GT::SMEM : PairTile<BN>::SMEM) + (count + 1) * (int)sizeof(int64_t) +
+                   count * (int)sizeof(uint32_t);
   if (device_setup() == 0) return cudaErrorInvalidDevice;
   const uint64_t limit_ns = (uint64_t)(timeout_s * 1e9);
   const int ck = accum_chunk_k > 0 ? accum_chunk_k : DEFAULT_CHUNK_K;
